@@ -357,6 +357,113 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(GemmArgs<T> g) {
     }
 }
 
+// FP64 GEMM.  The SM's FP64 pipe (a few FMAs per clock) is the bound, not shared
+// memory or L2: even an 8 x 8 tile asks for some 10 bytes per clock and SM.
+// What costs time is an uneven spread over the SMs, so the tiles are small:
+// 8 x 8 outputs per CTA (one per thread and K group) until there are eight
+// 16 x 16 tiles per SM, from where the larger tile leaves less to fetch.  KG
+// groups of threads split each K chunk; their sums are joined in shared
+// memory in a fixed order.  288 x 48 x 288 (n, k of D = 3, chi = 32): 7.3 us, with
+// 16 x 128 tiles 57; 288^3: 18 us (2.7 TFLOP/s), with 64 x 64 tiles 79.
+template <int TB, int TT>
+__global__ void __launch_bounds__(128) gemm_f64_kernel(GemmArgs<double> g) {
+    constexpr int RX = TB / TT;                    // threads along N of one K group
+    constexpr int GT = RX * RX;                    // threads of one K group
+    constexpr int KG = 128 / GT;
+    constexpr int KC = 32;                         // K chunk staged at a time
+    static_assert(KC % KG == 0 && (TB * KC) % 128 == 0, "tile/thread mismatch");
+    constexpr int NL = TB * KC / 128;
+    __shared__ double As[KC][TB + 1], Bs[KC][TB + 1];
+    __shared__ double red[KG > 1 ? (KG - 1) * TB * TB : 1];
+    const int tid = threadIdx.x, kg = tid / GT, t = tid % GT, tx = t % RX, ty = t / RX;
+    const int m0 = blockIdx.y * TB, n0 = blockIdx.x * TB;
+    const double* A = g.A + (long long)blockIdx.z * g.sAb;
+    const double* B = g.B + (long long)blockIdx.z * g.sBb;
+    const bool a_kfast = g.sAk == 1, b_nfast = g.sBn == 1;
+    double acc[TT][TT], ra[NL], rb[NL];
+#pragma unroll
+    for (int i = 0; i < TT; ++i)
+#pragma unroll
+        for (int j = 0; j < TT; ++j) acc[i][j] = 0.0;
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int q = 0; q < NL; ++q) {
+            const int e = tid + 128 * q;
+            const int ma = a_kfast ? e / KC : e % TB, ka = a_kfast ? e % KC : e / TB;
+            const int nb = b_nfast ? e % TB : e / KC, kb = b_nfast ? e / TB : e % KC;
+            ra[q] = (m0 + ma < g.M && k0 + ka < g.K) ? A[(m0 + ma) * g.sAm + (k0 + ka) * g.sAk] : 0.0;
+            rb[q] = (n0 + nb < g.N && k0 + kb < g.K) ? B[(k0 + kb) * g.sBk + (n0 + nb) * g.sBn] : 0.0;
+        }
+    };
+    load(0);
+    for (int k0 = 0; k0 < g.K; k0 += KC) {
+#pragma unroll
+        for (int q = 0; q < NL; ++q) {
+            const int e = tid + 128 * q;
+            As[a_kfast ? e % KC : e / TB][a_kfast ? e / KC : e % TB] = ra[q];
+            Bs[b_nfast ? e / TB : e % KC][b_nfast ? e % TB : e / KC] = rb[q];
+        }
+        __syncthreads();
+        if (k0 + KC < g.K) load(k0 + KC);
+        const int kn = min(KC, g.K - k0);
+#pragma unroll 4
+        for (int kk = kg; kk < kn; kk += KG) {
+            double a[TT], b[TT];
+#pragma unroll
+            for (int i = 0; i < TT; ++i) a[i] = As[kk][ty + RX * i];
+#pragma unroll
+            for (int j = 0; j < TT; ++j) b[j] = Bs[kk][tx + RX * j];
+#pragma unroll
+            for (int i = 0; i < TT; ++i)
+#pragma unroll
+                for (int j = 0; j < TT; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+        }
+        __syncthreads();
+    }
+    if (KG > 1) {
+        if (kg > 0)
+#pragma unroll
+            for (int i = 0; i < TT; ++i)
+#pragma unroll
+                for (int j = 0; j < TT; ++j) red[(kg - 1) * TB * TB + (i * TT + j) * GT + t] = acc[i][j];
+        __syncthreads();
+        if (kg > 0) return;
+#pragma unroll
+        for (int q = 0; q < KG - 1; ++q)
+#pragma unroll
+            for (int i = 0; i < TT; ++i)
+#pragma unroll
+                for (int j = 0; j < TT; ++j) acc[i][j] += red[q * TB * TB + (i * TT + j) * GT + t];
+    }
+    double* C = g.C + (long long)blockIdx.z * g.sCb;
+#pragma unroll
+    for (int i = 0; i < TT; ++i) {
+        const int gm = m0 + ty + RX * i;
+        if (gm >= g.M) continue;
+#pragma unroll
+        for (int j = 0; j < TT; ++j) {
+            const int gn = n0 + tx + RX * j;
+            if (gn >= g.N) continue;
+            double v = g.alpha * acc[i][j];
+            if (g.colscale) v *= g.colscale[gn];
+            double* dst = C + gm * g.sCm + gn * g.sCn;
+            if (g.beta != 0.0) v += g.beta * (*dst);
+            *dst = v;
+        }
+    }
+}
+
+inline void gemm_f64(const GemmArgs<double>& g, cudaStream_t st) {
+    auto tiles = [&](int tb) { return (long long)((g.M + tb - 1) / tb) * ((g.N + tb - 1) / tb) * g.batch; };
+    const bool small = tiles(16) < 8LL * 152;
+    const int tb = small ? 8 : 16;
+    dim3 grid((g.N + tb - 1) / tb, (g.M + tb - 1) / tb, g.batch);
+    if (grid.y > 65535) fail(KH_EINVAL, "gemm M too large");
+    if (small) gemm_f64_kernel<8, 1><<<grid, 128, 0, st>>>(g);
+    else gemm_f64_kernel<16, 2><<<grid, 128, 0, st>>>(g);
+    KH_LAUNCHED();
+}
+
 template <typename T, int BM, int BN, int TM, int TN>
 inline void gemm_launch(const GemmArgs<T>& g, cudaStream_t st) {
     dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.batch);
@@ -397,6 +504,10 @@ template <typename T>
 inline void gemm(const GemmArgs<T>& g, cudaStream_t st) {
     if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return;
     if (g.batch > 65535) fail(KH_EINVAL, "gemm batch > 65535");
+    if constexpr (sizeof(T) == 8) {
+        gemm_f64(g, st);
+        return;
+    } else {
     // few output tiles and a long K: split K over CTAs into the scratch,
     // then reduce in a fixed order (deterministic)
     const long long tiles = (long long)((g.M + 63) / 64) * ((g.N + 63) / 64);
@@ -437,6 +548,7 @@ inline void gemm(const GemmArgs<T>& g, cudaStream_t st) {
         }
     }
     gemm_dispatch<T>(g, st);
+    }
 }
 
 // Plain row-major C(MxN) = A(MxK) B(KxN) [+beta C]; transposes by flags.

@@ -388,6 +388,14 @@ size_t kh_selftest_bytes(int M, int N, int K);
 kh_status kh_selftest_gemm(int prec, int M, int N, int K, const double* dev_A, const double* dev_B,
                            double* dev_C, void* dev_scratch, size_t scratch_bytes, void* stream);
 
+/* The FP32-accurate tensor-core product of the tensor-core precisions (operands
+ * split into TF32 parts, partial sums of at most 32 terms added in FP32): as
+ * kh_selftest_gemm with FP32 copies of the operands, A's copy laid out
+ * row-major (a_colmajor = 0, K a multiple of 4) or column-major (1, M a
+ * multiple of 4).  KH_EINVAL otherwise.  Synchronises stream. */
+kh_status kh_selftest_gemm3x(int a_colmajor, int M, int N, int K, const double* dev_A, const double* dev_B,
+                             double* dev_C, void* dev_scratch, size_t scratch_bytes, void* stream);
+
 /* Eigen-decomposition of a symmetric k x k FP64 matrix by the library's
  * Jacobi kernel in FP64 (prec = KH_FP64) or FP32 (otherwise): dev_evals
  * descending, column j of dev_W its eigenvector.  Scratch as above with

@@ -26,7 +26,7 @@ ABI_FUNCTIONS = [
     "kh_set_state", "kh_get_state", "ctm_set_tensor", "ctm_build_composite", "ctm_init",
     "ctm_copy_env", "ctm_sweep", "ctm_projectors", "ctm_get_env", "ctm_metric", "ctm_kappa",
     "ctm_expval", "ctm_correlation_length", "ctm_plaquette", "ctm_flux", "eefu_apply_gate", "eefu_cost_gradient", "observables", "kh_version", "kh_bond_hamiltonian", "kh_gate", "kh_flux_operators",
-    "eefu_trotter_step", "eefu_evolve", "eefu_evolve_flux", "eefu_evolve_batch", "kh_launch_count", "kh_profile", "kh_selftest_bytes", "kh_selftest_gemm",
+    "eefu_trotter_step", "eefu_evolve", "eefu_evolve_flux", "eefu_evolve_batch", "kh_launch_count", "kh_profile", "kh_selftest_bytes", "kh_selftest_gemm", "kh_selftest_gemm3x",
     "kh_selftest_symeig", "kh_selftest_svd", "kh_selftest_svd_refined", "kh_selftest_orth", "kh_selftest_fp64_newton",
     "kh_selftest_site_layered_bytes", "kh_selftest_site_layered", "kh_gemm_noalloc",
     "kh_gemm_noalloc_max_bytes", "kh_save", "kh_load_config", "kh_load",
@@ -93,6 +93,7 @@ def load_library(path=LIB_PATH):
         "kh_profile": (I, [P, I, dp]),
         "kh_selftest_bytes": (S, [I, I, I]),
         "kh_selftest_gemm": (I, [I, I, I, I, P, P, P, P, S, P]),
+        "kh_selftest_gemm3x": (I, [I, I, I, I, P, P, P, P, S, P]),
         "kh_selftest_symeig": (I, [I, I, P, P, P, P, S, P]),
         "kh_selftest_svd": (I, [I, I, P, P, P, P, P, S, P]),
         "kh_selftest_orth": (I, [I, I, I, D, P, P, P, S, P]),
@@ -136,6 +137,24 @@ def selftest_gemm(A, B, prec="fp64"):
                                 ctypes.c_void_p(base), nb, ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
     if st != KH_OK:
         raise KhError(st, "kh_selftest_gemm")
+    return C
+
+
+def selftest_gemm3x(A, B, a_colmajor=False):
+    """C = A @ B (FP64 CUDA tensors) through the FP32-accurate tensor-core
+    product, A's FP32 copy laid out row-major or column-major."""
+    import torch
+    M, K = A.shape
+    N = B.shape[1]
+    C = torch.empty((M, N), dtype=torch.float64, device=A.device)
+    nb = lib().kh_selftest_bytes(M, N, K)
+    scr = torch.empty(nb + 256, dtype=torch.uint8, device=A.device)
+    base = (scr.data_ptr() + 255) // 256 * 256
+    st = lib().kh_selftest_gemm3x(1 if a_colmajor else 0, M, N, K, _tptr(A.contiguous()), _tptr(B.contiguous()), _tptr(C),
+                                  ctypes.c_void_p(base), nb,
+                                  ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    if st != KH_OK:
+        raise KhError(st, "kh_selftest_gemm3x")
     return C
 
 

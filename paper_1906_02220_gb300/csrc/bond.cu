@@ -98,8 +98,8 @@ __device__ __forceinline__ int frame_offset(int f, int L, int U, int R, int Dd, 
 // GEMM's second operand: for kind 0 (corner, TL = [L,U][p][R,D]) and kind 1
 // (edge, TL = [L,D][p][U,R]) of frame f,
 //   Wt_f[(ok,ob)][(ib,ik)] = sum_p TL_f[ik][p][ok] TL_f[ib][p][ob]
-// summed in FP64.  With lo != null the value is stored as its TF32 head
-// (13 low mantissa bits cleared) in W and the FP32 remainder in lo.
+// summed in FP64.  With lo != null the value is stored rounded to nearest TF32
+// in W and the FP32 remainder in lo.
 template <typename T>
 __global__ void wt_kernel(const double* __restrict__ Tm, int p, int D, T* Wc, T* We, T* Wc_lo, T* We_lo) {
     const int d2 = D * D, d4 = d2 * d2;
@@ -127,7 +127,7 @@ __global__ void wt_kernel(const double* __restrict__ Tm, int p, int D, T* Wc, T*
         T* Wl = kind == 0 ? Wc_lo : We_lo;
         if (Wl) {
             float v = (float)sacc;
-            float h = __uint_as_float(__float_as_uint(v) & 0xFFFFE000u);
+            float h = __uint_as_float((__float_as_uint(v) + 0x1000u) & 0xFFFFE000u);   // a NaN stays in the remainder
             *W = (T)h;
             Wl[rem] = (T)(v - h);
         } else {

@@ -129,9 +129,9 @@ __global__ void permute32_kernel(const Ti* __restrict__ in, To* __restrict__ out
     }
 }
 
-// Permutation fused with the 3xTF32 operand split: hi = the value with its 13
-// low mantissa bits cleared (exactly TF32), lo = value - hi (32-bit path);
-// the permuted value itself also goes to out when out is not null.
+// Permutation fused with the 3xTF32 operand split: hi = the value rounded to
+// nearest TF32 (11 bits), lo = value - hi (32-bit path); the permuted value
+// itself also goes to out when out is not null.
 static __global__ void permute_split32_kernel(const float* __restrict__ in, float* __restrict__ hi,
                                               float* __restrict__ lo, float* __restrict__ out, PermArgs a) {
     const uint32_t total = (uint32_t)a.total;
@@ -147,7 +147,7 @@ static __global__ void permute_split32_kernel(const float* __restrict__ in, floa
             }
         }
         const float v = in[src];
-        const float h = __uint_as_float(__float_as_uint(v) & 0xFFFFE000u);
+        const float h = __uint_as_float((__float_as_uint(v) + 0x1000u) & 0xFFFFE000u);   // a NaN stays in lo
         hi[idx] = h;
         lo[idx] = v - h;
         if (out) out[idx] = v;

@@ -198,6 +198,11 @@ void Engine<T>::carve_lane(Carver& cv) {
     }
     sk_elems = 16LL * n * (kk > d.chi ? kk : d.chi);
     skbuf = cv.take<T>(sk_elems);
+    if (d.npass) {
+        const size_t bsz = (size_t)n * ((kk > d.chi ? kk : d.chi) + 4);
+        Bh = cv.take<T>(bsz);
+        Bl = cv.take<T>(bsz);
+    }
 }
 
 template <typename T>
@@ -583,25 +588,9 @@ void Engine<T>::refresh_operands(Slot<T>& sl) {
 //    bra layer batched over b (K = p D^2)                                  (4 nb p D^6 flops);
 //    with TLb given, the bra layer reads TLb instead of TL (an operator on
 //    the ket layer only).
-// The double-layer site contraction runs as a 3xTF32 tensor-core GEMM: its
-// Y operand is then written directly as the (hi, lo) pair into (mup, mdn).
-template <typename T>
-bool Engine<T>::site_presplit(const Slot<T>& sl) const {
-    return sl.dl && tc_npass == 3 && sizeof(T) == 4 && dm.D4 % 4 == 0;
-}
-
-// Y permuted into the site contraction's block layout: into Yp, or as the
-// split pair (mup, mdn) when site_presplit.
-template <typename T>
-void Engine<T>::site_operand(const Slot<T>& sl, const T* Y, T* Yp, const std::vector<long long>& shape,
-                             const std::vector<int>& order) {
-    if (site_presplit(sl)) permute_split((const float*)Y, (float*)mup, (float*)mdn, shape, order, st);
-    else permute<T, T>(Y, Yp, shape, order, st);
-}
-
 template <typename T>
 void Engine<T>::site_layer(const T* Ybuf, long long nb, const T* TL, const T* L1, const T* L2, int p, T* out,
-                           const T* Wt, const T* Wt_lo, bool presplit, const T* TLb) {
+                           const T* Wt, const T* Wt_lo, const T* TLb) {
     const int d2 = dm.d2, d4 = dm.D4;
     prof_begin(1);
     if (!Wt && L1) {                                   // layered, on the tensor cores
@@ -612,14 +601,13 @@ void Engine<T>::site_layer(const T* Ybuf, long long nb, const T* TL, const T* L1
     }
     if (Wt) {
         if (tc_npass && sizeof(T) == 4 && d4 % 4 == 0) {       // TMA rows must be 16-byte multiples
-            TcOperand a{(const float*)Ybuf, nullptr, d4}, b{(const float*)Wt, nullptr, d4};
             if (tc_npass == 3) {
-                float *yh = (float*)mup, *yl = (float*)mdn;     // nb D^4 = n^2 elements
-                if (!presplit) tc_split((const float*)Ybuf, yh, yl, nb * d4, st);
-                a = TcOperand{yh, yl, d4};
-                b = TcOperand{(const float*)Wt, (const float*)Wt_lo, d4};
+                gemm3x((const float*)Ybuf, d4, false, (const float*)Wt, (const float*)Wt_lo, d4, (float*)out, (int)nb, d4,
+                       d4, d4, 1.f, nullptr, nullptr, 0, tc_err, st);
+            } else {
+                TcOperand a{(const float*)Ybuf, d4}, b{(const float*)Wt, d4};
+                tc_gemm(a, b, (float*)out, (int)nb, d4, d4, d4, 1.f, 0.f, nullptr, tc_err, st);
             }
-            tc_gemm(a, b, (float*)out, (int)nb, d4, d4, d4, 1.f, 0.f, nullptr, tc_npass, tc_err, st);
         } else {
             gemm_rm<T>((int)nb, d4, d4, Ybuf, false, Wt, true, out, st);
         }
@@ -640,6 +628,25 @@ void Engine<T>::site_layer(const T* Ybuf, long long nb, const T* TL, const T* L1
     prof_end(1, 4.0 * (double)nb * p * d2 * (double)d2 * d2);
 }
 
+// The tensor-core FP32 products need 16-byte rows of A (n a multiple of 4 in
+// every use) and enough work.  At n = 1024, k = 80 (1.7e8 flops: split of B 5 us,
+// product 10, reduction 4) they equal the SIMT tiles with split K (12 + 4); at
+// 2500 x 128 x 2500 (1.6e9) they take 28 us against 120.  kMin3x lies between.
+constexpr double kMin3x = 3e8;
+template <typename T>
+bool Engine<T>::product3x(int ln, const T* A, long long lda, bool a_mmajor, const T* B, long long sn, long long sk,
+                          T* C, int M, int N, int K, long long ldc, const T* colscale) {
+    if constexpr (sizeof(T) == 4) {
+        if (!tc_npass || 2.0 * M * N * (double)K < kMin3x || !gemm3x_usable(A, lda)) return false;
+        const Lane<T>& L = lanes[ln];
+        const int ldb = (K + 3) / 4 * 4;
+        gemm3x_split_b(B, sn, sk, N, K, L.Bh, L.Bl, ldb, L.st);
+        gemm3x(A, lda, a_mmajor, L.Bh, L.Bl, ldb, C, M, N, K, ldc, 1.f, colscale, L.skbuf, sk_elems, tc_err, L.st);
+        return true;
+    }
+    return false;
+}
+
 template <typename T>
 void Engine<T>::corner(Slot<T>& sl, int f, int which) {
     const int chi = dm.chi, d2 = dm.d2, D = dm.D;
@@ -649,20 +656,27 @@ void Engine<T>::corner(Slot<T>& sl, int f, int which) {
     const T* E4 = Eop + ((f + 3) & 3) * E1;
     T* X = X1[which];
     gemm_rm<T>(chi, d2 * chi, chi, C1, false, E1p, false, X, st);            // [x4][(uk,ub,z)]
-    gemm_rm<T>(chi * d2, d2 * chi, chi, E4, false, X, false, Y1, st);        // [(w,lk,lb)][(uk,ub,z)]
-    site_operand(sl, Y1, Yp, {chi, D, D, D, D, chi}, {0, 5, 2, 4, 1, 3});     // [w][z][lb][ub][lk][uk]
+    // Y = E4 X as [(w,lk,lb)][(uk,ub,z)], or on the tensor cores its transpose
+    // (X^T E4^T: X's rows of n values suit the tensor maps at any chi); then
+    // [w][z][lb][ub][lk][uk]
+    const int n = dm.n;
+    if (product3x(lane_id(), X, n, true, E4, chi, 1, Y1, n, n, chi, n)) {
+        permute<T, T>(Y1, Yp, {D, D, chi, chi, D, D}, {3, 2, 5, 1, 4, 0}, st);
+    } else {
+        gemm_rm<T>(chi * d2, d2 * chi, chi, E4, false, X, false, Y1, st);
+        permute<T, T>(Y1, Yp, {chi, D, D, D, D, chi}, {0, 5, 2, 4, 1, 3}, st);
+    }
     const long long w4 = (long long)f * dm.D4 * dm.D4;
     site_layer(Yp, chi2, sl.Tcor + (long long)f * dm.pmax * dm.D4, lay_img(sl, 1, 0, f), lay_img(sl, 2, 0, f), sl.p,
                Qt, sl.dl ? sl.Wcor + w4 : nullptr,
-               sl.dl && sl.Wcor_lo ? sl.Wcor_lo + w4 : nullptr, site_presplit(sl));   // [w][z][rk][dk][rb][db]
+               sl.dl && sl.Wcor_lo ? sl.Wcor_lo + w4 : nullptr);   // [w][z][rk][dk][rb][db]
     // Q_0 stored transposed, [(z,rk,rb)][(w,dk,db)], as the K-major operand of
-    // Mt = Q_{s+3} Q_s on tensor cores; with 3xTF32 the (hi, lo) pairs of both
-    // operands are written by the same pass (Q_1: q1_hi, q1_lo; Q_0: mupp, mdnp)
+    // Mt = Q_{s+3} Q_s on tensor cores; with 3xTF32 its (hi, lo) pair is written
+    // by the same pass (mupp, mdnp)
     const std::vector<int> order = (which == 0 && tc_npass) ? std::vector<int>{1, 2, 4, 0, 3, 5}
                                                             : std::vector<int>{0, 3, 5, 1, 2, 4};
-    if (mt_presplit())
-        permute_split((const float*)Qt, (float*)(which == 1 ? q1_hi : mupp), (float*)(which == 1 ? q1_lo : mdnp),
-                      {chi, chi, D, D, D, D}, order, st, (float*)Q[which]);
+    if (which == 0 && mt_presplit())
+        permute_split((const float*)Qt, (float*)mupp, (float*)mdnp, {chi, chi, D, D, D, D}, order, st, (float*)Q[0]);
     else
         permute<T, T>(Qt, Q[which], {chi, chi, D, D, D, D}, order, st);
 }
@@ -720,16 +734,12 @@ bool Engine<T>::mt_presplit() const {
 template <typename T>
 void Engine<T>::half_system_product(int n) {
     prof_begin(0);
-    if (tc_npass && sizeof(T) == 4 && n % 4 == 0) {     // TMA rows must be 16-byte multiples
-        const float* Qb = (const float*)Q[1];
-        const float* QaT = (const float*)Q[0];
-        TcOperand a{Qb, nullptr, n}, b{QaT, nullptr, n};
-        if (tc_npass == 3) {       // operands split when Q_0, Q_1 were written (mt_presplit)
-            float *ah = (float*)q1_hi, *al = (float*)q1_lo, *bh = (float*)mupp, *bl = (float*)mdnp;
-            a = TcOperand{ah, al, n};
-            b = TcOperand{bh, bl, n};
-        }
-        tc_gemm(a, b, (float*)Mt, n, n, n, n, 1.f, 0.f, nullptr, tc_npass, tc_err, st);
+    if (mt_presplit()) {                                // Q_0 split when it was written
+        gemm3x((const float*)Q[1], n, false, (const float*)mupp, (const float*)mdnp, n, (float*)Mt, n, n, n, n, 1.f,
+               nullptr, nullptr, 0, tc_err, st);
+    } else if (tc_npass && sizeof(T) == 4 && n % 4 == 0) {     // TMA rows must be 16-byte multiples
+        TcOperand a{(const float*)Q[1], n}, b{(const float*)Q[0], n};
+        tc_gemm(a, b, (float*)Mt, n, n, n, n, 1.f, 0.f, nullptr, tc_err, st);
     } else {      // Q_0 is stored transposed whenever the tensor cores are enabled
         gemm_rm<T>(n, n, n, Q[1], false, Q[0], tc_npass != 0, Mt, st);
     }
@@ -844,6 +854,7 @@ void Engine<T>::projector(Slot<T>& sl, int dir, int slot_id) {
     const double jtol = sizeof(T) == 8 ? 1e-14 : 2e-6;
     const T* Qa = Q[0];
     const T* Qb = Q[1];
+    const int ln = lane_id();
     half_system_product(n);
     double* normM2 = dscr + DscrOff::kNormM2;
     KH_CUDA(cudaMemsetAsync(normM2, 0, sizeof(double), st));
@@ -898,11 +909,13 @@ void Engine<T>::projector(Slot<T>& sl, int dir, int slot_id) {
         }
         for (int it = 0; it < q; ++it) {
             prof_begin(9);
-            gemm_rm<T>(n, k, n, Mt, true, Vin, false, Z1, st, T(1), T(0), nullptr, skbuf, sk_elems);                 // Y = M V
+            if (!product3x(ln, Mt, n, true, Vin, 1, k, Z1, n, k, n, k))            // Y = M V
+                gemm_rm<T>(n, k, n, Mt, true, Vin, false, Z1, st, T(1), T(0), nullptr, skbuf, sk_elems);
             prof_end(9, 2.0 * n * (double)n * k);
             orth(Z1, n, k, U);                                                 // U = orth(Y)
             prof_begin(9);
-            gemm_rm<T>(n, k, n, Mt, false, U, false, Z2, st, T(1), T(0), nullptr, skbuf, sk_elems);                  // Z = M^T U
+            if (!product3x(ln, Mt, n, false, U, 1, k, Z2, n, k, n, k))             // Z = M^T U
+                gemm_rm<T>(n, k, n, Mt, false, U, false, Z2, st, T(1), T(0), nullptr, skbuf, sk_elems);
             prof_end(9, 2.0 * n * (double)n * k);
             orth(Z2, n, k, Vo);                                                // V' = orth(Z)
             Vin = Vo;
@@ -947,7 +960,8 @@ void Engine<T>::projector(Slot<T>& sl, int dir, int slot_id) {
     // P and P~^T are independent: P on the side lane (its own split-K scratch)
     const bool side = side_lane();
     if (side) fork_side();
-    {   // P = Qb^T V S^-1/2
+    // P = Qb^T V S^-1/2
+    if (!product3x(side ? 1 : ln, Qb, n, true, Z1, 1, k, P, n, nkeep, n, chi, isq)) {
         GemmArgs<T> g;
         g.M = n; g.N = nkeep; g.K = n; g.batch = 1;
         g.A = Qb; g.sAm = 1; g.sAk = n; g.sAb = 0;
@@ -957,7 +971,8 @@ void Engine<T>::projector(Slot<T>& sl, int dir, int slot_id) {
         g.sk = side ? lanes[1].skbuf : skbuf; g.sk_elems = sk_elems;
         gemm<T>(g, side ? lanes[1].st : st);
     }
-    {   // P~^T = Qa U S^-1/2  (Qa stored transposed when tensor cores are used)
+    // P~^T = Qa U S^-1/2  (Qa stored transposed when tensor cores are used)
+    if (!product3x(ln, Qa, n, tc_npass != 0, Uf, 1, k, PtT, n, nkeep, n, chi, isq)) {
         GemmArgs<T> g;
         g.M = n; g.N = nkeep; g.K = n; g.batch = 1;
         g.A = Qa; g.sAm = tc_npass ? 1 : n; g.sAk = tc_npass ? n : 1; g.sAb = 0;
@@ -1018,14 +1033,17 @@ void Engine<T>::absorb(Slot<T>& sl, int s) {
         KH_LAUNCHED();
     }
     const T* E4 = Eop + ((s + 3) & 3) * E1;
-    gemm_rm<T>(d2 * chi, d2 * chi, chi, E4, true, P, false, Y1, st);             // [(lk,lb,x4)][(dk,db,a)]
-    site_operand(sl, Y1, Yp, {D, D, chi, D, D, chi}, {2, 5, 1, 4, 0, 3});         // [x4][a][lb][db][lk][dk]
+    const int ln = lane_id();
+    if (!product3x(ln, E4, n, true, P, 1, n, Y1, n, n, chi, n))                   // [(lk,lb,x4)][(dk,db,a)]
+        gemm_rm<T>(d2 * chi, d2 * chi, chi, E4, true, P, false, Y1, st);
+    permute<T, T>(Y1, Yp, {D, D, chi, D, D, chi}, {2, 5, 1, 4, 0, 3}, st);         // [x4][a][lb][db][lk][dk]
     const long long w4 = (long long)s * dm.D4 * dm.D4;
     site_layer(Yp, chi2, sl.Tedg + (long long)s * dm.pmax * dm.D4, lay_img(sl, 1, 1, s), lay_img(sl, 2, 1, s), sl.p,
                Qt, sl.dl ? sl.Wedg + w4 : nullptr,
-               sl.dl && sl.Wedg_lo ? sl.Wedg_lo + w4 : nullptr, site_presplit(sl));   // [x4][a][uk][rk][ub][rb]
+               sl.dl && sl.Wedg_lo ? sl.Wedg_lo + w4 : nullptr);   // [x4][a][uk][rk][ub][rb]
     permute<T, T>(Qt, Y1, {chi, chi, D, D, D, D}, {1, 3, 5, 0, 2, 4}, st);       // [a][rk][rb][x4][uk][ub]
-    gemm_rm<T>(chi * d2, chi, n, Y1, false, PtT, false, E4n, st, T(1), T(0), nullptr, skbuf, sk_elems);   // [a][rk][rb][a_up]
+    if (!product3x(ln, Y1, n, false, PtT, 1, chi, E4n, n, chi, n, chi))           // [a][rk][rb][a_up]
+        gemm_rm<T>(chi * d2, chi, n, Y1, false, PtT, false, E4n, st, T(1), T(0), nullptr, skbuf, sk_elems);
     double* ns = dscr + DscrOff::kNorms;
     KH_CUDA(cudaMemsetAsync(ns + 2, 0, sizeof(double), st));
     sumsq_kernel<T><<<sumsq_grid(E1), 256, 0, st>>>(E4n, E1, ns + 2);
@@ -1057,8 +1075,8 @@ void Engine<T>::move(Slot<T>& sl, int s, int slot_id) {
     if (nlanes >= 2 && !in_lanes) {
         // The two enlarged corners are independent: corner s+3 runs on lane 1
         // (its own stream and scratch) reading lane 0's environment operands
-        // and writing Q_{s+3} (and its split, into lane 1's mupp/mdnp) where
-        // the half-system product reads them; lane 0 waits before the projector.
+        // and writing Q_{s+3} where the half-system product reads it; lane 0
+        // waits before the projector.
         KH_CUDA(cudaEventRecord(lane_ev[0], st));
         KH_CUDA(cudaStreamWaitEvent(lanes[1].st, lane_ev[0], 0));
         corner(sl, s, 0);
@@ -1071,15 +1089,11 @@ void Engine<T>::move(Slot<T>& sl, int s, int slot_id) {
         Eop = lanes[0].Eop;
         X1[1] = lanes[0].X1[1];
         Q[1] = lanes[0].Q[1];
-        q1_hi = lanes[1].mupp;
-        q1_lo = lanes[1].mdnp;
         corner(sl, (s + 3) & 3, 1);
         KH_CUDA(cudaEventRecord(lane_ev[1], st));
         bind(0);
         KH_CUDA(cudaStreamWaitEvent(st, lane_ev[1], 0));
     } else {
-        q1_hi = mup;
-        q1_lo = mdn;
         corner(sl, s, 0);
         corner(sl, (s + 3) & 3, 1);
     }

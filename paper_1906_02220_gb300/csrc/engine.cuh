@@ -133,7 +133,7 @@ struct EngineBase {
 // move is latency-bound and leaves most SMs idle).
 #define KH_LANE_PTRS(X) X(Cop) X(Eop) X(Y1) X(Yp) X(Zk) X(Qt) X(Mt) X(V0) X(Z1) X(U) X(Z2) X(Vo) X(Uf) \
     X(Xk) X(Hk) X(Lk) X(Qk) X(Sk) X(isq) X(P) X(PtT) X(C4E3) X(C1n) \
-    X(C4n) X(E4n) X(mt1) X(mt2) X(mup) X(mdn) X(mupp) X(mdnp) X(mN4) X(skbuf)
+    X(C4n) X(E4n) X(Bh) X(Bl) X(mt1) X(mt2) X(mup) X(mdn) X(mupp) X(mdnp) X(mN4) X(skbuf)
 // Fixed regions of the small FP64 scratch dscr that every lane owns (offsets
 // in doubles); the Gram matrix of the orthonormalisation (kk^2) comes last.
 struct DscrOff {
@@ -187,6 +187,7 @@ struct Engine : EngineBase {
     T *Xk = nullptr, *Hk = nullptr, *Lk = nullptr, *Qk = nullptr, *Sk = nullptr;
     T *isq = nullptr, *P = nullptr, *PtT = nullptr, *C4E3 = nullptr;
     T *C1n = nullptr, *C4n = nullptr, *E4n = nullptr;
+    T *Bh = nullptr, *Bl = nullptr;          // split B operand of the tensor-core FP32 products
     double* dscr = nullptr;    // small FP64 scratch (norms etc.), regions in DscrOff
     // metric / bond scratch (FP64 unless noted)
     T *mt1 = nullptr, *mt2 = nullptr, *mup = nullptr, *mdn = nullptr, *mupp = nullptr, *mdnp = nullptr, *mN4 = nullptr;
@@ -208,7 +209,6 @@ struct Engine : EngineBase {
     bool own_streams = false;
     cudaEvent_t lane_ev[3] = {nullptr, nullptr, nullptr};
     bool in_lanes = false;     // lanes 1, 2 busy with other slots (sweep_lanes)
-    T *q1_hi = nullptr, *q1_lo = nullptr;   // where the 3xTF32 split of Q_{s+3} was written
     // Side lane for independent pieces of a move (lane 1), when not busy:
     // fork makes lane 1 wait for lane 0's work so far, join the reverse.
     bool side_lane() const { return nlanes >= 2 && !in_lanes; }
@@ -227,6 +227,16 @@ struct Engine : EngineBase {
     ~Engine() override;
     void half_system_product(int n);
     bool mt_presplit() const;
+    // C (M x N, row stride ldc) = A B diag(colscale) on the tensor cores at FP32
+    // accuracy (gemm3x.cu) with lane ln's scratch and stream, or false where
+    // that path does not apply or does not pay
+    bool product3x(int ln, const T* A, long long lda, bool a_mmajor, const T* B, long long sn, long long sk, T* C,
+                   int M, int N, int K, long long ldc, const T* colscale = nullptr);
+    int lane_id() const {      // the lane whose scratch is bound
+        for (int i = 1; i < nlanes; ++i)
+            if (skbuf == lanes[i].skbuf) return i;
+        return 0;
+    }
 
     Engine() {}
     Engine(const kh_config& c, void* ws, size_t bytes, cudaStream_t s);
@@ -238,8 +248,7 @@ struct Engine : EngineBase {
     void corner(Slot<T>& sl, int frame, int which);
     void site_layer(const T* Ybuf, long long nb, const T* TL, const T* L1, const T* L2, int p, T* out,
                     const T* Wt, const T* Wt_lo,
-                    bool presplit = false, const T* TLb = nullptr);
-    bool site_presplit(const Slot<T>& sl) const;
+                    const T* TLb = nullptr);
     // operand image (1 = ket, 2 = bra) of the layered tensor-core contraction
     // for (kind: 0 corner, 1 edge; frame f), or null when the slot uses
     // another form
@@ -247,8 +256,6 @@ struct Engine : EngineBase {
         if (sl.dl || !sl.L1) return nullptr;
         return img == 1 ? sl.L1 + (kind * 4 + f) * dm.lay1 : sl.L2 + (kind * 4 + f) * dm.lay2;
     }
-    void site_operand(const Slot<T>& sl, const T* Y, T* Yp, const std::vector<long long>& shape,
-                      const std::vector<int>& order);
     void projector(Slot<T>& sl, int dir, int slot_id);
     void orth(const T* Y, int n, int k, T* Uo);
     void rr_svd(const T* X, int k, T* L, T* Qm, double jtol, int nrel, const double* Xd = nullptr);
@@ -301,17 +308,27 @@ struct Engine : EngineBase {
     void load_checkpoint(std::FILE* f) override;
 };
 
-// Tensor-core GEMM (tcgen05.cu): C = alpha colscale (A B^T) + beta C with A
-// (M x K) and B (N x K) row-major FP32 read as TF32; npass = 3 uses the
-// hi/lo split operands (lo may be null for npass = 1).
+// One-pass tensor-core GEMM (tcgen05.cu): C = alpha colscale (A B^T) + beta C
+// with A (M x K) and B (N x K) row-major FP32 read as TF32.
 struct TcOperand {
-    const float* hi;
-    const float* lo;
+    const float* p;
     long long ld;
 };
 void tc_gemm(const TcOperand& A, const TcOperand& B, float* C, int M, int N, int K, long long ldc, float alpha,
-             float beta, const float* colscale, int npass, int* err, cudaStream_t st);
-void tc_split(const float* x, float* hi, float* lo, long long n, cudaStream_t st);
+             float beta, const float* colscale, int* err, cudaStream_t st);
+
+int device_sms();      // SMs of the current device (layered.cu)
+
+// FP32-accurate tensor-core GEMM (gemm3x.cu): C = alpha colscale (A B), A raw
+// FP32, row-major ([m][k]) or column-major (a_mmajor: [k][m], row stride lda),
+// B (N x K) split by gemm3x_split_b from any strides into K-major hi and lo
+// parts of row stride ldb (>= K, a multiple of 4).  sk: scratch of the K split.
+bool gemm3x_usable(const float* A, long long lda);
+void gemm3x_split_b(const float* B, long long sn, long long sk, int N, int K, float* hi, float* lo, int ld,
+                    cudaStream_t st);
+void gemm3x(const float* A, long long lda, bool a_mmajor, const float* Bhi, const float* Blo, int ldb, float* C,
+            int M, int N, int K, long long ldc, float alpha, const float* colscale, float* sk, long long sk_elems,
+            int* err, cudaStream_t st);
 
 // Orthonormal basis of the columns of Y (n x k, k <= the Jacobi limit) by the
 // ordered CholQR2 (ctm.cu); see Engine::orth.

@@ -526,9 +526,7 @@ layered_kernel(const float* __restrict__ Y, long long nb, int nc, const uint8_t*
 
 // ------------------------------------------------------------------ host side
 
-namespace {
-
-int sm_count() {
+int device_sms() {
     static std::atomic<int> cache[kMaxDevices] = {};
     int dev = 0;
     KH_CUDA(cudaGetDevice(&dev));
@@ -540,6 +538,8 @@ int sm_count() {
     }
     return v;
 }
+
+namespace {
 
 int smem_optin_max() {
     static std::atomic<int> cache[kMaxDevices] = {};
@@ -589,7 +589,7 @@ void launch_layered(const float* Y, long long nb, int p, const float* img1, cons
     if (P.tmem > 256 && smem <= cap / 2) smem = cap / 2 + 1024;
     static std::atomic<size_t> granted[kMaxDevices] = {};
     smem_opt_in(lay::layered_kernel<D, NPASS, BF>, smem, granted);
-    const int grid = ntiles < sm_count() ? ntiles : sm_count();
+    const int grid = ntiles < device_sms() ? ntiles : device_sms();
     lay::layered_kernel<D, NPASS, BF><<<grid, lay::THREADS, smem, st>>>(
         Y, nb, nc, (const uint8_t*)img1, (const uint8_t*)img2, out, ntiles, nst1, nst2, err);
     KH_LAUNCHED();

@@ -21,34 +21,50 @@ void run_gemm(int M, int N, int K, const double* A, const double* B, double* C, 
     kh::cast<T, double>(c, C, (long long)M * N, st);
 }
 
-// tensor-core path: B^T made K-major by a permutation, optional hi/lo split
-void run_tc_gemm(int npass, int M, int N, int K, const double* A, const double* B, double* C, void* scratch,
-                 size_t bytes, cudaStream_t st) {
-    kh::Carver cv(scratch, bytes);
-    float* a = cv.take<float>((size_t)M * K);
-    float* bt = cv.take<float>((size_t)K * N);
-    float* c = cv.take<float>((size_t)M * N);
-    float* ah = cv.take<float>((size_t)M * K);
-    float* al = cv.take<float>((size_t)M * K);
-    float* bh = cv.take<float>((size_t)K * N);
-    float* bl = cv.take<float>((size_t)K * N);
-    int* err = cv.take<int>(64);
-    KH_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
-    kh::cast<double, float>(A, a, (long long)M * K, st);
-    kh::permute<double, float>(B, bt, {K, N}, {1, 0}, st);
-    kh::TcOperand oa{a, nullptr, K}, ob{bt, nullptr, K};
-    if (npass == 3) {
-        kh::tc_split(a, ah, al, (long long)M * K, st);
-        kh::tc_split(bt, bh, bl, (long long)K * N, st);
-        oa = kh::TcOperand{ah, al, K};
-        ob = kh::TcOperand{bh, bl, K};
-    }
-    kh::tc_gemm(oa, ob, c, M, N, K, N, 1.f, 0.f, nullptr, npass, err, st);
-    kh::cast<float, double>(c, C, (long long)M * N, st);
+void check_wait(const int* err, cudaStream_t st) {
     int h = 0;
     KH_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, st));
     KH_CUDA(cudaStreamSynchronize(st));
     if (h) kh::fail(KH_ETIMEOUT, "tensor-core GEMM wait timed out");
+}
+
+// tensor-core path, one TF32 pass: B^T made K-major by a permutation
+void run_tc_gemm(int M, int N, int K, const double* A, const double* B, double* C, void* scratch, size_t bytes,
+                 cudaStream_t st) {
+    kh::Carver cv(scratch, bytes);
+    float* a = cv.take<float>((size_t)M * K);
+    float* bt = cv.take<float>((size_t)K * N);
+    float* c = cv.take<float>((size_t)M * N);
+    int* err = cv.take<int>(64);
+    KH_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
+    kh::cast<double, float>(A, a, (long long)M * K, st);
+    kh::permute<double, float>(B, bt, {K, N}, {1, 0}, st);
+    kh::tc_gemm(kh::TcOperand{a, K}, kh::TcOperand{bt, K}, c, M, N, K, N, 1.f, 0.f, nullptr, err, st);
+    kh::cast<float, double>(c, C, (long long)M * N, st);
+    check_wait(err, st);
+}
+
+// tensor-core path at FP32 accuracy, A row-major or (a_mmajor) stored [K][M]
+void run_gemm3x(bool a_mmajor, int M, int N, int K, const double* A, const double* B, double* C, void* scratch,
+                size_t bytes, cudaStream_t st) {
+    kh::Carver cv(scratch, bytes);
+    const int ldb = (K + 3) / 4 * 4;
+    float* a = cv.take<float>((size_t)M * K);
+    float* b = cv.take<float>((size_t)K * N);
+    float* c = cv.take<float>((size_t)M * N);
+    float* bh = cv.take<float>((size_t)N * ldb);
+    float* bl = cv.take<float>((size_t)N * ldb);
+    int* err = cv.take<int>(64);
+    const long long skn = 8LL * M * ((N + 3) / 4 * 4);
+    float* sk = (cv.off + skn * sizeof(float) + 256 <= bytes) ? cv.take<float>((size_t)skn) : nullptr;
+    KH_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
+    if (a_mmajor) kh::permute<double, float>(A, a, {M, K}, {1, 0}, st);
+    else kh::cast<double, float>(A, a, (long long)M * K, st);
+    kh::cast<double, float>(B, b, (long long)K * N, st);
+    kh::gemm3x_split_b(b, 1, N, N, K, bh, bl, ldb, st);
+    kh::gemm3x(a, a_mmajor ? M : K, a_mmajor, bh, bl, ldb, c, M, N, K, N, 1.f, nullptr, sk, sk ? skn : 0, err, st);
+    kh::cast<float, double>(c, C, (long long)M * N, st);
+    check_wait(err, st);
 }
 
 template <typename T>
@@ -180,8 +196,8 @@ kh_status selftest_gemm_on(int prec, int M, int N, int K, const double* A, const
     return run([&] {
         if (prec == KH_FP64) run_gemm<double>(M, N, K, A, B, C, scratch, bytes, st);
         else if (prec == KH_FP32) run_gemm<float>(M, N, K, A, B, C, scratch, bytes, st);
-        else if (prec == KH_TF32) run_tc_gemm(1, M, N, K, A, B, C, scratch, bytes, st);
-        else if (prec == KH_TF32X3) run_tc_gemm(3, M, N, K, A, B, C, scratch, bytes, st);
+        else if (prec == KH_TF32) run_tc_gemm(M, N, K, A, B, C, scratch, bytes, st);
+        else if (prec == KH_TF32X3) run_gemm3x(false, M, N, K, A, B, C, scratch, bytes, st);
         else kh::fail(KH_EINVAL, "precision not built");
         KH_CUDA(cudaStreamSynchronize(st));
     });
@@ -202,11 +218,19 @@ kh_status kh_selftest_gemm(int prec, int M, int N, int K, const double* A, const
     return run([&] {
         if (prec == KH_FP64) run_gemm<double>(M, N, K, A, B, C, scratch, bytes, st);
         else if (prec == KH_FP32) run_gemm<float>(M, N, K, A, B, C, scratch, bytes, st);
-        else if (prec == KH_TF32) run_tc_gemm(1, M, N, K, A, B, C, scratch, bytes, st);
-        else if (prec == KH_TF32X3) run_tc_gemm(3, M, N, K, A, B, C, scratch, bytes, st);
+        else if (prec == KH_TF32) run_tc_gemm(M, N, K, A, B, C, scratch, bytes, st);
+        else if (prec == KH_TF32X3) run_gemm3x(false, M, N, K, A, B, C, scratch, bytes, st);
         else kh::fail(KH_EINVAL, "precision not built");
         KH_CUDA(cudaStreamSynchronize(st));
     });
+}
+
+kh_status kh_selftest_gemm3x(int a_colmajor, int M, int N, int K, const double* A, const double* B, double* C,
+                             void* scratch, size_t bytes, void* stream) {
+    if (M < 1 || N < 1 || K < 1 || !A || !B || !C || !scratch) return KH_EINVAL;
+    if (bytes < kh_selftest_bytes(M, N, K)) return KH_ENOMEM;
+    cudaStream_t st = (cudaStream_t)stream;
+    return run([&] { run_gemm3x(a_colmajor != 0, M, N, K, A, B, C, scratch, bytes, st); });
 }
 
 kh_status kh_selftest_symeig(int prec, int k, const double* G, double* W, double* E, void* scratch, size_t bytes,

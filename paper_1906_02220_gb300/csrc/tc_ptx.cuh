@@ -69,6 +69,37 @@ __device__ __forceinline__ void umma_tf32(uint32_t tmem_d, uint64_t da, uint64_t
         : "memory");
 }
 
+// One lane of a converged warp (the same one each time), as a 0/1 value for
+// the *_by forms below.  With the whole warp in the issuing loop and only the
+// instruction predicated, descriptors and addresses stay in uniform registers;
+// inside an `if (lane == 0)` every operand of every MMA is moved there first,
+// which takes longer (~45 ns an MMA) than a narrow MMA itself.
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(e));
+    return e;
+}
+
+// MMA with A from tensor memory, and commit, issued by the lane whose `by` is 1
+__device__ __forceinline__ void umma_tf32_tmem_a_by(uint32_t by, uint32_t tmem_d, uint32_t tmem_a, uint64_t db,
+                                                    uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}\n"
+        ::"r"(tmem_d), "r"(tmem_a), "l"(db), "r"(idesc), "r"(acc), "r"(by)
+        : "memory");
+}
+
+__device__ __forceinline__ void umma_commit_by(uint32_t by, uint64_t* bar) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n"
+        ::"r"(smem_u32(bar)), "r"(by)
+        : "memory");
+}
+
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                  : "memory");

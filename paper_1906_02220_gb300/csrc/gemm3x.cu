@@ -225,21 +225,21 @@ gemm3x_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CU
                 if (K - kb * BK >= BK) {
 #pragma unroll
                     for (int ks = 0; ks < 4; ++ks)
-                        umma_tf32_tmem_a_by(by, d, al + ks * 8, bh + ks * 2, idesc, ks > 0 ? 1u : 0u);
+                        umma_tf32_tmem_a(by, d, al + ks * 8, bh + ks * 2, idesc, ks > 0 ? 1u : 0u);
 #pragma unroll
-                    for (int ks = 0; ks < 4; ++ks) umma_tf32_tmem_a_by(by, d, ah + ks * 8, bl + ks * 2, idesc, 1u);
+                    for (int ks = 0; ks < 4; ++ks) umma_tf32_tmem_a(by, d, ah + ks * 8, bl + ks * 2, idesc, 1u);
 #pragma unroll
-                    for (int ks = 0; ks < 4; ++ks) umma_tf32_tmem_a_by(by, d, ah + ks * 8, bh + ks * 2, idesc, 1u);
+                    for (int ks = 0; ks < 4; ++ks) umma_tf32_tmem_a(by, d, ah + ks * 8, bh + ks * 2, idesc, 1u);
                 } else {
                     const int steps = (K - kb * BK + 7) / 8;
                     for (int ks = 0; ks < steps; ++ks)
-                        umma_tf32_tmem_a_by(by, d, al + ks * 8, bh + ks * 2, idesc, ks > 0 ? 1u : 0u);
-                    for (int ks = 0; ks < steps; ++ks) umma_tf32_tmem_a_by(by, d, ah + ks * 8, bl + ks * 2, idesc, 1u);
-                    for (int ks = 0; ks < steps; ++ks) umma_tf32_tmem_a_by(by, d, ah + ks * 8, bh + ks * 2, idesc, 1u);
+                        umma_tf32_tmem_a(by, d, al + ks * 8, bh + ks * 2, idesc, ks > 0 ? 1u : 0u);
+                    for (int ks = 0; ks < steps; ++ks) umma_tf32_tmem_a(by, d, ah + ks * 8, bl + ks * 2, idesc, 1u);
+                    for (int ks = 0; ks < steps; ++ks) umma_tf32_tmem_a(by, d, ah + ks * 8, bh + ks * 2, idesc, 1u);
                 }
-                umma_commit_by(by, &bars.a_empty[a]);
-                umma_commit_by(by, &bars.b_empty[s]);
-                umma_commit_by(by, &bars.acc_full[c]);
+                umma_commit(by, &bars.a_empty[a]);
+                umma_commit(by, &bars.b_empty[s]);
+                umma_commit(by, &bars.acc_full[c]);
                 if (++s == BSTAGES) {
                     s = 0;
                     ++su;
@@ -251,7 +251,7 @@ gemm3x_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CU
             }
         }
         // every MMA issued completes before tensor memory is freed
-        umma_commit_by(by, &bars.drain);
+        umma_commit(by, &bars.drain);
         for (uint32_t i = 0; !mbar_try_wait(&bars.drain, 0); ++i)
             if (i >= (1u << 22)) {
                 if (lane == 0) atomicOr(err, 128);

@@ -194,106 +194,102 @@ layered_kernel(const float* __restrict__ Y, long long nb, int nc, const uint8_t*
         }
     } else if (warp < WORKER0) {
         // ---------------------------------------------------------- MMA issuers
-        // NI1 threads (warps 1 ..) issue the ket GEMMs, NI2 threads (the next
-        // warps) the bra GEMMs, one thread per warp: these narrow MMAs are
-        // bounded by their issue, not by the tensor pipe, so several issuers
-        // keep more of them in flight.  Issuer q of a GEMM issues the MMAs of
-        // the accumulators a with a % NI == q.
-        if (lane == 0) {
-            bool ok = true;
-            long long g0 = 0;
-            int it = 0;
-            const bool ket = warp <= NI1;
-            const int qi = ket ? warp - 1 : warp - 1 - NI1;   // issuer index within its GEMM
-            if (ket) {
-                for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++it, g0 += nc) {
-                    if (!mbar_wait(&bars.a1_full, it & 1, abort_flag)) { ok = false; break; }
+        // NI1 warps (1 ..) issue the ket GEMMs, NI2 (the next ones) the bra GEMMs.
+        // A warp walks its loop whole and one lane issues: in a one-lane branch
+        // every MMA's operands are moved to uniform registers first, ~50 ns an
+        // MMA, which is longer than these narrow MMAs take.  Issuer q of a GEMM
+        // issues the MMAs of the accumulators a with a % NI == q.
+        bool ok = true;
+        long long g0 = 0;
+        int it = 0;
+        const uint32_t by = elect_one();
+        const bool ket = warp <= NI1;
+        const int qi = ket ? warp - 1 : warp - 1 - NI1;   // issuer index within its GEMM
+        if (ket) {
+            for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++it, g0 += nc) {
+                if (!wait_warp(&bars.a1_full, it & 1, abort_flag)) { ok = false; break; }
+                fence_after();
+                for (int c = 0; c < nc; ++c) {                      // ket layer of chunk c
+                    const long long g = g0 + c;
+                    const int s1 = res1 ? c : (int)(g % nst1);
+                    const uint32_t ph1 = res1 ? 0u : (uint32_t)((g / nst1) & 1);
+                    const int j = (int)(g & 1);
+                    if (!wait_warp(&bars.b1_full[s1], ph1, abort_flag) ||
+                        !wait_warp(&bars.acc1_empty[j], (uint32_t)((g >> 1) & 1) ^ 1, abort_flag)) {
+                        ok = false;
+                        break;
+                    }
                     fence_after();
-                    for (int c = 0; c < nc; ++c) {                      // ket layer of chunk c
-                        const long long g = g0 + c;
-                        const int s1 = res1 ? c : (int)(g % nst1);
-                        const uint32_t ph1 = res1 ? 0u : (uint32_t)((g / nst1) & 1);
-                        const int j = (int)(g & 1);
-                        if (!mbar_wait(&bars.b1_full[s1], ph1, abort_flag) ||
-                            !mbar_wait(&bars.acc1_empty[j], (uint32_t)((g >> 1) & 1) ^ 1, abort_flag)) {
-                            ok = false;
-                            break;
-                        }
-                        fence_after();
-                        // MMAs round-robin over the buffer's nacc1 accumulators
-                        const uint32_t d0 = tmem + P.c_acc1 + j * P.nacc1 * P.acc1_cols;
-                        const uint32_t a0 = smem_u32(sA1), b0 = smem_u32(sB1 + (size_t)s1 * B1_SZ);
+                    // MMAs round-robin over the buffer's nacc1 accumulators
+                    const uint32_t d0 = tmem + P.c_acc1 + j * P.nacc1 * P.acc1_cols;
+                    const uint64_t da0 = smem_desc(smem_u32(sA1));
+                    const uint64_t db0 = smem_desc(smem_u32(sB1 + (size_t)s1 * B1_SZ));
 #pragma unroll
-                        for (int pass = 0; pass < NPASS; ++pass) {
-                            const uint32_t ab = a0 + (pass == 2 ? P.a1_bytes : 0);
-                            const uint32_t bb = b0 + (pass == 1 ? P.b1_bytes : 0);
+                    for (int pass = 0; pass < NPASS; ++pass) {
 #pragma unroll
-                            for (int ks = 0; ks < P.k1p / KS; ++ks) {
-                                const int i = pass * (P.k1p / KS) + ks;
-                                if ((i % P.nacc1) % NI1 != qi) continue;
-                                // 32 bytes of K per MMA, four per 128-byte block
-                                const uint64_t da = smem_desc(ab + (ks >> 2) * (128 * 128) + (ks & 3) * 32);
-                                const uint64_t db = smem_desc(bb + (ks >> 2) * (P.n1p * 128) + (ks & 3) * 32);
-                                const uint32_t dd = d0 + (i % P.nacc1) * P.acc1_cols;
-                                if constexpr (BF) umma_f16(dd, da, db, ID1, i >= P.nacc1 ? 1u : 0u);
-                                else umma_tf32(dd, da, db, ID1, i >= P.nacc1 ? 1u : 0u);
-                            }
+                        for (int ks = 0; ks < P.k1p / KS; ++ks) {
+                            const int i = pass * (P.k1p / KS) + ks;
+                            if ((i % P.nacc1) % NI1 != qi) continue;
+                            // 32 bytes of K per MMA, four per 128-byte block (16-byte descriptor units)
+                            const uint64_t da = da0 + ((pass == 2 ? P.a1_bytes : 0) + (ks >> 2) * (128 * 128) + (ks & 3) * 32) / 16;
+                            const uint64_t db = db0 + ((pass == 1 ? P.b1_bytes : 0) + (ks >> 2) * (P.n1p * 128) + (ks & 3) * 32) / 16;
+                            const uint32_t dd = d0 + (i % P.nacc1) * P.acc1_cols;
+                            if constexpr (BF) umma_f16(by, dd, da, db, ID1, i >= P.nacc1 ? 1u : 0u);
+                            else umma_tf32(by, dd, da, db, ID1, i >= P.nacc1 ? 1u : 0u);
                         }
-                        umma_commit(&bars.acc1_full[j]);
-                        if (!res1) umma_commit(&bars.b1_empty[s1]);
-                        if (c == nc - 1) umma_commit(&bars.a1_empty);
                     }
-                }
-            } else {
-                for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++it, g0 += nc) {
-                    for (int cc = 0; cc < nc; ++cc) {                   // bra layer of chunk cc
-                        const long long g = g0 + cc;
-                        const int s2 = res2 ? cc : (int)(g % nst2);
-                        const uint32_t ph2 = res2 ? 0u : (uint32_t)((g / nst2) & 1);
-                        const int ja = (int)(g % P.na2);
-                        const uint32_t pa = (uint32_t)((g / P.na2) & 1);
-                        if (!mbar_wait(&bars.b2_full[s2], ph2, abort_flag) ||
-                            !mbar_wait(&bars.a2_full[ja], pa, abort_flag) ||
-                            (cc == 0 && !mbar_wait(&bars.out_empty, (uint32_t)(it & 1) ^ 1, abort_flag))) {
-                            ok = false;
-                            break;
-                        }
-                        fence_after();
-                        // MMAs round-robin over the nacc2 output accumulators
-                        const uint32_t d0 = tmem + P.c_out;
-                        const uint32_t a2 = tmem + P.c_a2 + ja * NPL * P.a2_cols;
-                        const uint32_t b0 = smem_u32(sB2 + (size_t)s2 * B2_SZ);
-#pragma unroll
-                        for (int pass = 0; pass < NPASS; ++pass) {
-                            const uint32_t aa = a2 + (pass == 2 ? P.a2_cols : 0);
-                            const uint32_t bb = b0 + (pass == 1 ? P.b2_bytes : 0);
-#pragma unroll
-                            for (int ks = 0; ks < P.k2p / KS; ++ks) {
-                                const int i = pass * (P.k2p / KS) + ks;
-                                if ((i % P.nacc2) % NI2 != qi) continue;
-                                const uint64_t db = smem_desc(bb + (ks >> 2) * (P.n2p * 128) + (ks & 3) * 32);
-                                const uint32_t dd = d0 + (i % P.nacc2) * P.out_cols;
-                                const uint32_t acc = (cc > 0 || i >= P.nacc2) ? 1u : 0u;
-                                // 8 tensor-memory columns of Z per MMA (8 TF32 or 16 BF16 values)
-                                if constexpr (BF) umma_f16_tmem_a(dd, aa + ks * 8, db, ID2, acc);
-                                else umma_tf32_tmem_a(dd, aa + ks * 8, db, ID2, acc);
-                            }
-                        }
-                        umma_commit(&bars.a2_empty[ja]);
-                        if (!res2) umma_commit(&bars.b2_empty[s2]);
-                        if (cc == nc - 1) umma_commit(&bars.out_full);
-                    }
+                    umma_commit(by, &bars.acc1_full[j]);
+                    if (!res1) umma_commit(by, &bars.b1_empty[s1]);
+                    if (c == nc - 1) umma_commit(by, &bars.a1_empty);
                 }
             }
-            if (!ok) {
-                s_abort = 1;
-                atomicOr(err, 16);
+        } else {
+            for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++it, g0 += nc) {
+                for (int cc = 0; cc < nc; ++cc) {                   // bra layer of chunk cc
+                    const long long g = g0 + cc;
+                    const int s2 = res2 ? cc : (int)(g % nst2);
+                    const uint32_t ph2 = res2 ? 0u : (uint32_t)((g / nst2) & 1);
+                    const int ja = (int)(g % P.na2);
+                    const uint32_t pa = (uint32_t)((g / P.na2) & 1);
+                    if (!wait_warp(&bars.b2_full[s2], ph2, abort_flag) || !wait_warp(&bars.a2_full[ja], pa, abort_flag) ||
+                        (cc == 0 && !wait_warp(&bars.out_empty, (uint32_t)(it & 1) ^ 1, abort_flag))) {
+                        ok = false;
+                        break;
+                    }
+                    fence_after();
+                    // MMAs round-robin over the nacc2 output accumulators
+                    const uint32_t d0 = tmem + P.c_out;
+                    const uint32_t a2 = tmem + P.c_a2 + ja * NPL * P.a2_cols;
+                    const uint64_t db0 = smem_desc(smem_u32(sB2 + (size_t)s2 * B2_SZ));
+#pragma unroll
+                    for (int pass = 0; pass < NPASS; ++pass) {
+                        const uint32_t aa = a2 + (pass == 2 ? P.a2_cols : 0);
+#pragma unroll
+                        for (int ks = 0; ks < P.k2p / KS; ++ks) {
+                            const int i = pass * (P.k2p / KS) + ks;
+                            if ((i % P.nacc2) % NI2 != qi) continue;
+                            const uint64_t db = db0 + ((pass == 1 ? P.b2_bytes : 0) + (ks >> 2) * (P.n2p * 128) + (ks & 3) * 32) / 16;
+                            const uint32_t dd = d0 + (i % P.nacc2) * P.out_cols;
+                            const uint32_t acc = (cc > 0 || i >= P.nacc2) ? 1u : 0u;
+                            // 8 tensor-memory columns of Z per MMA (8 TF32 or 16 BF16 values)
+                            if constexpr (BF) umma_f16_tmem_a(by, dd, aa + ks * 8, db, ID2, acc);
+                            else umma_tf32_tmem_a(by, dd, aa + ks * 8, db, ID2, acc);
+                        }
+                    }
+                    umma_commit(by, &bars.a2_empty[ja]);
+                    if (!res2) umma_commit(by, &bars.b2_empty[s2]);
+                    if (cc == nc - 1) umma_commit(by, &bars.out_full);
+                }
             }
-            // every MMA this thread issued completes before tensor memory is freed
-            uint64_t* dr = &bars.drain[warp - 1];
-            umma_commit(dr);
-            if (!wait_drain(dr, 0)) atomicOr(err, 16);
         }
+        if (!ok) {
+            s_abort = 1;
+            if (lane == 0) atomicOr(err, 16);
+        }
+        // every MMA this warp issued completes before tensor memory is freed
+        uint64_t* dr = &bars.drain[warp - 1];
+        umma_commit(by, dr);
+        if (!wait_drain(dr, 0) && lane == 0) atomicOr(err, 16);
     } else {
         // ---------------------------------------------------------- workers
         const int wt = threadIdx.x - 32 * WORKER0;       // 0 .. 128 NSET - 1

@@ -60,17 +60,8 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
     return d;
 }
 
-__device__ __forceinline__ void umma_tf32(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n"
-        ::"r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(acc)
-        : "memory");
-}
-
 // One lane of a converged warp (the same one each time), as a 0/1 value for
-// the *_by forms below.  With the whole warp in the issuing loop and only the
+// the forms below.  With the whole warp in the issuing loop and only the
 // instruction predicated, descriptors and addresses stay in uniform registers;
 // inside an `if (lane == 0)` every operand of every MMA is moved there first,
 // which takes longer (~45 ns an MMA) than a narrow MMA itself.
@@ -80,9 +71,23 @@ __device__ __forceinline__ uint32_t elect_one() {
     return e;
 }
 
-// MMA with A from tensor memory, and commit, issued by the lane whose `by` is 1
-__device__ __forceinline__ void umma_tf32_tmem_a_by(uint32_t by, uint32_t tmem_d, uint32_t tmem_a, uint64_t db,
-                                                    uint32_t idesc, uint32_t acc) {
+// D (+)= A B, issued by the lane whose `by` is 1; acc = 0 overwrites D.  kind::tf32
+// has K = 8 per instruction, kind::f16 (BF16 or FP16 operands, by the
+// instruction descriptor's formats) K = 16.  A comes from shared memory, or in
+// the tmem_a forms from tensor memory: lanes = rows, one TF32 element per column
+// or two 16-bit values, the lower K index in the low half.
+__device__ __forceinline__ void umma_tf32(uint32_t by, uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc,
+                                            uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n"
+        ::"r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(acc), "r"(by)
+        : "memory");
+}
+__device__ __forceinline__ void umma_tf32_tmem_a(uint32_t by, uint32_t tmem_d, uint32_t tmem_a, uint64_t db, uint32_t idesc,
+                                            uint32_t acc) {
     asm volatile(
         "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
@@ -91,18 +96,33 @@ __device__ __forceinline__ void umma_tf32_tmem_a_by(uint32_t by, uint32_t tmem_d
         ::"r"(tmem_d), "r"(tmem_a), "l"(db), "r"(idesc), "r"(acc), "r"(by)
         : "memory");
 }
+__device__ __forceinline__ void umma_f16(uint32_t by, uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc,
+                                            uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
+        ::"r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(acc), "r"(by)
+        : "memory");
+}
+__device__ __forceinline__ void umma_f16_tmem_a(uint32_t by, uint32_t tmem_d, uint32_t tmem_a, uint64_t db, uint32_t idesc,
+                                            uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n"
+        ::"r"(tmem_d), "r"(tmem_a), "l"(db), "r"(idesc), "r"(acc), "r"(by)
+        : "memory");
+}
 
-__device__ __forceinline__ void umma_commit_by(uint32_t by, uint64_t* bar) {
+__device__ __forceinline__ void umma_commit(uint32_t by, uint64_t* bar) {
     asm volatile(
         "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
         "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n"
         ::"r"(smem_u32(bar)), "r"(by)
         : "memory");
-}
-
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
 }
 
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -119,41 +139,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
-}
-
-// D += A B with A (M x K) read from tensor memory at tmem_a (lanes = rows,
-// one TF32 element per column) and B from a shared-memory descriptor.
-__device__ __forceinline__ void umma_tf32_tmem_a(uint32_t tmem_d, uint32_t tmem_a, uint64_t db, uint32_t idesc,
-                                                 uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}\n"
-        ::"r"(tmem_d), "r"(tmem_a), "l"(db), "r"(idesc), "r"(acc)
-        : "memory");
-}
-
-// kind::f16 (BF16 or FP16 operands, K = 16 per instruction, FP32 accumulate
-// with the instruction descriptor's formats): A, B from shared memory, and A
-// from tensor memory (two 16-bit values per column, the lower K index in the
-// low half).
-__device__ __forceinline__ void umma_f16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
-        ::"r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(acc)
-        : "memory");
-}
-
-__device__ __forceinline__ void umma_f16_tmem_a(uint32_t tmem_d, uint32_t tmem_a, uint64_t db, uint32_t idesc,
-                                                uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n"
-        ::"r"(tmem_d), "r"(tmem_a), "l"(db), "r"(idesc), "r"(acc)
-        : "memory");
 }
 
 // Stores 16 consecutive 32-bit columns of this warp's 32 tensor-memory lanes

@@ -6,7 +6,7 @@
 // One 128 x BN output tile per CTA, 6 warps:
 //   warp 0     TMA producer: 128B-swizzled K-major tiles into a STAGES-deep
 //              ring of shared-memory buffers (mbarrier full/empty pairs);
-//   warp 1     allocates the TMEM accumulator; one elected lane issues
+//   warp 1     allocates the TMEM accumulator and issues (one elected lane)
 //              tcgen05.mma (M=128, N=BN, K=8 per instruction) and commits
 //              to the empty barriers;
 //   warps 2-5  epilogue: tcgen05.ld of their TMEM lane quadrant, scaling,
@@ -93,29 +93,29 @@ gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUte
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            bool ok = true;
-            for (int kt = 0; kt < KT; ++kt) {
-                const int s = kt % G::STAGES;
-                const uint32_t ph = (kt / G::STAGES) & 1;
-                if (!mbar_wait(&full_bar[s], ph, abort_flag)) { s_abort = 1; atomicOr(err, 2); ok = false; break; }
-                fence_after();
-                const uint32_t a0 = smem_u32(base + s * G::STAGE_BYTES);
-                const uint32_t b0 = a0 + G::A_BYTES;
-#pragma unroll
-                for (int kk = 0; kk < BK / 8; ++kk) {
-                    const uint32_t off = kk * 32;               // 8 TF32 = 32 bytes along K
-                    const uint64_t da = smem_desc(a0 + off), db = smem_desc(b0 + off);
-                    // accumulator of this k-step; its first use (first k-steps of the tile) overwrites
-                    const int i = kt * (BK / 8) + kk;
-                    const uint32_t d = tmem + (uint32_t)((i % G::NACC) * G::ACC_COLS);
-                    umma_tf32(d, da, db, G::IDESC, i >= G::NACC ? 1u : 0u);
-                }
-                umma_commit(&empty_bar[s]);
+        const uint32_t by = elect_one();       // the whole warp walks the loop, one lane issues
+        for (int kt = 0; kt < KT; ++kt) {
+            const int s = kt % G::STAGES;
+            const uint32_t ph = (kt / G::STAGES) & 1;
+            if (!__all_sync(0xffffffffu, mbar_wait(&full_bar[s], ph, abort_flag))) {
+                s_abort = 1;
+                if (lane == 0) atomicOr(err, 2);
+                break;
             }
-            (void)ok;
-            umma_commit(&acc_bar);   // also after an abort: lets the epilogue wait for MMAs in flight
+            fence_after();
+            const uint64_t da = smem_desc(smem_u32(base + s * G::STAGE_BYTES));
+            const uint64_t db = smem_desc(smem_u32(base + s * G::STAGE_BYTES + G::A_BYTES));
+#pragma unroll
+            for (int kk = 0; kk < BK / 8; ++kk) {
+                // 8 TF32 = 32 bytes along K = 2 descriptor units; accumulator of this
+                // k-step; its first use (first k-steps of the tile) overwrites
+                const int i = kt * (BK / 8) + kk;
+                const uint32_t d = tmem + (uint32_t)((kk % G::NACC) * G::ACC_COLS);
+                umma_tf32(by, d, da + kk * 2, db + kk * 2, G::IDESC, i >= G::NACC ? 1u : 0u);
+            }
+            umma_commit(by, &empty_bar[s]);
         }
+        umma_commit(by, &acc_bar);   // also after an abort: lets the epilogue wait for MMAs in flight
     } else {
         // epilogue: warp w reads TMEM lanes [32 (w % 4), +32)
         const int q = warp & 3;

@@ -143,7 +143,7 @@ __global__ void wt_kernel(const double* __restrict__ Tm, int p, int D, T* Wc, T*
 // and the bra image
 //   B2_c[ob][(ib, pl)] = TL_f[ib][c pc + pl][ob],
 // each stored byte for byte as its 128-byte-swizzled K-major shared-memory
-// tile (the TF32 head, then the FP32 remainder, with 3 passes), zero outside
+// tile (rounded to nearest TF32, then the FP32 remainder, with 3 passes), zero outside
 // the operand.  Layout [kind][frame][chunk][hi, lo], per1 / per2 floats per
 // (kind, frame).
 __global__ void layered_img_kernel(const double* __restrict__ Tm, const double* __restrict__ Tb, int p, int D,
@@ -188,7 +188,7 @@ __global__ void layered_img_kernel(const double* __restrict__ Tm, const double* 
         } else {
             float x = (float)v;
             if (npass == 3) {
-                const float h = __uint_as_float(__float_as_uint(x) & 0xFFFFE000u);
+                const float h = __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);   // nearest TF32
                 x = hl == 0 ? h : x - h;
             }
             (ket ? img1 : img2)[e] = x;

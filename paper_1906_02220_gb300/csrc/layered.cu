@@ -8,28 +8,34 @@
 //   warp 0 (lanes 0, 1)  bulk-copies the chunk's ket (B1) and bra (B2) operand
 //                        images into shared-memory rings (or once, when all
 //                        chunks fit: resident images);
-//   warp 1               allocates tensor memory; one lane issues the ket GEMMs
-//                          acc1[c % 2]  = Y_tile * B1_c    (A, B in shared memory)
-//   warps 2, 3           one lane each issues half of the bra GEMMs' MMAs
-//                          out         += Z_c   * B2_c    (A = Z in tensor memory)
-//                        (each group committed to an mbarrier);
-//   warps 4-7 (workers)  load the Y tile (hi/lo split, or BF16) into shared
-//                        memory (the next tile's values fetched into registers
-//                        while this tile's chunks run), read acc1 row (b, ib)
-//                        per thread, scatter it into a shared-memory buffer in
-//                        (b, ok) row order, read back row (b, ok), split it into
-//                        TF32 hi/lo (or round it to BF16 pairs) and store it to
-//                        tensor memory as the bra GEMM's A operand; at the end
-//                        of a tile they read the output accumulators and store
-//                        out rows (b, ok).
-// With 3 passes every product is A_hi B_hi + A_hi B_lo + A_lo B_hi (FP32-level
-// accuracy from TF32 inputs); BF16 runs one kind::f16 pass (K = 16 per MMA).
-// The MMAs of each GEMM are spread round-robin over independent accumulators
-// (summed when read) and, for the bra GEMM, over two issuing threads: these
-// narrow MMAs are bound by their issue, not by the tensor pipe.  Every wait is bounded: on time-out the kernel
-// raises a flag, the roles drain, tensor memory is freed and the kernel
+//   warp 1               tensor memory; issues the ket GEMMs
+//                          acc1[c % nb1] = Y_tile * B1_c
+//   warp 2               issues the bra GEMMs
+//                          out         += Z_c   * B2_c
+//                        (both with A in tensor memory, one elected lane issuing,
+//                        each group committed to an mbarrier);
+//   warps 4-7, 8-11      two worker sets, taking chunks in turn: read acc1 row
+//                        (b, ib) per thread, scatter it into a shared-memory
+//                        buffer in (b, ok) row order, read back row (b, ok), split
+//                        it into TF32 hi/lo (or round it to BF16 pairs) and store it
+//                        to tensor memory as the bra GEMM's A operand.  The first
+//                        set also loads the next Y tile into tensor memory (one row
+//                        per thread) and stores the output rows.
+// With 3 passes every product is A_hi B_hi + A_hi B_lo + A_lo B_hi from operands
+// rounded to nearest TF32; the ket accumulator takes the two small ones first, the
+// bra GEMM has an accumulator for them (the tensor core truncates the accumulator
+// at every instruction).  BF16 runs one kind::f16 pass (K = 16 per MMA).
+// What bounds it: the tensor pipe's narrow MMAs at D >= 6 (73 % of the TF32 rate
+// over the padded shapes at D = 8), the chunk's chain of hand-offs below.  Time of a
+// launch, 3xTF32, p = 16: (4, 64) 20 us, (5, 100) 140, (6, 144) 454 (137 TFLOP/s),
+// (8, 144) 1494 (233); with Y as a shared-memory operand, one worker set and MMAs
+// issued from a one-lane branch: 25.5, 167, 722, 2113.  Y in tensor memory frees
+// 64 KB for two stages of both image rings, whose reload was on the chain.
+// Every wait is bounded: on time-out the kernel raises a flag, the roles drain,
+// tensor memory is freed and the kernel
 // returns with bits set in *err (8 producer, 16 MMA issuer, 32 workers).
 #include <atomic>
+#include <type_traits>
 
 #include <cuda_bf16.h>
 
@@ -43,17 +49,15 @@ namespace lay {
 
 using namespace tc;
 
-constexpr int NSET = 1;                        // worker sets (4 warps each), chunks split by index mod NSET
-// issuing threads (one per warp) of the ket and the bra GEMMs; the bra GEMM
-// has four times the MMAs of the ket GEMM at D = 4.  Eight warps in all keep
-// the per-thread register limit at 255 (a ninth warp on one SM sub-partition
-// would cut it to 168 and spill the workers).
-constexpr int NI1 = 1, NI2 = 2;
-constexpr int WORKER0 = 1 + NI1 + NI2;          // first worker warp
-constexpr int THREADS = 32 * WORKER0 + 128 * NSET;   // producer, issuers, workers
+constexpr int NSET = 2;                         // worker sets (4 warps each)
+constexpr int WORKER0 = 4;                      // first worker warp (its tensor-memory quadrant is its number mod 4)
+constexpr int THREADS = 32 * WORKER0 + 128 * NSET;
 constexpr int MAXST = 16;
 
-__device__ __forceinline__ float tf32_hi(float v) { return __uint_as_float(__float_as_uint(v) & 0xFFFFE000u); }
+// nearest TF32 (a NaN may come out as zero, but stays in the remainder v - hi)
+__device__ __forceinline__ float tf32_hi(float v) {
+    return __uint_as_float((__float_as_uint(v) + 0x1000u) & 0xFFFFE000u);
+}
 
 // instruction descriptor: FP32 accumulator, A and B TF32 (kind::tf32) or BF16
 // (kind::f16), K-major, N and M = 128
@@ -73,7 +77,7 @@ struct Bars {
     uint64_t b1_full[MAXST], b1_empty[MAXST], b2_full[MAXST], b2_empty[MAXST];
     uint64_t acc1_full[2], acc1_empty[2], a2_full[2], a2_empty[2];
     uint64_t zs_w[NSET], zs_r[NSET];
-    uint64_t a1_full, a1_empty, out_full, out_empty, drain[NI1 + NI2];
+    uint64_t y_full, y_empty, out_full, out_empty, drain[2];
 };
 
 // Bounded wait made uniform over the warp: false on time-out or abort.
@@ -100,7 +104,7 @@ layered_kernel(const float* __restrict__ Y, long long nb, int nc, const uint8_t*
     constexpr int NPL = NPASS == 3 ? 2 : 1;
     constexpr int KS = P.kstep;
     constexpr uint32_t ID1 = idesc(P.n1p, BF), ID2 = idesc(P.n2p, BF);
-    constexpr int A1_SZ = NPL * P.a1_bytes, B1_SZ = NPL * P.b1_bytes, B2_SZ = NPL * P.b2_bytes;
+    constexpr int B1_SZ = NPL * P.b1_bytes, B2_SZ = NPL * P.b2_bytes;
 
     extern __shared__ uint8_t smem_raw[];
     __shared__ Bars bars;
@@ -109,33 +113,32 @@ layered_kernel(const float* __restrict__ Y, long long nb, int nc, const uint8_t*
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool res1 = nst1 == nc, res2 = nst2 == nc;      // images loaded once
     uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t* sA1 = base;
-    uint8_t* sB1 = sA1 + A1_SZ;
+    uint8_t* sB1 = base;
     uint8_t* sB2 = sB1 + (size_t)nst1 * B1_SZ;
     float* sZ = (float*)(sB2 + (size_t)nst2 * B2_SZ);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < MAXST; ++s) {
             mbar_init(&bars.b1_full[s], 1);
-            mbar_init(&bars.b1_empty[s], NI1);
+            mbar_init(&bars.b1_empty[s], 1);
             mbar_init(&bars.b2_full[s], 1);
-            mbar_init(&bars.b2_empty[s], NI2);
+            mbar_init(&bars.b2_empty[s], 1);
         }
         for (int j = 0; j < 2; ++j) {
-            mbar_init(&bars.acc1_full[j], NI1);
+            mbar_init(&bars.acc1_full[j], 1);
             mbar_init(&bars.acc1_empty[j], 128);
             mbar_init(&bars.a2_full[j], 128);
-            mbar_init(&bars.a2_empty[j], NI2);
+            mbar_init(&bars.a2_empty[j], 1);
         }
-        mbar_init(&bars.a1_full, 128 * NSET);
-        mbar_init(&bars.a1_empty, NI1);
-        mbar_init(&bars.out_full, NI2);
+        mbar_init(&bars.y_full, 128);
+        mbar_init(&bars.y_empty, 1);
+        mbar_init(&bars.out_full, 1);
         mbar_init(&bars.out_empty, 128);
         for (int s = 0; s < NSET; ++s) {
             mbar_init(&bars.zs_w[s], 128);
             mbar_init(&bars.zs_r[s], 128);
         }
-        for (int q = 0; q < NI1 + NI2; ++q) mbar_init(&bars.drain[q], 1);
+        for (int q = 0; q < 2; ++q) mbar_init(&bars.drain[q], 1);
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -192,55 +195,50 @@ layered_kernel(const float* __restrict__ Y, long long nb, int nc, const uint8_t*
             for (int s = 0; s < MAXST; ++s)
                 if (armed[s] && !wait_drain(&full[s], (uint32_t)(armed[s] - 1) & 1)) atomicOr(err, 8);
         }
-    } else if (warp < WORKER0) {
+    } else if (warp <= 2) {
         // ---------------------------------------------------------- MMA issuers
-        // NI1 warps (1 ..) issue the ket GEMMs, NI2 (the next ones) the bra GEMMs.
         // A warp walks its loop whole and one lane issues: in a one-lane branch
         // every MMA's operands are moved to uniform registers first, ~50 ns an
-        // MMA, which is longer than these narrow MMAs take.  Issuer q of a GEMM
-        // issues the MMAs of the accumulators a with a % NI == q.
+        // MMA, which is longer than these narrow MMAs take.
         bool ok = true;
         long long g0 = 0;
         int it = 0;
         const uint32_t by = elect_one();
-        const bool ket = warp <= NI1;
-        const int qi = ket ? warp - 1 : warp - 1 - NI1;   // issuer index within its GEMM
-        if (ket) {
+        constexpr int S1 = P.k1p / KS, S2 = P.k2p / KS;       // K steps of the two GEMMs
+        if (warp == 1) {
             for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++it, g0 += nc) {
-                if (!wait_warp(&bars.a1_full, it & 1, abort_flag)) { ok = false; break; }
+                if (!wait_warp(&bars.y_full, it & 1, abort_flag)) { ok = false; break; }
                 fence_after();
                 for (int c = 0; c < nc; ++c) {                      // ket layer of chunk c
                     const long long g = g0 + c;
                     const int s1 = res1 ? c : (int)(g % nst1);
                     const uint32_t ph1 = res1 ? 0u : (uint32_t)((g / nst1) & 1);
-                    const int j = (int)(g & 1);
+                    const int j = (int)(g % P.nb1);
+                    const long long h = g - P.nb1;              // the chunk that had this accumulator
                     if (!wait_warp(&bars.b1_full[s1], ph1, abort_flag) ||
-                        !wait_warp(&bars.acc1_empty[j], (uint32_t)((g >> 1) & 1) ^ 1, abort_flag)) {
+                        (h >= 0 && !wait_warp(&bars.acc1_empty[h & 1], (uint32_t)((h >> 1) & 1), abort_flag))) {
                         ok = false;
                         break;
                     }
                     fence_after();
-                    // MMAs round-robin over the buffer's nacc1 accumulators
-                    const uint32_t d0 = tmem + P.c_acc1 + j * P.nacc1 * P.acc1_cols;
-                    const uint64_t da0 = smem_desc(smem_u32(sA1));
+                    const uint32_t d = tmem + P.c_acc1 + j * P.acc1_cols, y = tmem + P.c_y;
                     const uint64_t db0 = smem_desc(smem_u32(sB1 + (size_t)s1 * B1_SZ));
+                    // lo B_hi, hi B_lo, hi B_hi with 3 passes, hi B_hi alone with one
 #pragma unroll
-                    for (int pass = 0; pass < NPASS; ++pass) {
+                    for (int pass = 3 - NPASS; pass < 3; ++pass) {
 #pragma unroll
-                        for (int ks = 0; ks < P.k1p / KS; ++ks) {
-                            const int i = pass * (P.k1p / KS) + ks;
-                            if ((i % P.nacc1) % NI1 != qi) continue;
+                        for (int ks = 0; ks < S1; ++ks) {
                             // 32 bytes of K per MMA, four per 128-byte block (16-byte descriptor units)
-                            const uint64_t da = da0 + ((pass == 2 ? P.a1_bytes : 0) + (ks >> 2) * (128 * 128) + (ks & 3) * 32) / 16;
                             const uint64_t db = db0 + ((pass == 1 ? P.b1_bytes : 0) + (ks >> 2) * (P.n1p * 128) + (ks & 3) * 32) / 16;
-                            const uint32_t dd = d0 + (i % P.nacc1) * P.acc1_cols;
-                            if constexpr (BF) umma_f16(by, dd, da, db, ID1, i >= P.nacc1 ? 1u : 0u);
-                            else umma_tf32(by, dd, da, db, ID1, i >= P.nacc1 ? 1u : 0u);
+                            const uint32_t a = y + (NPASS == 3 && pass == 0 ? P.y_cols : 0) + ks * 8;
+                            const uint32_t acc = (pass > 3 - NPASS || ks > 0) ? 1u : 0u;
+                            if constexpr (BF) umma_f16_tmem_a(by, d, a, db, ID1, acc);
+                            else umma_tf32_tmem_a(by, d, a, db, ID1, acc);
                         }
                     }
-                    umma_commit(by, &bars.acc1_full[j]);
+                    umma_commit(by, &bars.acc1_full[g & 1]);
                     if (!res1) umma_commit(by, &bars.b1_empty[s1]);
-                    if (c == nc - 1) umma_commit(by, &bars.a1_empty);
+                    if (c == nc - 1) umma_commit(by, &bars.y_empty);
                 }
             }
         } else {
@@ -257,26 +255,25 @@ layered_kernel(const float* __restrict__ Y, long long nb, int nc, const uint8_t*
                         break;
                     }
                     fence_after();
-                    // MMAs round-robin over the nacc2 output accumulators
                     const uint32_t d0 = tmem + P.c_out;
                     const uint32_t a2 = tmem + P.c_a2 + ja * NPL * P.a2_cols;
                     const uint64_t db0 = smem_desc(smem_u32(sB2 + (size_t)s2 * B2_SZ));
 #pragma unroll
-                    for (int pass = 0; pass < NPASS; ++pass) {
-                        const uint32_t aa = a2 + (pass == 2 ? P.a2_cols : 0);
+                    for (int pass = 3 - NPASS; pass < 3; ++pass) {
 #pragma unroll
-                        for (int ks = 0; ks < P.k2p / KS; ++ks) {
-                            const int i = pass * (P.k2p / KS) + ks;
-                            if ((i % P.nacc2) % NI2 != qi) continue;
+                        for (int ks = 0; ks < S2; ++ks) {
                             const uint64_t db = db0 + ((pass == 1 ? P.b2_bytes : 0) + (ks >> 2) * (P.n2p * 128) + (ks & 3) * 32) / 16;
-                            const uint32_t dd = d0 + (i % P.nacc2) * P.out_cols;
-                            const uint32_t acc = (cc > 0 || i >= P.nacc2) ? 1u : 0u;
                             // 8 tensor-memory columns of Z per MMA (8 TF32 or 16 BF16 values)
-                            if constexpr (BF) umma_f16_tmem_a(by, dd, aa + ks * 8, db, ID2, acc);
-                            else umma_tf32_tmem_a(by, dd, aa + ks * 8, db, ID2, acc);
+                            const uint32_t a = a2 + (NPASS == 3 && pass == 0 ? P.a2_cols : 0) + ks * 8;
+                            const bool main = pass == 2;            // leading products: accumulators 0 .. nm - 1
+                            const uint32_t dd = d0 + (main ? ks % P.nm : P.nm) * P.out_cols;
+                            const bool first = main ? ks < P.nm : (pass == 0 && ks == 0);
+                            const uint32_t acc = (cc > 0 || !first) ? 1u : 0u;
+                            if constexpr (BF) umma_f16_tmem_a(by, dd, a, db, ID2, acc);
+                            else umma_tf32_tmem_a(by, dd, a, db, ID2, acc);
                         }
                     }
-                    umma_commit(by, &bars.a2_empty[ja]);
+                    umma_commit(by, &bars.a2_empty[g & 1]);
                     if (!res2) umma_commit(by, &bars.b2_empty[s2]);
                     if (cc == nc - 1) umma_commit(by, &bars.out_full);
                 }
@@ -290,10 +287,9 @@ layered_kernel(const float* __restrict__ Y, long long nb, int nc, const uint8_t*
         uint64_t* dr = &bars.drain[warp - 1];
         umma_commit(by, dr);
         if (!wait_drain(dr, 0) && lane == 0) atomicOr(err, 16);
-    } else {
+    } else if (warp >= WORKER0) {
         // ---------------------------------------------------------- workers
-        const int wt = threadIdx.x - 32 * WORKER0;       // 0 .. 128 NSET - 1
-        const int set = wt >> 7;                         // chunks g with g % NSET == set
+        const int set = (warp - WORKER0) >> 2;           // chunks g with g % NSET == set
         const int q = warp & 3;                          // tensor-memory lane quadrant
         const int t = 32 * q + lane;                     // tile row of this thread
         const uint32_t lane_base = (uint32_t)(32 * q) << 16;
@@ -301,193 +297,194 @@ layered_kernel(const float* __restrict__ Y, long long nb, int nc, const uint8_t*
         float* zbuf = sZ + set * 128 * P.zs;
         bool ok = true;
 
-        // zero the Y tile images once: padding rows and columns stay zero
-        for (int i = wt; i < A1_SZ / 16; i += 128 * NSET) ((float4*)sA1)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        asm volatile("bar.sync 1, %0;" ::"r"(128 * NSET) : "memory");   // zeros land before the first tile's values
-
-        // the tile's R D^2 values of Y (contiguous), all loads in flight at once:
-        // fetched into registers, then written (hi/lo split) into the tile image
-        constexpr int YPER = (P.rows * D2 + 128 * NSET - 1) / (128 * NSET);
-        auto fetch_y = [&](int tile, float (&yv)[YPER]) {
-            const long long e0 = (long long)tile * P.rows * D2, etot = total_rows * D2;
+        // n values v(i) as A operand columns: TF32 hi columns at `dst`, lo columns
+        // npad columns on with 3 passes; or BF16 pairs, the lower index in the low half
+        auto store_a = [&](uint32_t dst, auto npad_c, int lo_off, const float* v) {
+            constexpr int NP = decltype(npad_c)::value;   // columns (a multiple of 8)
+            auto col = [&](int c, bool lo) {
+                if constexpr (BF) return __uint_as_float(pack_bf16x2(v[2 * c], v[2 * c + 1]));
+                const float x = v[c];
+                if (NPASS != 3) return x;
+                const float h = tf32_hi(x);
+                return lo ? x - h : h;
+            };
 #pragma unroll
-            for (int j = 0; j < YPER; ++j) {
-                const int i = wt + 128 * NSET * j;
-                const long long e = e0 + i;
-                yv[j] = (i < P.rows * D2 && e < etot) ? __ldg(Y + e) : 0.f;
-            }
-        };
-        auto store_y = [&](const float (&yv)[YPER]) {
+            for (int l = 0; l < NPL; ++l) {
 #pragma unroll
-            for (int j = 0; j < YPER; ++j) {
-                const int i = wt + 128 * NSET * j;
-                if (i < P.rows * D2) {
-                    const int o = swz_offset(i / D2, i % D2, 128, P.esz);
-                    if constexpr (BF) {
-                        *(__nv_bfloat16*)(sA1 + o) = __float2bfloat16_rn(yv[j]);
-                    } else if (NPASS == 3) {
-                        const float h = tf32_hi(yv[j]);
-                        *(float*)(sA1 + o) = h;
-                        *(float*)(sA1 + P.a1_bytes + o) = yv[j] - h;
-                    } else {
-                        *(float*)(sA1 + o) = yv[j];
-                    }
+                for (int c0 = 0; c0 + 16 <= NP; c0 += 16) {
+                    float w[16];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) w[i] = col(c0 + i, l == 1);
+                    tmem_st16(dst + l * lo_off + c0, w);
+                }
+                if constexpr (NP % 16 != 0) {
+                    float w[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) w[i] = col(NP - 8 + i, l == 1);
+                    tmem_st8(dst + l * lo_off + NP - 8, w);
                 }
             }
-            fence_proxy_async();
-            mbar_arrive(&bars.a1_full);
         };
+        // one row of the tile's Y into tensor memory (zero past the rows)
         auto load_y = [&](int tile) {
-            float yv[YPER];
-            fetch_y(tile, yv);
-            store_y(yv);
+            constexpr int NV = P.k1p;
+            float y[NV];
+#pragma unroll
+            for (int i = 0; i < NV; ++i) y[i] = 0.f;
+            const long long row = (long long)tile * P.rows + t;
+            if (t < P.rows && row < total_rows) {
+                const float* src = Y + row * D2;
+                if constexpr (D2 % 4 == 0) {
+#pragma unroll
+                    for (int i = 0; i < D2; i += 4) {
+                        const float4 w = __ldg((const float4*)(src + i));
+                        y[i] = w.x;
+                        y[i + 1] = w.y;
+                        y[i + 2] = w.z;
+                        y[i + 3] = w.w;
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < D2; ++i) y[i] = __ldg(src + i);
+                }
+            }
+            store_a(tmem + lane_base + P.c_y, std::integral_constant<int, P.y_cols>{}, P.y_cols, y);
+            tmem_st_wait();
+            fence_before();
+            mbar_arrive(&bars.y_full);
         };
-        // the next tile's values are fetched while this tile's chunks run (where
-        // the registers allow it), so their latency leaves the critical path
-        constexpr bool kPrefetch = YPER <= 32;
-        float ynext[kPrefetch ? YPER : 1];
 
-        if ((int)blockIdx.x < ntiles) load_y(blockIdx.x);
+        if (set == 0 && (int)blockIdx.x < ntiles) load_y(blockIdx.x);
         long long g0 = 0;
         int it = 0;
         uint32_t zcount = 0;                             // chunks this set has transposed
         for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++it, g0 += nc) {
+            const int next = tile + gridDim.x;
+            // set 0 loads the next tile's Y (asked into L2 now) and stores this
+            // tile's output.  One set does it for every tile: it then waits for
+            // every phase of y_empty and out_full, while a wait by parity that
+            // skips a phase could return on the one before.
+            if (set == 0 && next < ntiles) {
+                const long long row = (long long)next * P.rows + t;
+                if (t < P.rows && row < total_rows) {
+                    const float* src = Y + row * D2;
+#pragma unroll
+                    for (int i = 0; i < D2; i += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(src + i));
+                }
+            }
             for (int c = 0; c < nc && ok; ++c) {
                 const long long g = g0 + c;
                 if ((int)(g % NSET) != set) continue;
-                const int j = (int)(g & 1);
                 // ---- ket accumulator row (b, ib) -> transpose buffer rows (b, ok)
-                if (!wait_warp(&bars.acc1_full[j], (uint32_t)((g >> 1) & 1), abort_flag)) { ok = false; break; }
+                // (chunks signal two barriers in turn, one for each set, whatever the
+                // number of buffers: a set then waits for every phase of its own)
+                const int j = (int)(g % P.nb1);
+                if (!wait_warp(&bars.acc1_full[g & 1], (uint32_t)((g >> 1) & 1), abort_flag)) { ok = false; break; }
                 fence_after();
-                // the buffer's nacc1 accumulators, summed
-                uint32_t vr[P.nacc1][P.n1p / 16][16];
+                uint32_t vr[P.n1p / 16][16];
 #pragma unroll
-                for (int a = 0; a < P.nacc1; ++a)
-#pragma unroll
-                    for (int c0 = 0; c0 < P.n1p; c0 += 16)
-                        tmem_ld16_async(tmem + lane_base +
-                                            (uint32_t)(P.c_acc1 + (j * P.nacc1 + a) * P.acc1_cols + c0),
-                                        vr[a][c0 / 16]);
+                for (int c0 = 0; c0 < P.n1p; c0 += 16)
+                    tmem_ld16_async(tmem + lane_base + (uint32_t)(P.c_acc1 + j * P.acc1_cols + c0), vr[c0 / 16]);
                 tmem_ld_wait();
 #pragma unroll
-                for (int a = 0; a < P.nacc1; ++a)
-#pragma unroll
-                    for (int c0 = 0; c0 < P.n1p; c0 += 16) tmem_regs_ready(vr[a][c0 / 16]);
-                auto v = [&](int n) {
-                    float x = __uint_as_float(vr[0][n >> 4][n & 15]);
-#pragma unroll
-                    for (int a = 1; a < P.nacc1; ++a) x += __uint_as_float(vr[a][n >> 4][n & 15]);
-                    return x;
-                };
+                for (int c0 = 0; c0 < P.n1p; c0 += 16) tmem_regs_ready(vr[c0 / 16]);
+                auto v = [&](int n) { return __uint_as_float(vr[n >> 4][n & 15]); };
                 fence_before();
-                mbar_arrive(&bars.acc1_empty[j]);
-                if constexpr (kPrefetch) {
-                    if (c == 0 && tile + (int)gridDim.x < ntiles) fetch_y(tile + gridDim.x, ynext);
-                }
+                mbar_arrive(&bars.acc1_empty[g & 1]);
+                // the set's previous chunk has been read out of the buffer
+                if (zcount > 0 && !wait_warp(&bars.zs_r[set], (zcount - 1) & 1, abort_flag)) { ok = false; break; }
                 if (t < P.rows) {
                     const int b = t / D2, ib = t % D2;
+                    float* zrow = zbuf + b * D2 * P.zs;
+                    constexpr int NCH = P.pc >= 4 ? P.pc / 4 : 1;   // 16-byte chunks this row's values span
+                    // chunk of the values, with the permutation by row & 7 = (b D^2 & 7) ^ ok
+                    // (D^2 is 4 or a multiple of 8 where the chunks are permuted)
+                    const int ch0 = ((ib * P.pc) >> 2) ^ (P.zswz ? (b * D2) & 7 : 0);
+                    int xo[P.zswz ? 8 : 1];
+                    if constexpr (P.zswz && NCH == 1) {
+#pragma unroll
+                        for (int m = 0; m < 8; ++m) xo[m] = ((ch0 ^ m) << 2) + ((ib * P.pc) & 3);
+                    }
 #pragma unroll
                     for (int ok_ = 0; ok_ < D2; ++ok_) {
-                        float* dst = zbuf + (b * D2 + ok_) * P.zs + ib * P.pc;
-                        if constexpr (P.pc % 4 == 0) {
 #pragma unroll
-                            for (int pl = 0; pl < P.pc; pl += 4)
-                                *(float4*)(dst + pl) = make_float4(v(pl * D2 + ok_), v((pl + 1) * D2 + ok_),
-                                                                   v((pl + 2) * D2 + ok_), v((pl + 3) * D2 + ok_));
-                        } else if constexpr (P.pc == 2) {
-                            *(float2*)dst = make_float2(v(ok_), v(D2 + ok_));
-                        } else {
-                            *dst = v(ok_);
+                        for (int e = 0; e < NCH; ++e) {
+                            float* dst;
+                            if constexpr (P.zswz && NCH == 1) dst = zrow + ok_ * P.zs + xo[ok_ & 7];
+                            else if constexpr (P.zswz) dst = zrow + ok_ * P.zs + ((ch0 ^ e ^ (ok_ & 7)) << 2);
+                            else dst = zrow + ok_ * P.zs + ib * P.pc + 4 * e;
+                            if constexpr (P.pc >= 4)
+                                *(float4*)dst = make_float4(v(4 * e * D2 + ok_), v((4 * e + 1) * D2 + ok_),
+                                                            v((4 * e + 2) * D2 + ok_), v((4 * e + 3) * D2 + ok_));
+                            else if constexpr (P.pc == 2) *(float2*)dst = make_float2(v(ok_), v(D2 + ok_));
+                            else *dst = v(ok_);
                         }
                     }
                 }
                 mbar_arrive(&bars.zs_w[set]);
                 if (!wait_warp(&bars.zs_w[set], zcount & 1, abort_flag)) { ok = false; break; }
                 // ---- row (b, ok) of Z -> tensor memory (bra GEMM A operand)
-                const int ja = (int)(g % P.na2);
-                if (!wait_warp(&bars.a2_empty[ja], (uint32_t)((g / P.na2) & 1) ^ 1, abort_flag)) {
-                    ok = false;
-                    break;
-                }
-                fence_after();
                 constexpr int K2R = pad_to(P.k2, 4);          // values read per row
-                constexpr int K2S = pad_to(P.k2p, BF ? 32 : 16);   // values stored per row (whole 16-column groups)
-                float z[K2S];
+                float z[P.k2p];
 #pragma unroll
-                for (int i = 0; i < K2S; ++i) z[i] = 0.f;
+                for (int i = 0; i < P.k2p; ++i) z[i] = 0.f;
                 if (t < P.rows) {
                     const float* src = zbuf + t * P.zs;
+                    int xo[8];
+#pragma unroll
+                    for (int m = 0; m < 8; ++m) xo[m] = (P.zswz ? m ^ (t & 7) : m) << 2;
 #pragma unroll
                     for (int i = 0; i < K2R; i += 4) {
-                        const float4 w = *(const float4*)(src + i);
+                        const float4 w = *(const float4*)(src + (i & ~31) + xo[(i >> 2) & 7]);
                         z[i] = w.x;
                         if (i + 1 < P.k2) z[i + 1] = w.y;
                         if (i + 2 < P.k2) z[i + 2] = w.z;
                         if (i + 3 < P.k2) z[i + 3] = w.w;
                     }
                 }
-                const uint32_t a2 = tmem + lane_base + (uint32_t)(P.c_a2 + ja * NPL * P.a2_cols);
-                if constexpr (BF) {
-                    // two BF16 values per column, the lower K index in the low half
-#pragma unroll
-                    for (int c0 = 0; c0 < K2S / 2; c0 += 16) {
-                        float w[16];
-#pragma unroll
-                        for (int i = 0; i < 16; ++i)
-                            w[i] = __uint_as_float(pack_bf16x2(z[2 * (c0 + i)], z[2 * (c0 + i) + 1]));
-                        tmem_st16(a2 + (uint32_t)c0, w);
-                    }
-                } else {
-#pragma unroll
-                    for (int c0 = 0; c0 < K2S; c0 += 16) {
-                        float hi[16], lo[16];
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) {
-                            const float x = z[c0 + i];
-                            hi[i] = NPASS == 3 ? tf32_hi(x) : x;
-                            lo[i] = x - hi[i];
-                        }
-                        tmem_st16(a2 + (uint32_t)c0, hi);
-                        if (NPASS == 3) tmem_st16(a2 + (uint32_t)(P.a2_cols + c0), lo);
-                    }
+                mbar_arrive(&bars.zs_r[set]);
+                // the bra GEMM of chunk g - na2 has read this Z buffer
+                const int ja = (int)(g % P.na2);
+                const long long h = g - P.na2;
+                if (h >= 0 && !wait_warp(&bars.a2_empty[h & 1], (uint32_t)((h >> 1) & 1), abort_flag)) {
+                    ok = false;
+                    break;
                 }
+                fence_after();
+                store_a(tmem + lane_base + (uint32_t)(P.c_a2 + ja * NPL * P.a2_cols),
+                        std::integral_constant<int, P.a2_cols>{}, P.a2_cols, z);
                 tmem_st_wait();
                 fence_before();
                 mbar_arrive(&bars.a2_full[ja]);
-                mbar_arrive(&bars.zs_r[set]);
-                if (!wait_warp(&bars.zs_r[set], zcount & 1, abort_flag)) { ok = false; break; }
                 ++zcount;
             }
             if (!ok) break;
-            // next tile's Y once the ket GEMMs of this tile have read it
-            const int next = tile + gridDim.x;
-            if (next < ntiles) {
-                if (!wait_warp(&bars.a1_empty, it & 1, abort_flag)) { ok = false; break; }
-                if constexpr (kPrefetch) store_y(ynext);
-                else load_y(next);
-            }
             if (set != 0) continue;
-            // ---- output rows (b, ok) (first set)
+            // ---- next tile's Y once the ket GEMMs of this tile have read it
+            if (next < ntiles) {
+                if (!wait_warp(&bars.y_empty, it & 1, abort_flag)) { ok = false; break; }
+                fence_after();
+                load_y(next);
+            }
+            // ---- output rows (b, ok)
             if (!wait_warp(&bars.out_full, it & 1, abort_flag)) { ok = false; break; }
             fence_after();
-            uint32_t orr[P.nacc2][P.n2p / 16][16];
-#pragma unroll
-            for (int a = 0; a < P.nacc2; ++a)
-#pragma unroll
-                for (int c0 = 0; c0 < P.n2p; c0 += 16)
-                    tmem_ld16_async(tmem + lane_base + (uint32_t)(P.c_out + a * P.out_cols + c0), orr[a][c0 / 16]);
-            tmem_ld_wait();
             float o[P.n2p];
 #pragma unroll
-            for (int c0 = 0; c0 < P.n2p; c0 += 16) {
+            for (int a = P.nacc2 - 1; a >= 0; --a) {           // the small products first
+                uint32_t orr[P.n2p / 16][16];
 #pragma unroll
-                for (int a = 0; a < P.nacc2; ++a) tmem_regs_ready(orr[a][c0 / 16]);
+                for (int c0 = 0; c0 < P.n2p; c0 += 16)
+                    tmem_ld16_async(tmem + lane_base + (uint32_t)(P.c_out + a * P.out_cols + c0), orr[c0 / 16]);
+                tmem_ld_wait();
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    float x = __uint_as_float(orr[0][c0 / 16][i]);
+                for (int c0 = 0; c0 < P.n2p; c0 += 16) {
+                    tmem_regs_ready(orr[c0 / 16]);
 #pragma unroll
-                    for (int a = 1; a < P.nacc2; ++a) x += __uint_as_float(orr[a][c0 / 16][i]);
-                    o[c0 + i] = x;
+                    for (int i = 0; i < 16; ++i) {
+                        const float x = __uint_as_float(orr[c0 / 16][i]);
+                        o[c0 + i] = a == P.nacc2 - 1 ? x : o[c0 + i] + x;
+                    }
                 }
             }
             fence_before();
@@ -561,14 +558,14 @@ void launch_layered(const float* Y, long long nb, int p, const float* img1, cons
     if (ntiles_ll > 0x7fffffffLL) fail(KH_EINVAL, "layered site contraction: too many tiles");
     const int ntiles = (int)ntiles_ll;
     if (ntiles == 0) return;
-    const size_t fixed = 1024 + (size_t)NPL * P.a1_bytes + (size_t)lay::NSET * 128 * P.zs * 4;
+    const size_t fixed = 1024 + (size_t)lay::NSET * 128 * P.zs * 4;
     const size_t s1 = (size_t)NPL * P.b1_bytes, s2 = (size_t)NPL * P.b2_bytes;
     const size_t cap = (size_t)smem_optin_max() - 2048;   // the static barriers share the per-block limit
     int nst1 = 0, nst2 = 0;
     if (nc <= lay::MAXST && fixed + nc * (s1 + s2) <= cap) {
         nst1 = nst2 = nc;                                  // resident images
     } else {
-        const int tries[4][2] = {{2, 2}, {2, 1}, {1, 2}, {1, 1}};
+        const int tries[6][2] = {{3, 3}, {2, 3}, {2, 2}, {1, 2}, {2, 1}, {1, 1}};
         for (auto& tr : tries) {
             const int a = tr[0] < nc ? tr[0] : nc, b = tr[1] < nc ? tr[1] : nc;
             if (fixed + a * s1 + b * s2 <= cap) {
@@ -624,7 +621,7 @@ long long layered_img2_floats(int D, int p, int npass, bool bf16) {
 void site_layered_tc(const float* Y, long long nb, int D, int p, const float* img1, const float* img2, float* out,
                      int npass, bool bf16, int* err, cudaStream_t st) {
     if (nb <= 0) return;
-    if (((uintptr_t)img1 & 15) || ((uintptr_t)img2 & 15) || ((uintptr_t)out & 15) || ((uintptr_t)Y & 3))
+    if (((uintptr_t)img1 & 15) || ((uintptr_t)img2 & 15) || ((uintptr_t)out & 15) || ((uintptr_t)Y & 15))
         fail(KH_EINVAL, "layered site contraction: misaligned operand");
     if (bf16) {
         if (npass != 1) fail(KH_EINVAL, "layered site contraction: BF16 runs one pass");

@@ -30,27 +30,28 @@ __host__ __device__ constexpr int pad_to(int x, int m) { return (x + m - 1) / m 
 struct Plan {
     int esz = 4, kstep = 8;                  // element bytes; K per MMA
     int d2 = 0, bt = 0, rows = 0;            // D^2; blocks b per tile; rows (b, ib) used of 128
-    int pc = 0, na2 = 0;                     // physical indices per chunk; Z buffers in tensor memory
-    int nacc1 = 0, nacc2 = 0;                // independent accumulators of the ket and the bra GEMM
+    int pc = 0, nb1 = 0, na2 = 0;            // physical indices per chunk; ket accumulators; Z buffers
+    int nm = 0, nacc2 = 0;                   // bra accumulators: of the leading products, and in all
     int n1 = 0, n1p = 0, k1p = 0, kb1 = 0;   // ket GEMM: N = pc D^2 (padded to 16), K = D^2 (padded to kstep)
     int n2p = 0, k2 = 0, k2p = 0, kb2 = 0;   // bra GEMM: N = D^2 (padded to 16), K = pc D^2 (padded to kstep)
     int zs = 0;                              // row stride (floats) of the shared-memory transpose buffer
+    bool zswz = false;                       // its 16-byte chunks permuted by the row
     int acc1_cols = 0, out_cols = 0;         // columns of one ket / bra accumulator (32-aligned)
-    int c_acc1 = 0, c_a2 = 0, a2_cols = 0, c_out = 0, tmem = 0;   // tensor-memory columns
-    int a1_bytes = 0, b1_bytes = 0, b2_bytes = 0;                 // one (hi or lo) operand image
+    int c_acc1 = 0, c_out = 0, c_a2 = 0, a2_cols = 0, c_y = 0, y_cols = 0, tmem = 0;   // tensor-memory columns
+    int b1_bytes = 0, b2_bytes = 0;          // one (hi or lo) operand image
 };
 
-// The tensor core runs consecutive MMAs into one accumulator as a dependent
-// chain; these GEMMs are thin (N = D^2 for the bra layer), so the chain's
-// latency, not the MMA throughput, sets the time.  Each GEMM therefore
-// spreads its MMAs round-robin over nacc independent accumulators (summed
-// when read).  The plan picks pc (a power of two <= 16), the accumulator
-// counts and the Z double buffering that fit the 512 tensor-memory columns
-// (every region 32-column aligned: two ket buffers of nacc1 accumulators, na2
-// Z buffers (hi and lo with 3 passes), nacc2 bra accumulators), minimising a
-// latency model: per chunk one worker hand-off plus the two dependent MMA
-// chains (0.1 of a hand-off per chained MMA).  Shared-memory operands use the
-// 128-byte-swizzle K-major layout in K blocks of 128 bytes.
+// Tensor-memory regions (512 columns): nb1 ket accumulators and nacc2 bra
+// accumulators (32-column aligned), then the A operands, packed: na2 Z buffers
+// and the Y tile, hi and lo with 3 passes.  The bra accumulators live through
+// all chunks of a tile, and the tensor core truncates an accumulator at every
+// instruction: with 3 passes the products of remainders have one of their own,
+// so that they do not truncate the leading sum, which is spread over nm.  The
+// plan picks pc (a power of two <= 16), nm, nb1 and na2, minimising a model of the
+// tensor pipe: an MMA of N columns takes about 20 + 0.64 N clocks (measured on
+// this kernel at N = 48 and 64 and on gemm3x.cu at 160), a chunk 100 more for
+// its hand-off and 100 for each operand that has one buffer only.  Shared-memory
+// operands use the 128-byte-swizzle K-major layout in K blocks of 128 bytes.
 __host__ __device__ constexpr Plan make_plan(int D, int npass, bool bf16 = false) {
     Plan P{};
     P.esz = bf16 ? 2 : 4;
@@ -67,45 +68,52 @@ __host__ __device__ constexpr Plan make_plan(int D, int npass, bool bf16 = false
     double best = 1e30;
     for (int pc = 16; pc >= 1; pc /= 2) {
         const int n1p = pad_to(pc * P.d2, 16);
-        if (n1p > 256) continue;
+        if (n1p > (npass == 3 ? 96 : 128)) continue;    // a row of Z, or its two parts, fits the workers' registers
         const int k2p = pad_to(pc * P.d2, P.kstep);
-        const int zcols = k2p * P.esz / 4;                // tensor-memory columns of one Z operand
-        const int nc = (16 + pc - 1) / pc;                // chunks at p = 16
+        const int zcols = k2p * P.esz / 4, ycols = P.k1p * P.esz / 4;   // columns of one Z / Y operand
+        const int nc = (16 + pc - 1) / pc;              // chunks at p = 16
         const int mm1 = (P.k1p / P.kstep) * npass, mm2 = (k2p / P.kstep) * npass;
-        for (int nacc2 = 4; nacc2 >= 1; nacc2 /= 2)
-            for (int nacc1 = 2; nacc1 >= 1; --nacc1)
-                for (int na2 = 2; na2 >= 1; --na2) {
-                    if (nacc1 > mm1 || nacc2 > mm2) continue;
-                    const int cols = 2 * nacc1 * pad_to(n1p, 32) + na2 * npl * pad_to(zcols, 32) +
-                                     nacc2 * pad_to(P.n2p, 32);
-                    if (cols > 512) continue;
-                    const double cost = nc * (1.0 + 0.1 * ((mm1 + nacc1 - 1) / nacc1) +
-                                              0.1 * ((mm2 + nacc2 - 1) / nacc2)) - 0.01 * na2;
-                    if (cost >= best) continue;
-                    best = cost;
-                    P.pc = pc;
-                    P.na2 = na2;
-                    P.nacc1 = nacc1;
-                    P.nacc2 = nacc2;
-                    P.n1 = pc * P.d2;
-                    P.n1p = n1p;
-                    P.k2 = pc * P.d2;
-                    P.k2p = k2p;
-                    P.kb2 = (k2p + per_block - 1) / per_block;
-                    P.zs = pad_to(P.k2, 4);
-                    if ((P.zs / 4) % 2 == 0) P.zs += 4;          // odd 16-byte stride: conflict-free row reads
-                    P.acc1_cols = pad_to(n1p, 32);
-                    P.out_cols = pad_to(P.n2p, 32);
-                    P.c_acc1 = 0;
-                    P.c_a2 = 2 * nacc1 * P.acc1_cols;
-                    P.a2_cols = pad_to(zcols, 32);
-                    P.c_out = P.c_a2 + na2 * npl * P.a2_cols;
-                    P.tmem = 32;
-                    while (P.tmem < P.c_out + nacc2 * P.out_cols) P.tmem *= 2;
-                    P.a1_bytes = 128 * P.kb1 * 128;
-                    P.b1_bytes = n1p * P.kb1 * 128;
-                    P.b2_bytes = P.n2p * P.kb2 * 128;
-                }
+        const double c1 = 20.0 + 0.64 * n1p, c2 = 20.0 + 0.64 * P.n2p;
+        for (int nm = 2; nm >= 1; --nm)
+            for (int nb = 4; nb >= 1; --nb) {
+                const int nb1 = nb >= 3 ? 2 : 1, na2 = nb % 2 == 0 ? 2 : 1;
+                const int nacc2 = nm + (npass == 3 ? 1 : 0);
+                if (nm > k2p / P.kstep) continue;
+                const int cols = nb1 * pad_to(n1p, 32) + nacc2 * pad_to(P.n2p, 32) + npl * (na2 * zcols + ycols);
+                if (cols > 512) continue;
+                const double cost = nc * (mm1 * c1 + mm2 * c2 + 500.0 - 100.0 * (nb1 + na2)) - nm;
+                if (cost >= best) continue;
+                best = cost;
+                P.pc = pc;
+                P.nb1 = nb1;
+                P.na2 = na2;
+                P.nm = nm;
+                P.nacc2 = nacc2;
+                P.n1 = pc * P.d2;
+                P.n1p = n1p;
+                P.k2 = pc * P.d2;
+                P.k2p = k2p;
+                P.kb2 = (k2p + per_block - 1) / per_block;
+                // an odd number of 16-byte chunks a row, or whole 128-byte rows
+                // with their chunks permuted by the row: conflict-free row reads
+                P.zs = pad_to(P.k2, 4);
+                P.zswz = P.zs % 32 == 0;
+                // (without the odd stride, two-way conflicts, where it would cost the rings a stage)
+                const int rings = 2 * npl * (n1p * P.kb1 + P.n2p * P.kb2) * 128;
+                if (!P.zswz && (P.zs / 4) % 2 == 0 && 1024 + 2 * 128 * (P.zs + 4) * 4 + rings <= 230400) P.zs += 4;
+                P.acc1_cols = pad_to(n1p, 32);
+                P.out_cols = pad_to(P.n2p, 32);
+                P.c_acc1 = 0;
+                P.c_out = nb1 * P.acc1_cols;
+                P.c_a2 = P.c_out + nacc2 * P.out_cols;
+                P.a2_cols = zcols;
+                P.c_y = P.c_a2 + na2 * npl * zcols;
+                P.y_cols = ycols;
+                P.tmem = 32;
+                while (P.tmem < cols) P.tmem *= 2;
+                P.b1_bytes = n1p * P.kb1 * 128;
+                P.b2_bytes = P.n2p * P.kb2 * 128;
+            }
     }
     return P;
 }

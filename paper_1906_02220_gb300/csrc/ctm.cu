@@ -1351,6 +1351,11 @@ static void svd_jacobi_launch(const T* X, int k, T* sv, T* L, T* Qm, int max_swe
     KH_LAUNCHED();
 }
 
+// FP64 matrices beyond this size go to the cluster kernel: 64 x 64 takes 0.50 ms
+// there and 2.05 ms in one CTA (D = 2, chi = 16), 48 x 48 0.10 and 0.16; up to 16
+// columns the cluster's eight CTAs would not have a pair each.
+constexpr int kSvdClusterMin = 16;
+
 // Rows per lane chosen at compile time: 8 lanes per column pair, R (even)
 // rows per lane with 8 R >= kp (at most 640 threads).
 template <typename T>
@@ -1358,6 +1363,12 @@ void svd_jacobi(const T* X, int k, T* sv, T* L, T* Qm, int max_sweeps, double to
                 int* sweep_count, int nrel) {
     if (k > jacobi_kmax<T>() || k < 1) fail(KH_EINVAL, "svd_jacobi: k beyond limit");
     const int kp = (k + 1) & ~1;
+    if constexpr (sizeof(T) == 8) {
+        if (k > kSvdClusterMin) {
+            svd_jacobi_cluster(X, k, sv, L, Qm, max_sweeps, tol, cut, st, sweep_count, nrel);
+            return;
+        }
+    }
 #define KH_SVDJ(LP, R) svd_jacobi_launch<T, LP, R>(X, k, sv, L, Qm, max_sweeps, tol, cut, st, sweep_count, nrel)
     if (kp <= 16) KH_SVDJ(8, 2);
     else if (kp <= 32) KH_SVDJ(8, 4);

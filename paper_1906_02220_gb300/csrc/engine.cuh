@@ -317,6 +317,10 @@ struct TcOperand {
 void tc_gemm(const TcOperand& A, const TcOperand& B, float* C, int M, int N, int K, long long ldc, float alpha,
              float beta, const float* colscale, int* err, cudaStream_t st);
 
+// FP64 one-sided Jacobi SVD on a cluster of eight CTAs (svd_cluster.cu), k <= 112
+void svd_jacobi_cluster(const double* X, int k, double* s, double* L, double* Q, int max_sweeps, double tol,
+                        double cut, cudaStream_t st, int* sweep_count, int nrel);
+
 int device_sms();      // SMs of the current device (layered.cu)
 
 // FP32-accurate tensor-core GEMM (gemm3x.cu): C = alpha colscale (A B), A raw

@@ -598,7 +598,7 @@ __global__ void sumsq_kernel(const T* __restrict__ x, long long n, double* out) 
     double s = 0.0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
-        double v = (double)x[i];
+        double v = f2d(x[i]);
         s += v * v;
     }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);

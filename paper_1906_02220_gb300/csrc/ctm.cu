@@ -14,6 +14,8 @@
 //   P = Q_{s+3}^T V S^-1/2, P~^T = Q_s U S^-1/2;
 //   C1 <- P^T (C1 E1), C4 <- (C4 E3) P~^T, E4 <- P^T (E4 T T) P~^T,
 //   each divided by its Frobenius norm (FP64).
+#include <algorithm>
+
 #define KH_JACOBI_KERNEL
 #include "engine.cuh"
 #include "layered.cuh"
@@ -297,66 +299,111 @@ __global__ void rand_kernel(T* V, long long tot, uint64_t seed, uint64_t stream)
         V[i] = (T)rnd_uniform(seed, stream, (uint64_t)i);
 }
 
-// Gram G = Z^T Z (Z: n x k row-major, k <= 16 KT): one CTA per chunk of rows,
-// staged in shared memory; thread (ti, tj) of a 16 x 16 grid holds the
-// KT x KT register tile G[ti + 16 a][tj + 16 b] and accumulates it over the
-// chunk (in T), then adds it to the FP64 result.
-template <typename T, int KT>
+// Gram matrix G += Z^T Z2 (n x k row-major, Z2 = Z in the symmetric case): a CTA
+// takes one tile of 16 KT x 16 KT entries over a range of rows; thread (ti, tj)
+// of a 16 x 16 grid holds the entries (ti + 16 a, tj + 16 b).  FP32 products are
+// summed in FP32 over 16 rows and the sums of the chunks as unevaluated pairs of
+// FP32 numbers (two-sum, ~2^-47, which costs less here than FP64 additions),
+// then added to the FP64 result.  What bounds it is those FP64 atomics: k^2 a
+// range of rows, so the ranges are long (one CTA per SM over all tiles), and
+// the symmetric case computes the lower triangle of tiles only.  5184 x 160:
+// 19 us, with full ranges of 16 rows and k^2 atomics each 64; 1024 x 80: 6.6 and 9.5.
+template <typename T, int KT, bool SYM>
 __global__ void __launch_bounds__(256) gram_kernel(const T* __restrict__ Z, const T* __restrict__ Z2, int n, int k,
-                                                   double* __restrict__ G, int rows_per) {
-    extern __shared__ unsigned char smem_raw[];
-    T* Ys = reinterpret_cast<T*>(smem_raw);   // rows_per x k (Z), then rows_per x k (Z2) when given
-    T* Ys2 = Z2 ? Ys + rows_per * k : Ys;
-    const int r0 = blockIdx.x * rows_per, nr = min(rows_per, n - r0);
-    for (int e = threadIdx.x; e < nr * k; e += blockDim.x) Ys[e] = Z[(long long)r0 * k + e];
-    if (Z2)
-        for (int e = threadIdx.x; e < nr * k; e += blockDim.x) Ys2[e] = Z2[(long long)r0 * k + e];
-    __syncthreads();
-    const int ti = threadIdx.x >> 4, tj = threadIdx.x & 15;
-    T acc[KT][KT];
+                                                   int nt, double* __restrict__ G, int rows_cta) {
+    constexpr int TS = 16 * KT, CH = 16;
+    __shared__ T As[CH][TS], Bs[CH][TS];
+    const int y = blockIdx.y;
+    const int bi = SYM ? (y == 0 ? 0 : 1) : y / nt, bj = SYM ? (y == 2 ? 1 : 0) : y % nt;
+    const int i0 = bi * TS, j0 = bj * TS;
+    const int rbeg = blockIdx.x * rows_cta, rend = min(n, rbeg + rows_cta);
+    const int tid = threadIdx.x, ti = tid >> 4, tj = tid & 15;
+    T hi[KT][KT], lo[KT][KT], ra[KT], rb[KT];
 #pragma unroll
     for (int a = 0; a < KT; ++a)
 #pragma unroll
-        for (int b = 0; b < KT; ++b) acc[a][b] = T(0);
-    for (int r = 0; r < nr; ++r) {
-        const T* y = Ys + r * k;
-        const T* y2 = Ys2 + r * k;
-        T yi[KT], yj[KT];
+        for (int b = 0; b < KT; ++b) hi[a][b] = lo[a][b] = T(0);
+    auto load = [&](int r0) {
 #pragma unroll
-        for (int a = 0; a < KT; ++a) {
-            const int i = ti + 16 * a, j = tj + 16 * a;
-            yi[a] = i < k ? y[i] : T(0);
-            yj[a] = j < k ? y2[j] : T(0);
+        for (int q = 0; q < KT; ++q) {
+            const int e = tid + 256 * q, r = r0 + e / TS, c = e % TS;
+            ra[q] = (r < rend && i0 + c < k) ? Z[(long long)r * k + i0 + c] : T(0);
+            rb[q] = (r < rend && j0 + c < k) ? Z2[(long long)r * k + j0 + c] : T(0);
         }
+    };
+    load(rbeg);
+    for (int r0 = rbeg; r0 < rend; r0 += CH) {
+#pragma unroll
+        for (int q = 0; q < KT; ++q) {
+            const int e = tid + 256 * q;
+            As[e / TS][e % TS] = ra[q];
+            Bs[e / TS][e % TS] = rb[q];
+        }
+        __syncthreads();
+        if (r0 + CH < rend) load(r0 + CH);
+        T acc[KT][KT];
 #pragma unroll
         for (int a = 0; a < KT; ++a)
 #pragma unroll
-            for (int b = 0; b < KT; ++b) acc[a][b] = fma(yi[a], yj[b], acc[a][b]);
+            for (int b = 0; b < KT; ++b) acc[a][b] = T(0);
+#pragma unroll 4
+        for (int r = 0; r < CH; ++r) {
+            T yi[KT], yj[KT];
+#pragma unroll
+            for (int a = 0; a < KT; ++a) {
+                yi[a] = As[r][ti + 16 * a];
+                yj[a] = Bs[r][tj + 16 * a];
+            }
+#pragma unroll
+            for (int a = 0; a < KT; ++a)
+#pragma unroll
+                for (int b = 0; b < KT; ++b) acc[a][b] = fma(yi[a], yj[b], acc[a][b]);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int a = 0; a < KT; ++a)
+#pragma unroll
+            for (int b = 0; b < KT; ++b) {
+                if constexpr (sizeof(T) == 8) {
+                    hi[a][b] += acc[a][b];
+                } else {
+                    const T s = hi[a][b] + acc[a][b], d = s - hi[a][b];      // s + err = hi + acc exactly
+                    lo[a][b] += (hi[a][b] - (s - d)) + (acc[a][b] - d);
+                    hi[a][b] = s;
+                }
+            }
     }
 #pragma unroll
     for (int a = 0; a < KT; ++a)
 #pragma unroll
         for (int b = 0; b < KT; ++b) {
-            const int i = ti + 16 * a, j = tj + 16 * b;
-            if (i < k && j < k) atomicAdd(&G[i * k + j], (double)acc[a][b]);
+            const int i = i0 + ti + 16 * a, j = j0 + tj + 16 * b;
+            if (i < k && j < k) {
+                const double v = f2d(hi[a][b]) + f2d(lo[a][b]);
+                atomicAdd(&G[i * k + j], v);
+                if (SYM && bi != bj) atomicAdd(&G[j * k + i], v);
+            }
         }
 }
 
-// G = Z^T Z2 (Z2 = Z when null), k x k, accumulated in T over chunks of 16
-// rows and in FP64 across chunks.
+// G = Z^T Z2 (Z2 = Z when null), k x k.
 template <typename T>
 void gram(const T* Z, int n, int k, double* dG, cudaStream_t st, const T* Z2 = nullptr) {
     if (k > 160) fail(KH_EINVAL, "gram: k > 160");
     KH_CUDA(cudaMemsetAsync(dG, 0, sizeof(double) * k * k, st));
-    const int nmat = Z2 ? 2 : 1;
-    int rows_per = (int)((48 * 1024) / (sizeof(T) * k * nmat));   // stay within the default shared-memory limit
-    if (rows_per > 16) rows_per = 16;
-    const int grid = (n + rows_per - 1) / rows_per;
-    const size_t sm = sizeof(T) * rows_per * k * nmat;
-    switch ((k + 15) / 16) {
-#define KH_GRAM(KT) case KT: gram_kernel<T, KT><<<grid, 256, sm, st>>>(Z, Z2, n, k, dG, rows_per); break;
+    const int nt = k <= 48 ? 1 : 2;                                  // tiles along a side
+    const int kt = ((k + nt - 1) / nt + 15) / 16;
+    const int tiles = Z2 ? nt * nt : nt * (nt + 1) / 2;
+    const int want = std::max(1, std::min((n + 31) / 32, 152 / tiles));
+    const int rows = ((n + want - 1) / want + 15) / 16 * 16;
+    const dim3 grid((n + rows - 1) / rows, tiles);
+    switch (kt) {
+#define KH_GRAM(KT)                                                                                            \
+    case KT:                                                                                                   \
+        if (Z2) gram_kernel<T, KT, false><<<grid, 256, 0, st>>>(Z, Z2, n, k, nt, dG, rows);                    \
+        else gram_kernel<T, KT, true><<<grid, 256, 0, st>>>(Z, Z, n, k, nt, dG, rows);                         \
+        break;
         KH_GRAM(1) KH_GRAM(2) KH_GRAM(3) KH_GRAM(4) KH_GRAM(5)
-        KH_GRAM(6) KH_GRAM(7) KH_GRAM(8) KH_GRAM(9) KH_GRAM(10)
 #undef KH_GRAM
     }
     KH_LAUNCHED();
@@ -410,9 +457,10 @@ __global__ void store_normalized_kernel(const T* x, long long n, const double* s
     double inv = s > 0.0 ? 1.0 / sqrt(s) : 1.0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
-        double v = (double)x[i] * inv;
+        double v = f2d(x[i]) * inv;
         master[i] = v;
-        op[i] = (T)v;
+        if constexpr (sizeof(T) == 4) op[i] = d2f(v);
+        else op[i] = v;
     }
 }
 
@@ -939,7 +987,9 @@ void Engine<T>::projector(Slot<T>& sl, int dir, int slot_id) {
         KH_CUDA(cudaMemcpyAsync(Vw, Z1, sizeof(T) * (size_t)n * k, cudaMemcpyDeviceToDevice, st));
         {
             const int thr = 256 / k > 0 ? 256 / k * k : k;
-            live_mask_kernel<T><<<16, thr, sizeof(float) * thr, st>>>(
+            // a CTA per 64 rows or so: 16 CTAs took 148 us at n = 5184, k = 160
+            const int blocks = std::min(152, std::max(16, n / 64));
+            live_mask_kernel<T><<<blocks, thr, sizeof(float) * thr, st>>>(
                 Z1, n, k, live, (float*)(dscr + DscrOff::kLiveAcc), (int*)(dscr + DscrOff::kLiveCount));
         }
         KH_LAUNCHED();
@@ -1388,10 +1438,25 @@ template <typename T>
 void cholqr_factor(const double* dG, int k, double cut_abs, double tau, T* X, cudaStream_t st, bool sorted,
                    double ns_tol, double defer) {
     if (k > jacobi_kmax<T>()) fail(KH_EINVAL, "cholqr: k beyond limit");
-    const size_t sm = (size_t)2 * k * (k | 1) * sizeof(T);
-    static std::atomic<size_t> granted[kMaxDevices] = {};
-    smem_opt_in(cholqr_kernel<T>, sm, granted);
-    cholqr_kernel<T><<<1, 1024, sm, st>>>(dG, k, cut_abs, tau, X, sorted ? 1 : 0, ns_tol, defer);
+    const size_t sm = (size_t)k * (k | 1) * sizeof(T);
+    if constexpr (sizeof(T) == 4) {
+        if (defer > tau) fail(KH_EINVAL, "cholqr: the FP32 factor defers no pivot");
+        switch ((k + 31) / 32) {
+#define KH_CHOL(KT)                                                                                          \
+    case KT: {                                                                                               \
+        static std::atomic<size_t> granted[kMaxDevices] = {};                                                \
+        smem_opt_in(cholqr_reg_kernel<T, KT>, sm, granted);                                                  \
+        cholqr_reg_kernel<T, KT><<<1, 512, sm, st>>>(dG, k, cut_abs, tau, X, sorted ? 1 : 0, ns_tol);        \
+        break;                                                                                               \
+    }
+            KH_CHOL(1) KH_CHOL(2) KH_CHOL(3) KH_CHOL(4) KH_CHOL(5)
+#undef KH_CHOL
+        }
+    } else {
+        static std::atomic<size_t> granted[kMaxDevices] = {};
+        smem_opt_in(cholqr_kernel<T>, 2 * sm, granted);
+        cholqr_kernel<T><<<1, 1024, 2 * sm, st>>>(dG, k, cut_abs, tau, X, sorted ? 1 : 0, ns_tol, defer);
+    }
     KH_LAUNCHED();
 }
 template void cholqr_factor<float>(const double*, int, double, double, float*, cudaStream_t, bool, double, double);

@@ -765,6 +765,206 @@ cholqr_kernel(const double* __restrict__ G, int k, double cut_abs, double tau, T
     cholqr_epilogue<T>(k, tau, X, Lm, Li, ld, sh);
 }
 
+// The factor of the orders that defer no pivot (the single-precision paths), in
+// registers: thread (tx, ty) of a 32 x 16 grid holds rows ty + 16 a and columns
+// tx + 32 b of the matrix.  Elimination by panels of four pivots, in place as in
+// Gauss-Jordan: for a pivot j every row i > j gets x_ic -= (a_ij / d_j) y_c with y
+// the pivot row, whose entries right of the diagonal are the Schur complement's
+// and left of it those of the unit triangular inverse, so that the inverse is
+// complete with the factor and no triangular solve follows.  Per panel its four
+// rows (one warp each) go to shared memory; one thread per column eliminates
+// within the 4 x 4 block and carries the column through it (y; by symmetry also
+// a_ij, scaled to z); then every thread subtracts four products per entry.  What
+// bounds it is that chain: two barriers, four reciprocals.  k = 80: 19 us and, with the Newton-Schulz
+// shortcut, 6; the shared-memory kernel above 32 and 9.  k = 160: 68 and 16, 100 and 18.
+template <typename T>
+struct alignas(4 * sizeof(T)) Quad {
+    T v[4];
+};
+template <typename T, int KT>
+__global__ void __launch_bounds__(512, 1)
+cholqr_reg_kernel(const double* __restrict__ G, int k, double cut_abs, double tau, T* __restrict__ X, int sorted,
+                  double ns_tol) {
+    extern __shared__ unsigned char smem_raw[];
+    T* Xs = reinterpret_cast<T*>(smem_raw);        // k x (k | 1): the result, transposed for coalesced rows
+    constexpr int KR = 2 * KT, KM = 32 * KT;       // rows (16 apart) and KT columns (32 apart) of a thread
+    __shared__ Quad<T> P[KM], Y[KM], Z[KM];        // .[c].v[q]: column c of the panel's row q
+    __shared__ T s_diag[KM], s_inv[KM], s_piv[KM], s_red[16];
+    __shared__ int s_perm[KM];
+    const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
+    const T tauT = (T)tau, cutT = (T)cut_abs;
+    for (int j = tid; j < k; j += 512) s_diag[j] = fmax(d2f(G[(long long)j * k + j]), T(0));
+    __syncthreads();
+    T w[KR][KT];
+    auto block_max = [&](T x) {
+        for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, o));
+        if (tx == 0) s_red[ty] = x;
+        __syncthreads();
+        x = T(0);
+#pragma unroll
+        for (int q = 0; q < 16; ++q) x = fmax(x, s_red[q]);
+        return x;
+    };
+    if (ns_tol > 0.0) {
+        // Gram of the nonzero columns close to the identity: one Newton-Schulz step
+        T dev = T(0);
+#pragma unroll
+        for (int a = 0; a < KR; ++a)
+#pragma unroll
+            for (int b = 0; b < KT; ++b) {
+                const int i = ty + 16 * a, c = tx + 32 * b;
+                // no branch around a load: all of a thread's loads in flight together
+                const T x = d2f(G[(long long)min(i, k - 1) * k + min(c, k - 1)]);
+                w[a][b] = (i < k && c < k) ? x : T(0);
+            }
+#pragma unroll
+        for (int a = 0; a < KR; ++a)
+#pragma unroll
+            for (int b = 0; b < KT; ++b) {
+                const int i = ty + 16 * a, c = tx + 32 * b;
+                const bool live = s_diag[min(i, k - 1)] > T(0) && s_diag[min(c, k - 1)] > T(0) && i < k && c < k;
+                dev = fmax(dev, live ? fabs(w[a][b] - (i == c ? T(1) : T(0))) : T(0));
+            }
+        dev = block_max(dev);
+        if (dev < (T)ns_tol) {
+#pragma unroll
+            for (int a = 0; a < KR; ++a)
+#pragma unroll
+                for (int b = 0; b < KT; ++b) {
+                    const int i = ty + 16 * a, c = tx + 32 * b;
+                    if (i < k && c < k)
+                        X[(long long)i * k + c] = (s_diag[i] > T(0) && s_diag[c] > T(0))
+                                                      ? ((i == c ? T(1.5) : T(0)) - T(0.5) * w[a][b]) : T(0);
+                }
+            return;
+        }
+        __syncthreads();                           // s_red is used again
+    }
+    T mx = T(0);
+    for (int j = tid; j < k; j += 512) mx = fmax(mx, s_diag[j]);
+    mx = sqrt(block_max(mx));
+    for (int j = ty; j < k; j += 16) {             // a warp per column: its place in the order
+        const T dj = s_diag[j];
+        int rank = j;
+        if (sorted) {
+            rank = 0;
+            for (int i = tx; i < k; i += 32) rank += (s_diag[i] > dj) || (s_diag[i] == dj && i < j);
+            rank = __reduce_add_sync(0xffffffffu, rank);
+        }
+        if (tx == 0) {
+            const T nj = sqrt(dj);
+            s_inv[j] = (mx > T(0) && nj > cutT * mx) ? T(1) / nj : T(0);
+            s_perm[rank] = j;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < KR; ++a)
+#pragma unroll
+        for (int b = 0; b < KT; ++b) {
+            const int i = ty + 16 * a, c = tx + 32 * b;
+            const int pa = s_perm[min(i, k - 1)], pb = s_perm[min(c, k - 1)];
+            const T x = d2f(G[(long long)pa * k + pb]) * s_inv[pa] * s_inv[pb];
+            w[a][b] = (i < k && c < k) ? x : T(0);
+        }
+#pragma unroll
+    for (int a0 = 0; a0 < KR; ++a0) {
+#pragma unroll 1
+        for (int p4 = 0; p4 < 4; ++p4) {
+            const int j0 = 16 * a0 + 4 * p4;
+            if (j0 >= k) break;
+            const bool pivot_row = (ty >> 2) == p4;            // this warp holds row j0 + (ty & 3)
+            if (pivot_row) {
+#pragma unroll
+                for (int b = 0; b < KT; ++b) P[tx + 32 * b].v[ty & 3] = w[a0][b];
+            }
+            __syncthreads();
+            if (tid < KM) {                                    // one thread per column
+                // the 4 x 4 block: multipliers m and reciprocal pivots (0: dropped, updates nothing)
+                T x[4][4], m[4][4], rd[4];
+#pragma unroll
+                for (int p = 0; p < 4; ++p) {
+                    const Quad<T> u = P[j0 + p];
+#pragma unroll
+                    for (int q = p; q < 4; ++q) x[q][p] = u.v[q];
+                }
+                Quad<T> u = P[tid];
+#pragma unroll
+                for (int p = 0; p < 4; ++p) {
+                    rd[p] = x[p][p] > tauT ? chol_recip(x[p][p]) : T(0);
+#pragma unroll
+                    for (int q = p + 1; q < 4; ++q) m[q][p] = x[q][p] * rd[p];
+#pragma unroll
+                    for (int q = p + 1; q < 4; ++q)
+#pragma unroll
+                        for (int c = p + 1; c <= q; ++c) x[q][c] -= m[q][p] * x[c][p];
+                }
+                // the panel's own columns start as unit vectors: the inverse's block
+                const int own = tid - j0;
+                if (own >= 0 && own < 4) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        if (q == own) s_piv[tid] = x[q][q];
+                        u.v[q] = q == own ? T(1) : T(0);
+                    }
+                }
+#pragma unroll
+                for (int q = 1; q < 4; ++q)
+#pragma unroll
+                    for (int c = 0; c < q; ++c) u.v[q] -= m[q][c] * u.v[c];
+                Y[tid] = u;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) u.v[q] = own >= 4 ? u.v[q] * rd[q] : T(0);
+                Z[tid] = u;
+            }
+            __syncthreads();
+            Quad<T> y[KT];
+#pragma unroll
+            for (int b = 0; b < KT; ++b) y[b] = Y[tx + 32 * b];
+            const bool own = (tx >> 2) == ((j0 & 31) >> 2);    // column slot a0 / 2 holds column j0 + (tx & 3)
+#pragma unroll
+            for (int a = a0; a < KR; ++a) {
+                const int i = ty + 16 * a;
+                const Quad<T> z = Z[i];                        // zero for the rows above
+#pragma unroll
+                for (int b = 0; b < KT; ++b) {
+                    T v = (b == a0 / 2 && own && i >= j0 + 4) ? T(0) : w[a][b];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) v -= z.v[q] * y[b].v[q];
+                    w[a][b] = v;
+                }
+            }
+            if (pivot_row) {
+                const int q = ty & 3;
+#pragma unroll
+                for (int b = 0; b < KT; ++b)
+                    w[a0][b] = q == 0 ? y[b].v[0] : q == 1 ? y[b].v[1] : q == 2 ? y[b].v[2] : y[b].v[3];
+            }
+        }
+    }
+    __syncthreads();
+    // X[perm c][i] = inv[perm c] L^-1[i][c], L^-1 = D^-1/2 times the unit inverse
+    // (Q = Y_s L^-T; dropped i give zero columns)
+    const int ld = k | 1;
+#pragma unroll
+    for (int a = 0; a < KR; ++a) {
+        const int i = ty + 16 * a;
+        if (i >= k) continue;
+        const T d = s_piv[i], rs = d > tauT ? T(1) / sqrt(d) : T(0);
+#pragma unroll
+        for (int b = 0; b < KT; ++b) {
+            const int c = tx + 32 * b;
+            if (c < k) Xs[c * ld + i] = c > i ? T(0) : (c == i ? rs : rs * w[a][b]);
+        }
+    }
+    __syncthreads();
+    for (int c = ty; c < k; c += 16) {
+        const int pc = s_perm[c];
+        const T f = s_inv[pc];
+        for (int i = tx; i < k; i += 32) X[(long long)pc * k + i] = f * Xs[c * ld + i];
+    }
+}
+
 #endif  // KH_JACOBI_KERNEL
 
 }  // namespace kh

@@ -500,55 +500,73 @@ inline void gemm_dispatch(const GemmArgs<T>& g, cudaStream_t st) {
     else gemm_launch<T, 64, 64, 4, 4>(g, st);
 }
 
+// Few output tiles and a long K (FP32): the partial products of K split over
+// CTAs go to the scratch as parts of M x N each, and their number is returned;
+// 0 where K is not split (nothing is launched).
+template <typename T>
+inline int gemm_parts(const GemmArgs<T>& g, cudaStream_t st) {
+    const long long tiles = (long long)((g.M + 63) / 64) * ((g.N + 63) / 64);
+    if (sizeof(T) == 8 || g.batch != 1 || !g.sk || tiles >= 76 || g.K < 256) return 0;
+    int splits = (int)((304 + tiles - 1) / tiles);   // about two CTAs per SM
+    int maxs = g.K / 128;
+    if (splits > maxs) splits = maxs;
+    if (splits > 32) splits = 32;
+    const long long mn = (long long)g.M * g.N;
+    if (splits < 2 || splits * mn > g.sk_elems) return 0;
+    const int kchunk = ((g.K + splits - 1) / splits + GT_K - 1) / GT_K * GT_K;
+    splits = (g.K + kchunk - 1) / kchunk;
+    GemmArgs<T> p = g;
+    p.K = kchunk;
+    p.batch = splits;
+    p.sAb = kchunk * g.sAk;            // batch b = K range [b*kchunk, ...)
+    p.sBb = kchunk * g.sBk;
+    p.C = g.sk; p.sCm = g.N; p.sCn = 1; p.sCb = mn;
+    p.alpha = T(1); p.beta = T(0); p.colscale = nullptr; p.sk = nullptr;
+    // the last chunk may overrun K: handled by a separate launch with the remainder
+    const int last = g.K - (splits - 1) * kchunk;
+    if (last == kchunk) {
+        gemm_dispatch<T>(p, st);
+    } else {
+        p.batch = splits - 1;
+        gemm_dispatch<T>(p, st);
+        GemmArgs<T> r = p;
+        r.batch = 1; r.K = last;
+        r.A = g.A + (long long)(splits - 1) * kchunk * g.sAk;
+        r.B = g.B + (long long)(splits - 1) * kchunk * g.sBk;
+        r.C = g.sk + (long long)(splits - 1) * mn;
+        gemm_dispatch<T>(r, st);
+    }
+    return splits;
+}
+
 template <typename T>
 inline void gemm(const GemmArgs<T>& g, cudaStream_t st) {
     if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return;
     if (g.batch > 65535) fail(KH_EINVAL, "gemm batch > 65535");
     if constexpr (sizeof(T) == 8) {
         gemm_f64(g, st);
-        return;
     } else {
-    // few output tiles and a long K: split K over CTAs into the scratch,
-    // then reduce in a fixed order (deterministic)
-    const long long tiles = (long long)((g.M + 63) / 64) * ((g.N + 63) / 64);
-    if (g.batch == 1 && g.sk && tiles < 76 && g.K >= 256) {
-        int splits = (int)((304 + tiles - 1) / tiles);   // about two CTAs per SM
-        int maxs = g.K / 128;
-        if (splits > maxs) splits = maxs;
-        if (splits > 32) splits = 32;
-        const long long mn = (long long)g.M * g.N;
-        if (splits >= 2 && splits * mn <= g.sk_elems) {
-            const int kchunk = ((g.K + splits - 1) / splits + GT_K - 1) / GT_K * GT_K;
-            splits = (g.K + kchunk - 1) / kchunk;
-            GemmArgs<T> p = g;
-            p.K = kchunk;
-            p.batch = splits;
-            p.sAb = kchunk * g.sAk;            // batch b = K range [b*kchunk, ...)
-            p.sBb = kchunk * g.sBk;
-            p.C = g.sk; p.sCm = g.N; p.sCn = 1; p.sCb = mn;
-            p.alpha = T(1); p.beta = T(0); p.colscale = nullptr; p.sk = nullptr;
-            // the last chunk may overrun K: handled by a separate launch with the remainder
-            const int last = g.K - (splits - 1) * kchunk;
-            if (last == kchunk) {
-                gemm_dispatch<T>(p, st);
-            } else {
-                p.batch = splits - 1;
-                gemm_dispatch<T>(p, st);
-                GemmArgs<T> r = p;
-                r.batch = 1; r.K = last;
-                r.A = g.A + (long long)(splits - 1) * kchunk * g.sAk;
-                r.B = g.B + (long long)(splits - 1) * kchunk * g.sBk;
-                r.C = g.sk + (long long)(splits - 1) * mn;
-                gemm_dispatch<T>(r, st);
-            }
-            splitk_reduce_kernel<T><<<grid_for(mn), 256, 0, st>>>(g.sk, splits, g.M, g.N, g.C, g.sCm, g.sCn, g.alpha,
-                                                                  g.beta, g.colscale);
+        const int splits = gemm_parts<T>(g, st);     // joined in a fixed order (deterministic)
+        if (splits) {
+            splitk_reduce_kernel<T><<<grid_for((long long)g.M * g.N), 256, 0, st>>>(
+                g.sk, splits, g.M, g.N, g.C, g.sCm, g.sCn, g.alpha, g.beta, g.colscale);
             KH_LAUNCHED();
             return;
         }
+        gemm_dispatch<T>(g, st);
     }
-    gemm_dispatch<T>(g, st);
-    }
+}
+
+// Arguments of the plain row-major C(MxN) = A(MxK) B(KxN); transposes by flags.
+template <typename T>
+inline GemmArgs<T> rm_args(int M, int N, int K, const T* A, bool tA, const T* B, bool tB, T* C) {
+    GemmArgs<T> g;
+    g.M = M; g.N = N; g.K = K; g.batch = 1;
+    g.A = A; g.sAm = tA ? 1 : K; g.sAk = tA ? M : 1; g.sAb = 0;
+    g.B = B; g.sBk = tB ? 1 : N; g.sBn = tB ? K : 1; g.sBb = 0;
+    g.C = C; g.sCm = N; g.sCn = 1; g.sCb = 0;
+    g.alpha = T(1); g.beta = T(0); g.colscale = nullptr;
+    return g;
 }
 
 // Plain row-major C(MxN) = A(MxK) B(KxN) [+beta C]; transposes by flags.
@@ -556,13 +574,9 @@ template <typename T>
 inline void gemm_rm(int M, int N, int K, const T* A, bool tA, const T* B, bool tB, T* C,
                     cudaStream_t st, T alpha = T(1), T beta = T(0), const T* colscale = nullptr,
                     T* sk = nullptr, long long sk_elems = 0) {
-    GemmArgs<T> g;
+    GemmArgs<T> g = rm_args<T>(M, N, K, A, tA, B, tB, C);
     g.sk = sk;
     g.sk_elems = sk_elems;
-    g.M = M; g.N = N; g.K = K; g.batch = 1;
-    g.A = A; g.sAm = tA ? 1 : K; g.sAk = tA ? M : 1; g.sAb = 0;
-    g.B = B; g.sBk = tB ? 1 : N; g.sBn = tB ? K : 1; g.sBb = 0;
-    g.C = C; g.sCm = N; g.sCn = 1; g.sCb = 0;
     g.alpha = alpha; g.beta = beta; g.colscale = colscale;
     gemm(g, st);
 }

@@ -179,7 +179,7 @@ void Engine<T>::carve_lane(Carver& cv) {
     C1n = cv.take<T>(chi2);
     C4n = cv.take<T>(chi2);
     E4n = cv.take<T>(E1);
-    dscr = cv.take<double>(DscrOff::kFixed + kk * kk);
+    dscr = cv.take<double>(DscrOff::kFixed + 3 * kk * kk);
     mt1 = cv.take<T>(E1);
     mt2 = cv.take<T>(E1);
     mup = cv.take<T>(n2);
@@ -735,7 +735,8 @@ void Engine<T>::corner(Slot<T>& sl, int f, int which) {
 // orthogonality that the first loses to the conditioning of Y (by a single
 // Newton-Schulz step when that loss is already small).  Scratch: tmp (n x k), Xk (k x k), dG (k x k FP64).
 template <typename T>
-void cholqr2(const T* Y, int n, int k, double cut, T* tmp, T* Xk, double* dG, T* Uo, cudaStream_t st) {
+void cholqr2(T* Y, int n, int k, double cut, T* tmp, T* Xk, double* dG, T* Uo, cudaStream_t st, const T* part,
+             int parts, bool dG_clear) {
     const double tau = sizeof(T) == 8 ? 1e-12 : 1e-5;
     // FP64: pivots below k 2^-53 / tau, whose acceptance could lift the
     // rounding noise of a later, exactly dependent column above tau, are
@@ -744,17 +745,32 @@ void cholqr2(const T* Y, int n, int k, double cut, T* tmp, T* Xk, double* dG, T*
     // bound (k 2^-24 / 1e-5, about 0.5) would reorder most columns of an early,
     // poorly converged iteration.
     const double defer = sizeof(T) == 8 ? k * 0x1p-53 / tau : 0.0;
+    // the second pass sees nearly orthonormal columns: a Newton-Schulz step
+    // (3I - G)/2 suffices when G is within 1e-4 (FP32) / 1e-8 (FP64) of I
+    const double ns_tol = sizeof(T) == 8 ? 1e-8 : 1e-4;
+    if constexpr (sizeof(T) == 4) {
+        if (rows_usable(n, k)) {           // one launch per pass over the block (rows.cu)
+            if (!dG_clear) KH_CUDA(cudaMemsetAsync(dG, 0, sizeof(double) * k * k, st));
+            if (parts) rows_reduce(part, parts, n, k, Y, dG, st);
+            else rows_reduce(Y, 1, n, k, nullptr, dG, st);
+            cholqr_factor<T>(dG, k, cut, tau, Xk, st, true, 0.0, defer, true);
+            rows_apply(Y, Xk, n, k, tmp, dG, st);
+            cholqr_factor<T>(dG, k, 1e-3, tau, Xk, st, false, ns_tol, 0.0, true);
+            rows_apply(tmp, Xk, n, k, Uo, nullptr, st);
+            return;
+        }
+    }
     gram<T>(Y, n, k, dG, st);
     cholqr_factor<T>(dG, k, cut, tau, Xk, st, true, 0.0, defer);
     gemm_rm<T>(n, k, k, Y, false, Xk, false, tmp, st);
     gram<T>(tmp, n, k, dG, st);
-    // the second pass sees nearly orthonormal columns: a Newton-Schulz step
-    // (3I - G)/2 suffices when G is within 1e-4 (FP32) / 1e-8 (FP64) of I
-    cholqr_factor<T>(dG, k, 1e-3, tau, Xk, st, false, sizeof(T) == 8 ? 1e-8 : 1e-4);
+    cholqr_factor<T>(dG, k, 1e-3, tau, Xk, st, false, ns_tol);
     gemm_rm<T>(n, k, k, tmp, false, Xk, false, Uo, st);
 }
-template void cholqr2<float>(const float*, int, int, double, float*, float*, double*, float*, cudaStream_t);
-template void cholqr2<double>(const double*, int, int, double, double*, double*, double*, double*, cudaStream_t);
+template void cholqr2<float>(float*, int, int, double, float*, float*, double*, float*, cudaStream_t, const float*, int,
+                             bool);
+template void cholqr2<double>(double*, int, int, double, double*, double*, double*, double*, cudaStream_t,
+                              const double*, int, bool);
 
 // Algorithmic flops of one CholQR2 of an n x k block: two symmetric Gram
 // matrices (n k (k+1) each), one Cholesky factor and triangular inverse
@@ -766,9 +782,10 @@ static double cholqr2_flops(int n, int k) {
 }
 
 template <typename T>
-void Engine<T>::orth(const T* Y, int n, int k, T* Uo) {
+void Engine<T>::orth(T* Y, int n, int k, T* Uo, int parts) {
     prof_begin(8);
-    cholqr2<T>(Y, n, k, cfg.svd_cut, Qt, Xk, dscr + DscrOff::kGram, Uo, st);
+    // the Gram matrices are cleared at the start of a projector, and by every factor that reads one
+    cholqr2<T>(Y, n, k, cfg.svd_cut, Qt, Xk, dscr + DscrOff::kGram, Uo, st, skbuf, parts, true);
     prof_end(8, cholqr2_flops(n, k));
 }
 
@@ -877,12 +894,24 @@ void Engine<T>::rr_svd(const T* X, int k, T* L, T* Qm, double jtol, int nrel, co
             cast<T, double>(X, Hd, (long long)k * k, st);
             Xd = Hd;
         }
-        cast<T, double>(L, Ld, (long long)k * k, st);
-        cast<T, double>(Qm, Qd, (long long)k * k, st);
-        svd_refine_fp64(Xd, k, Ld, Qd, Sd, Lr, Qr, Rw, 1e-5, st);
-        cast<double, T>(Lr, L, (long long)k * k, st);
-        cast<double, T>(Qr, Qm, (long long)k * k, st);
+        svd_refine_fp64(Xd, k, Ld, Qd, Sd, Lr, Qr, Rw, 1e-5, st, (float*)L, (float*)Qm);
     }
+}
+
+// Y = M V (tr) or Mt V (n x k): the number of parts left in skbuf for the
+// caller to join when K was split and keep_parts is set, else 0.
+template <typename T>
+int Engine<T>::subspace_product(bool tr, const T* V, T* Y, bool keep_parts) {
+    const int n = dm.n, k = dm.kk;
+    GemmArgs<T> g = rm_args<T>(n, k, n, Mt, tr, V, false, Y);
+    g.sk = skbuf;
+    g.sk_elems = sk_elems;
+    if (keep_parts) {
+        const int parts = gemm_parts<T>(g, st);
+        if (parts) return parts;
+    }
+    gemm<T>(g, st);
+    return 0;
 }
 
 // Top-chi SVD of M = Mt^T, written into (Sk, V = Z1, U = Uf).
@@ -911,6 +940,9 @@ void Engine<T>::projector(Slot<T>& sl, int dir, int slot_id) {
     uint64_t stream = (uint64_t)slot_id * 4 + dir;
     T* Vw = sl.Vw + (long long)dir * n * k;
     int* live = sl.live + dir * k;
+    const bool rows = sizeof(T) == 4 && rows_usable(n, k);      // row-block kernels for the passes over n x k
+    double* dG = dscr + DscrOff::kGram;
+    if (!dm.full && rows) KH_CUDA(cudaMemsetAsync(dG, 0, sizeof(double) * 3 * k * k, st));
     if (dm.full) {
         if (!sl.warm[dir]) {
             identity_kernel<T><<<grid_for((long long)n * k), 256, 0, st>>>(Vw, n, k);
@@ -940,15 +972,24 @@ void Engine<T>::projector(Slot<T>& sl, int dir, int slot_id) {
             Vin = U;
             q = cfg.svd_iters_cold;
         } else {
-            warm_split_kernel<T><<<grid_for((long long)n * k), 256, 0, st>>>(
-                Vw, live, n, k, Vo, Z2, cfg.seed, stream * 1000003ULL + (rng_counter++));
-            KH_LAUNCHED();
-            for (int r = 0; r < 2; ++r) {                                       // R <- R - Vl (Vl^T R), twice
-                gemm_rm<T>(k, k, n, Vo, true, Z2, false, Xk, st, T(1), T(0), nullptr, skbuf, sk_elems);
-                gemm_rm<T>(n, k, k, Vo, false, Xk, false, Z2, st, T(-1), T(1));
+            const uint64_t draw = stream * 1000003ULL + (rng_counter++);
+            if constexpr (sizeof(T) == 4) {
+                if (rows) {
+                    rows_split(Vw, live, n, k, Vo, Z2, cfg.seed, draw, dG + k * k, st);
+                    rows_project(Vo, dG + k * k, n, k, Z2, dG + 2 * k * k, st);  // R <- R - Vl (Vl^T R), twice
+                    rows_project(Vo, dG + 2 * k * k, n, k, Z2, nullptr, st);     // then Vl + R
+                }
             }
-            add_kernel<T><<<grid_for((long long)n * k), 256, 0, st>>>(Vo, Z2, (long long)n * k);
-            KH_LAUNCHED();
+            if (!rows) {
+                warm_split_kernel<T><<<grid_for((long long)n * k), 256, 0, st>>>(Vw, live, n, k, Vo, Z2, cfg.seed, draw);
+                KH_LAUNCHED();
+                for (int r = 0; r < 2; ++r) {                                   // R <- R - Vl (Vl^T R), twice
+                    gemm_rm<T>(k, k, n, Vo, true, Z2, false, Xk, st, T(1), T(0), nullptr, skbuf, sk_elems);
+                    gemm_rm<T>(n, k, k, Vo, false, Xk, false, Z2, st, T(-1), T(1));
+                }
+                add_kernel<T><<<grid_for((long long)n * k), 256, 0, st>>>(Vo, Z2, (long long)n * k);
+                KH_LAUNCHED();
+            }
             // no orthonormalisation needed: only span(M V) matters, and with
             // the complement projected off the live span, M V keeps the
             // trusted (large) columns first for the ordered CholQR below
@@ -957,15 +998,19 @@ void Engine<T>::projector(Slot<T>& sl, int dir, int slot_id) {
         }
         for (int it = 0; it < q; ++it) {
             prof_begin(9);
-            if (!product3x(ln, Mt, n, true, Vin, 1, k, Z1, n, k, n, k))            // Y = M V
-                gemm_rm<T>(n, k, n, Mt, true, Vin, false, Z1, st, T(1), T(0), nullptr, skbuf, sk_elems);
+            // Y = M V, U = orth(Y): where K is split, the row-block path joins the
+            // parts in its first pass over Y
+            int parts = 0;
+            if (!product3x(ln, Mt, n, true, Vin, 1, k, Z1, n, k, n, k))
+                parts = subspace_product(true, Vin, Z1, rows);
             prof_end(9, 2.0 * n * (double)n * k);
-            orth(Z1, n, k, U);                                                 // U = orth(Y)
+            orth(Z1, n, k, U, parts);
             prof_begin(9);
-            if (!product3x(ln, Mt, n, false, U, 1, k, Z2, n, k, n, k))             // Z = M^T U
-                gemm_rm<T>(n, k, n, Mt, false, U, false, Z2, st, T(1), T(0), nullptr, skbuf, sk_elems);
+            parts = 0;
+            if (!product3x(ln, Mt, n, false, U, 1, k, Z2, n, k, n, k))          // Z = M^T U, V' = orth(Z)
+                parts = subspace_product(false, U, Z2, rows);
             prof_end(9, 2.0 * n * (double)n * k);
-            orth(Z2, n, k, Vo);                                                // V' = orth(Z)
+            orth(Z2, n, k, Vo, parts);
             Vin = Vo;
         }
         // G = H^T = Z^T V' with H = V'^T Z the Rayleigh-Ritz matrix (M ~ U G V'^T).
@@ -982,8 +1027,18 @@ void Engine<T>::projector(Slot<T>& sl, int dir, int slot_id) {
         prof_begin(7);
         rr_svd(Hk, k, Lk, Qk, jtol, chi + 8, proj64() ? Hd : nullptr);         // G Q = L S
         prof_end(7, 0.0);
-        gemm_rm<T>(n, k, k, Vo, false, Qk, false, Z1, st);                     // right vectors of M: V' Q
-        gemm_rm<T>(n, k, k, U, false, Lk, false, Uf, st);                      // left vectors of M: U L
+        // right and left vectors of M: V' Q, U L
+        bool applied = false;
+        if constexpr (sizeof(T) == 4) {
+            if (rows) {
+                rows_apply(Vo, Qk, n, k, Z1, nullptr, st, U, Lk, Uf);
+                applied = true;
+            }
+        }
+        if (!applied) {
+            gemm_rm<T>(n, k, k, Vo, false, Qk, false, Z1, st);
+            gemm_rm<T>(n, k, k, U, false, Lk, false, Uf, st);
+        }
         KH_CUDA(cudaMemcpyAsync(Vw, Z1, sizeof(T) * (size_t)n * k, cudaMemcpyDeviceToDevice, st));
         {
             const int thr = 256 / k > 0 ? 256 / k * k : k;
@@ -1435,8 +1490,8 @@ void svd_jacobi(const T* X, int k, T* sv, T* L, T* Qm, int max_sweeps, double to
 #undef KH_SVDJ
 }
 template <typename T>
-void cholqr_factor(const double* dG, int k, double cut_abs, double tau, T* X, cudaStream_t st, bool sorted,
-                   double ns_tol, double defer) {
+void cholqr_factor(double* dG, int k, double cut_abs, double tau, T* X, cudaStream_t st, bool sorted,
+                   double ns_tol, double defer, bool clear) {
     if (k > jacobi_kmax<T>()) fail(KH_EINVAL, "cholqr: k beyond limit");
     const size_t sm = (size_t)k * (k | 1) * sizeof(T);
     if constexpr (sizeof(T) == 4) {
@@ -1446,7 +1501,7 @@ void cholqr_factor(const double* dG, int k, double cut_abs, double tau, T* X, cu
     case KT: {                                                                                               \
         static std::atomic<size_t> granted[kMaxDevices] = {};                                                \
         smem_opt_in(cholqr_reg_kernel<T, KT>, sm, granted);                                                  \
-        cholqr_reg_kernel<T, KT><<<1, 512, sm, st>>>(dG, k, cut_abs, tau, X, sorted ? 1 : 0, ns_tol);        \
+        cholqr_reg_kernel<T, KT><<<1, 512, sm, st>>>(dG, k, cut_abs, tau, X, sorted ? 1 : 0, ns_tol, clear ? 1 : 0); \
         break;                                                                                               \
     }
             KH_CHOL(1) KH_CHOL(2) KH_CHOL(3) KH_CHOL(4) KH_CHOL(5)
@@ -1459,8 +1514,8 @@ void cholqr_factor(const double* dG, int k, double cut_abs, double tau, T* X, cu
     }
     KH_LAUNCHED();
 }
-template void cholqr_factor<float>(const double*, int, double, double, float*, cudaStream_t, bool, double, double);
-template void cholqr_factor<double>(const double*, int, double, double, double*, cudaStream_t, bool, double, double);
+template void cholqr_factor<float>(double*, int, double, double, float*, cudaStream_t, bool, double, double, bool);
+template void cholqr_factor<double>(double*, int, double, double, double*, cudaStream_t, bool, double, double, bool);
 
 template void svd_jacobi<float>(const float*, int, float*, float*, float*, int, double, double, cudaStream_t, int*,
                                 int);

@@ -145,8 +145,8 @@ struct DscrOff {
     static constexpr int kNormM2 = 8000;     // ||Mt||^2 of the half-system product
     static constexpr int kNorms = 8010;      // sums of squares of C1n, C4n, E4n
     static constexpr int kKappa = 8020;      // Z11, Z00, Z10, Z01 of the free energy
-    static constexpr int kGram = 8192;       // FP64 Gram matrix, kk^2
-    static constexpr int kFixed = kGram;     // doubles before the Gram matrix
+    static constexpr int kGram = 8192;       // FP64 Gram matrices: orthonormalisation, two of the projection (kk^2 each)
+    static constexpr int kFixed = kGram;     // doubles before the Gram matrices
 };
 static_assert(DscrOff::kStage + 16 * 16 * 16 <= DscrOff::kExpvalOut && DscrOff::kExpvalOut + 16 <= DscrOff::kObsOut &&
                   DscrOff::kObsOut + 10 <= DscrOff::kLiveAcc && DscrOff::kLiveAcc + 160 / 2 <= DscrOff::kLiveCount &&
@@ -257,7 +257,8 @@ struct Engine : EngineBase {
         return img == 1 ? sl.L1 + (kind * 4 + f) * dm.lay1 : sl.L2 + (kind * 4 + f) * dm.lay2;
     }
     void projector(Slot<T>& sl, int dir, int slot_id);
-    void orth(const T* Y, int n, int k, T* Uo);
+    void orth(T* Y, int n, int k, T* Uo, int parts = 0);
+    int subspace_product(bool tr, const T* V, T* Y, bool keep_parts);
     void rr_svd(const T* X, int k, T* L, T* Qm, double jtol, int nrel, const double* Xd = nullptr);
     void absorb(Slot<T>& sl, int s);
     void move(Slot<T>& sl, int s, int slot_id);
@@ -317,6 +318,20 @@ struct TcOperand {
 void tc_gemm(const TcOperand& A, const TcOperand& B, float* C, int M, int N, int K, long long ldc, float alpha,
              float beta, const float* colscale, int* err, cudaStream_t st);
 
+// Row-block kernels of small FP32 bases (rows.cu): n x k blocks, k <= 96; a
+// non-null G (k x k, FP64) has the named Gram matrix added to it.
+inline bool rows_usable(int n, int k) { return k <= 96 && n <= 2048; }
+// Y = sum of the K split's parts (G: Y^T Y); Y null: the sum is not stored
+void rows_reduce(const float* part, int splits, int n, int k, float* Y, double* G, cudaStream_t st);
+// Q = Y X (G: Q^T Q), and a second such product when Q2 is given (G null)
+void rows_apply(const float* Y, const float* X, int n, int k, float* Q, double* G, cudaStream_t st,
+                const float* Y2 = nullptr, const float* X2 = nullptr, float* Q2 = nullptr);
+// warm basis into live columns Vl and random R in the dead ones (G: Vl^T R)
+void rows_split(const float* Vw, const int* live, int n, int k, float* Vl, float* R, uint64_t seed, uint64_t stream,
+                double* G, cudaStream_t st);
+// R -= Vl C (G: Vl^T R); G null: R = Vl + (R - Vl C)
+void rows_project(const float* Vl, const double* C, int n, int k, float* R, double* G, cudaStream_t st);
+
 // FP64 one-sided Jacobi SVD on a cluster of eight CTAs (svd_cluster.cu), k <= 112
 void svd_jacobi_cluster(const double* X, int k, double* s, double* L, double* Q, int max_sweeps, double tol,
                         double cut, cudaStream_t st, int* sweep_count, int nrel);
@@ -336,8 +351,11 @@ void gemm3x(const float* A, long long lda, bool a_mmajor, const float* Bhi, cons
 
 // Orthonormal basis of the columns of Y (n x k, k <= the Jacobi limit) by the
 // ordered CholQR2 (ctm.cu); see Engine::orth.
+// (parts > 0: Y itself is first formed as the sum of that many n x k blocks at
+// `part`; dG_clear: dG holds zeros already, and again afterwards)
 template <typename T>
-void cholqr2(const T* Y, int n, int k, double cut, T* tmp, T* Xk, double* dG, T* Uo, cudaStream_t st);
+void cholqr2(T* Y, int n, int k, double cut, T* tmp, T* Xk, double* dG, T* Uo, cudaStream_t st,
+             const T* part = nullptr, int parts = 0, bool dG_clear = false);
 // G = A^T B (n x k each, T) accumulated in FP64 across row chunks (ctm.cu)
 template <typename T>
 void gram2(const T* A, const T* B, int n, int k, double* dG, cudaStream_t st);
@@ -345,8 +363,8 @@ void gram2(const T* A, const T* B, int n, int k, double* dG, cudaStream_t st);
 // Three FP64 Newton steps on a single-precision SVD G Q ~ L diag(s) of a k x k
 // FP64 matrix G (refine.cu): refined factors to Lo, Qo, singular values to s.
 size_t svd_refine_scratch(int k);
-void svd_refine_fp64(const double* G, int k, const double* L, const double* Q, double* s, double* Lo, double* Qo,
-                     double* work, double rel_gap, cudaStream_t st);
+void svd_refine_fp64(const double* G, int k, double* L, double* Q, double* s, double* Lo, double* Qo, double* work,
+                     double rel_gap, cudaStream_t st, float* Lf = nullptr, float* Qf = nullptr);
 
 // Frame layouts of a site tensor Tm[p][D^4] for the two-layer site
 // contraction (bond.cu): Tcor, Tedg 4 frames x pmax D^4 each.

@@ -484,9 +484,10 @@ svd_jacobi_kernel(const T* __restrict__ Xin, int k, T* __restrict__ s_out, T* __
 // outside span(Y); a column nearly parallel to the ones before it is therefore
 // taken after the well-conditioned ones, by which time its residual has
 // usually become exactly zero (a rank-revealing order, as in column pivoting).
+// clear: dG is set to zero once read (FP32 only).
 template <typename T>
-void cholqr_factor(const double* dG, int k, double cut_abs, double tau, T* X, cudaStream_t st, bool sorted = true,
-                   double ns_tol = 0.0, double defer = 0.0);
+void cholqr_factor(double* dG, int k, double cut_abs, double tau, T* X, cudaStream_t st, bool sorted = true,
+                   double ns_tol = 0.0, double defer = 0.0, bool clear = false);
 
 #ifdef KH_JACOBI_KERNEL
 __device__ __forceinline__ float chol_recip(float x) { return __fdividef(1.f, x); }
@@ -783,8 +784,8 @@ struct alignas(4 * sizeof(T)) Quad {
 };
 template <typename T, int KT>
 __global__ void __launch_bounds__(512, 1)
-cholqr_reg_kernel(const double* __restrict__ G, int k, double cut_abs, double tau, T* __restrict__ X, int sorted,
-                  double ns_tol) {
+cholqr_reg_kernel(double* __restrict__ G, int k, double cut_abs, double tau, T* __restrict__ X, int sorted,
+                  double ns_tol, int clear) {
     extern __shared__ unsigned char smem_raw[];
     T* Xs = reinterpret_cast<T*>(smem_raw);        // k x (k | 1): the result, transposed for coalesced rows
     constexpr int KR = 2 * KT, KM = 32 * KT;       // rows (16 apart) and KT columns (32 apart) of a thread
@@ -827,6 +828,8 @@ cholqr_reg_kernel(const double* __restrict__ G, int k, double cut_abs, double ta
             }
         dev = block_max(dev);
         if (dev < (T)ns_tol) {
+            if (clear)
+                for (int e = tid; e < k * k; e += 512) G[e] = 0.0;
 #pragma unroll
             for (int a = 0; a < KR; ++a)
 #pragma unroll
@@ -943,6 +946,8 @@ cholqr_reg_kernel(const double* __restrict__ G, int k, double cut_abs, double ta
         }
     }
     __syncthreads();
+    if (clear)
+        for (int e = tid; e < k * k; e += 512) G[e] = 0.0;
     // X[perm c][i] = inv[perm c] L^-1[i][c], L^-1 = D^-1/2 times the unit inverse
     // (Q = Y_s L^-T; dropped i give zero columns)
     const int ld = k | 1;

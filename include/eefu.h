@@ -396,6 +396,13 @@ kh_status kh_selftest_gemm(int prec, int M, int N, int K, const double* dev_A, c
 kh_status kh_selftest_gemm3x(int a_colmajor, int M, int N, int K, const double* dev_A, const double* dev_B,
                              double* dev_C, void* dev_scratch, size_t scratch_bytes, void* stream);
 
+/* Axis permutation of a row-major FP64 device array: output axis j is input axis
+ * order[j] (rank <= 8, host arrays).  kind 0 in FP64, 1 in FP32, 2 as the pair
+ * of TF32 head and FP32 remainder, whose sum is returned.  Scratch of 16 bytes
+ * an element and 1024 more.  Synchronises stream. */
+kh_status kh_selftest_permute(int kind, int rank, const long long* shape, const int* order, const double* dev_in,
+                              double* dev_out, void* dev_scratch, size_t scratch_bytes, void* stream);
+
 /* Eigen-decomposition of a symmetric k x k FP64 matrix by the library's
  * Jacobi kernel in FP64 (prec = KH_FP64) or FP32 (otherwise): dev_evals
  * descending, column j of dev_W its eigenvector.  Scratch as above with

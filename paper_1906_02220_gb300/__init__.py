@@ -26,7 +26,7 @@ ABI_FUNCTIONS = [
     "kh_set_state", "kh_get_state", "ctm_set_tensor", "ctm_build_composite", "ctm_init",
     "ctm_copy_env", "ctm_sweep", "ctm_projectors", "ctm_get_env", "ctm_metric", "ctm_kappa",
     "ctm_expval", "ctm_correlation_length", "ctm_plaquette", "ctm_flux", "eefu_apply_gate", "eefu_cost_gradient", "observables", "kh_version", "kh_bond_hamiltonian", "kh_gate", "kh_flux_operators",
-    "eefu_trotter_step", "eefu_evolve", "eefu_evolve_flux", "eefu_evolve_batch", "kh_launch_count", "kh_profile", "kh_selftest_bytes", "kh_selftest_gemm", "kh_selftest_gemm3x",
+    "eefu_trotter_step", "eefu_evolve", "eefu_evolve_flux", "eefu_evolve_batch", "kh_launch_count", "kh_profile", "kh_selftest_bytes", "kh_selftest_gemm", "kh_selftest_gemm3x", "kh_selftest_permute",
     "kh_selftest_symeig", "kh_selftest_svd", "kh_selftest_svd_refined", "kh_selftest_orth", "kh_selftest_fp64_newton",
     "kh_selftest_site_layered_bytes", "kh_selftest_site_layered", "kh_gemm_noalloc",
     "kh_gemm_noalloc_max_bytes", "kh_save", "kh_load_config", "kh_load",
@@ -94,6 +94,7 @@ def load_library(path=LIB_PATH):
         "kh_selftest_bytes": (S, [I, I, I]),
         "kh_selftest_gemm": (I, [I, I, I, I, P, P, P, P, S, P]),
         "kh_selftest_gemm3x": (I, [I, I, I, I, P, P, P, P, S, P]),
+        "kh_selftest_permute": (I, [I, I, ctypes.POINTER(ctypes.c_longlong), ctypes.POINTER(I), P, P, P, S, P]),
         "kh_selftest_symeig": (I, [I, I, P, P, P, P, S, P]),
         "kh_selftest_svd": (I, [I, I, P, P, P, P, P, S, P]),
         "kh_selftest_orth": (I, [I, I, I, D, P, P, P, S, P]),
@@ -156,6 +157,23 @@ def selftest_gemm3x(A, B, a_colmajor=False):
     if st != KH_OK:
         raise KhError(st, "kh_selftest_gemm3x")
     return C
+
+
+def selftest_permute(x, order, kind=0):
+    """x.permute(order) of an FP64 CUDA tensor through the library's permutation
+    kernels: kind 0 in FP64, 1 in FP32, 2 as the sum of its TF32 head and remainder."""
+    import torch
+    out = torch.empty([x.shape[i] for i in order], dtype=torch.float64, device=x.device)
+    nb = 16 * x.numel() + 1024
+    scr = torch.empty(nb + 256, dtype=torch.uint8, device=x.device)
+    base = (scr.data_ptr() + 255) // 256 * 256
+    st = lib().kh_selftest_permute(kind, x.dim(), (ctypes.c_longlong * x.dim())(*x.shape),
+                                   (ctypes.c_int * x.dim())(*order), _tptr(x.contiguous()), _tptr(out),
+                                   ctypes.c_void_p(base), nb,
+                                   ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    if st != KH_OK:
+        raise KhError(st, "kh_selftest_permute")
+    return out
 
 
 def selftest_symeig(G, prec="fp64"):

@@ -21,6 +21,11 @@ void run_gemm(int M, int N, int K, const double* A, const double* B, double* C, 
     kh::cast<T, double>(c, C, (long long)M * N, st);
 }
 
+__global__ void add_kernel(const float* a, float* b, long long n) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        b[i] += a[i];
+}
+
 void check_wait(const int* err, cudaStream_t st) {
     int h = 0;
     KH_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -231,6 +236,44 @@ kh_status kh_selftest_gemm3x(int a_colmajor, int M, int N, int K, const double* 
     if (bytes < kh_selftest_bytes(M, N, K)) return KH_ENOMEM;
     cudaStream_t st = (cudaStream_t)stream;
     return run([&] { run_gemm3x(a_colmajor != 0, M, N, K, A, B, C, scratch, bytes, st); });
+}
+
+kh_status kh_selftest_permute(int kind, int rank, const long long* shape, const int* order, const double* in,
+                              double* out, void* scratch, size_t bytes, void* stream) {
+    if (kind < 0 || kind > 2 || rank < 1 || rank > 8 || !shape || !order || !in || !out || !scratch) return KH_EINVAL;
+    long long total = 1;
+    int seen = 0;
+    for (int j = 0; j < rank; ++j) {
+        if (shape[j] < 1 || shape[j] > (1LL << 28) || order[j] < 0 || order[j] >= rank) return KH_EINVAL;
+        total *= shape[j];
+        seen |= 1 << order[j];
+        if (total > (1LL << 28)) return KH_EINVAL;
+    }
+    if (seen != (1 << rank) - 1) return KH_EINVAL;
+    if (bytes < 16 * (size_t)total + 1024) return KH_ENOMEM;
+    cudaStream_t st = (cudaStream_t)stream;
+    return run([&] {
+        const std::vector<long long> sh(shape, shape + rank);
+        const std::vector<int> od(order, order + rank);
+        kh::Carver cv(scratch, bytes);
+        float* a = cv.take<float>((size_t)total);
+        float* b = cv.take<float>((size_t)total);
+        float* c = cv.take<float>((size_t)total);
+        if (kind == 0) {
+            kh::permute<double, double>(in, out, sh, od, st);
+        } else {
+            kh::cast<double, float>(in, a, total, st);
+            if (kind == 1) {
+                kh::permute<float, float>(a, b, sh, od, st);
+            } else {
+                kh::permute_split(a, b, c, sh, od, st);
+                add_kernel<<<kh::grid_for(total), 256, 0, st>>>(c, b, total);
+                KH_LAUNCHED();
+            }
+            kh::cast<float, double>(b, out, total, st);
+        }
+        KH_CUDA(cudaStreamSynchronize(st));
+    });
 }
 
 kh_status kh_selftest_symeig(int prec, int k, const double* G, double* W, double* E, void* scratch, size_t bytes,

@@ -15,6 +15,7 @@
 //   C1 <- P^T (C1 E1), C4 <- (C4 E3) P~^T, E4 <- P^T (E4 T T) P~^T,
 //   each divided by its Frobenius norm (FP64).
 #include <algorithm>
+#include <functional>
 
 #define KH_JACOBI_KERNEL
 #include "engine.cuh"
@@ -679,8 +680,8 @@ void Engine<T>::site_layer(const T* Ybuf, long long nb, const T* TL, const T* L1
 // The tensor-core FP32 products need 16-byte rows of A (n a multiple of 4 in
 // every use) and enough work.  At n = 1024, k = 80 (1.7e8 flops: split of B 5 us,
 // product 10, reduction 4) they equal the SIMT tiles with split K (12 + 4); at
-// 2500 x 128 x 2500 (1.6e9) they take 28 us against 120.  kMin3x lies between.
-constexpr double kMin3x = 3e8;
+// 5184 x 160 x 160 (2.7e8) they take 5 + 10 us against 26.  kMin3x lies between.
+constexpr double kMin3x = 2e8;
 template <typename T>
 bool Engine<T>::product3x(int ln, const T* A, long long lda, bool a_mmajor, const T* B, long long sn, long long sk,
                           T* C, int M, int N, int K, long long ldc, const T* colscale) {
@@ -703,7 +704,8 @@ void Engine<T>::corner(Slot<T>& sl, int f, int which) {
     const T* E1p = Eop + f * E1;
     const T* E4 = Eop + ((f + 3) & 3) * E1;
     T* X = X1[which];
-    gemm_rm<T>(chi, d2 * chi, chi, C1, false, E1p, false, X, st);            // [x4][(uk,ub,z)]
+    if (!product3x(lane_id(), C1, chi, false, E1p, 1, (long long)d2 * chi, X, chi, d2 * chi, chi, (long long)d2 * chi))
+        gemm_rm<T>(chi, d2 * chi, chi, C1, false, E1p, false, X, st);        // [x4][(uk,ub,z)]
     // Y = E4 X as [(w,lk,lb)][(uk,ub,z)], or on the tensor cores its transpose
     // (X^T E4^T: X's rows of n values suit the tensor maps at any chi); then
     // [w][z][lb][ub][lk][uk]
@@ -736,7 +738,7 @@ void Engine<T>::corner(Slot<T>& sl, int f, int which) {
 // Newton-Schulz step when that loss is already small).  Scratch: tmp (n x k), Xk (k x k), dG (k x k FP64).
 template <typename T>
 void cholqr2(T* Y, int n, int k, double cut, T* tmp, T* Xk, double* dG, T* Uo, cudaStream_t st, const T* part,
-             int parts, bool dG_clear) {
+             int parts, bool dG_clear, const std::function<bool(const T*, const T*, T*)>& product) {
     const double tau = sizeof(T) == 8 ? 1e-12 : 1e-5;
     // FP64: pivots below k 2^-53 / tau, whose acceptance could lift the
     // rounding noise of a later, exactly dependent column above tau, are
@@ -760,17 +762,21 @@ void cholqr2(T* Y, int n, int k, double cut, T* tmp, T* Xk, double* dG, T* Uo, c
             return;
         }
     }
+    auto apply = [&](const T* A, T* Q) {
+        if (!product || !product(A, Xk, Q)) gemm_rm<T>(n, k, k, A, false, Xk, false, Q, st);
+    };
     gram<T>(Y, n, k, dG, st);
     cholqr_factor<T>(dG, k, cut, tau, Xk, st, true, 0.0, defer);
-    gemm_rm<T>(n, k, k, Y, false, Xk, false, tmp, st);
+    apply(Y, tmp);
     gram<T>(tmp, n, k, dG, st);
     cholqr_factor<T>(dG, k, 1e-3, tau, Xk, st, false, ns_tol);
-    gemm_rm<T>(n, k, k, tmp, false, Xk, false, Uo, st);
+    apply(tmp, Uo);
 }
 template void cholqr2<float>(float*, int, int, double, float*, float*, double*, float*, cudaStream_t, const float*, int,
-                             bool);
+                             bool, const std::function<bool(const float*, const float*, float*)>&);
 template void cholqr2<double>(double*, int, int, double, double*, double*, double*, double*, cudaStream_t,
-                              const double*, int, bool);
+                              const double*, int, bool,
+                              const std::function<bool(const double*, const double*, double*)>&);
 
 // Algorithmic flops of one CholQR2 of an n x k block: two symmetric Gram
 // matrices (n k (k+1) each), one Cholesky factor and triangular inverse
@@ -785,7 +791,9 @@ template <typename T>
 void Engine<T>::orth(T* Y, int n, int k, T* Uo, int parts) {
     prof_begin(8);
     // the Gram matrices are cleared at the start of a projector, and by every factor that reads one
-    cholqr2<T>(Y, n, k, cfg.svd_cut, Qt, Xk, dscr + DscrOff::kGram, Uo, st, skbuf, parts, true);
+    const int ln = lane_id();
+    cholqr2<T>(Y, n, k, cfg.svd_cut, Qt, Xk, dscr + DscrOff::kGram, Uo, st, skbuf, parts, true,
+               [&](const T* A, const T* X, T* Q) { return product3x(ln, A, k, false, X, 1, k, Q, n, k, k, k); });
     prof_end(8, cholqr2_flops(n, k));
 }
 
@@ -985,7 +993,12 @@ void Engine<T>::projector(Slot<T>& sl, int dir, int slot_id) {
                 KH_LAUNCHED();
                 for (int r = 0; r < 2; ++r) {                                   // R <- R - Vl (Vl^T R), twice
                     gemm_rm<T>(k, k, n, Vo, true, Z2, false, Xk, st, T(1), T(0), nullptr, skbuf, sk_elems);
-                    gemm_rm<T>(n, k, k, Vo, false, Xk, false, Z2, st, T(-1), T(1));
+                    if (product3x(ln, Vo, k, false, Xk, 1, k, Z1, n, k, k, k)) {
+                        axpby_kernel<T><<<grid_for((long long)n * k), 256, 0, st>>>(Z1, Z2, (long long)n * k, T(-1));
+                        KH_LAUNCHED();
+                    } else {
+                        gemm_rm<T>(n, k, k, Vo, false, Xk, false, Z2, st, T(-1), T(1));
+                    }
                 }
                 add_kernel<T><<<grid_for((long long)n * k), 256, 0, st>>>(Vo, Z2, (long long)n * k);
                 KH_LAUNCHED();
@@ -1036,8 +1049,10 @@ void Engine<T>::projector(Slot<T>& sl, int dir, int slot_id) {
             }
         }
         if (!applied) {
-            gemm_rm<T>(n, k, k, Vo, false, Qk, false, Z1, st);
-            gemm_rm<T>(n, k, k, U, false, Lk, false, Uf, st);
+            if (!product3x(ln, Vo, k, false, Qk, 1, k, Z1, n, k, k, k))
+                gemm_rm<T>(n, k, k, Vo, false, Qk, false, Z1, st);
+            if (!product3x(ln, U, k, false, Lk, 1, k, Uf, n, k, k, k))
+                gemm_rm<T>(n, k, k, U, false, Lk, false, Uf, st);
         }
         KH_CUDA(cudaMemcpyAsync(Vw, Z1, sizeof(T) * (size_t)n * k, cudaMemcpyDeviceToDevice, st));
         {

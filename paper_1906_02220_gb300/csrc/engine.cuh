@@ -1,6 +1,8 @@
 // eeFU engine: context layout and the declarations shared by the CTMRG
 // (ctm.cu), bond-update (bond.cu) and C-ABI (abi.cu) translation units.
 #pragma once
+#include <functional>
+
 #include "common.cuh"
 #include "jacobi.cuh"
 
@@ -352,10 +354,12 @@ void gemm3x(const float* A, long long lda, bool a_mmajor, const float* Bhi, cons
 // Orthonormal basis of the columns of Y (n x k, k <= the Jacobi limit) by the
 // ordered CholQR2 (ctm.cu); see Engine::orth.
 // (parts > 0: Y itself is first formed as the sum of that many n x k blocks at
-// `part`; dG_clear: dG holds zeros already, and again afterwards)
+// `part`; dG_clear: dG holds zeros already, and again afterwards; product: Q = Y X
+// by another route, false where that does not apply)
 template <typename T>
 void cholqr2(T* Y, int n, int k, double cut, T* tmp, T* Xk, double* dG, T* Uo, cudaStream_t st,
-             const T* part = nullptr, int parts = 0, bool dG_clear = false);
+             const T* part = nullptr, int parts = 0, bool dG_clear = false,
+             const std::function<bool(const T* Y, const T* X, T* Q)>& product = nullptr);
 // G = A^T B (n x k each, T) accumulated in FP64 across row chunks (ctm.cu)
 template <typename T>
 void gram2(const T* A, const T* B, int n, int k, double* dG, cudaStream_t st);

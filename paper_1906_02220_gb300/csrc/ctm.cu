@@ -312,6 +312,7 @@ __global__ void rand_kernel(T* V, long long tot, uint64_t seed, uint64_t stream)
 template <typename T, int KT, bool SYM>
 __global__ void __launch_bounds__(256) gram_kernel(const T* __restrict__ Z, const T* __restrict__ Z2, int n, int k,
                                                    int nt, double* __restrict__ G, int rows_cta) {
+    pdl_start();
     constexpr int TS = 16 * KT, CH = 16;
     __shared__ T As[CH][TS], Bs[CH][TS];
     const int y = blockIdx.y;
@@ -401,13 +402,12 @@ void gram(const T* Z, int n, int k, double* dG, cudaStream_t st, const T* Z2 = n
     switch (kt) {
 #define KH_GRAM(KT)                                                                                            \
     case KT:                                                                                                   \
-        if (Z2) gram_kernel<T, KT, false><<<grid, 256, 0, st>>>(Z, Z2, n, k, nt, dG, rows);                    \
-        else gram_kernel<T, KT, true><<<grid, 256, 0, st>>>(Z, Z, n, k, nt, dG, rows);                         \
+        if (Z2) launch(gram_kernel<T, KT, false>, grid, 256, 0, st, Z, Z2, n, k, nt, dG, rows);                    \
+        else launch(gram_kernel<T, KT, true>, grid, 256, 0, st, Z, Z, n, k, nt, dG, rows);                         \
         break;
         KH_GRAM(1) KH_GRAM(2) KH_GRAM(3) KH_GRAM(4) KH_GRAM(5)
 #undef KH_GRAM
     }
-    KH_LAUNCHED();
 }
 
 template <typename T>
@@ -428,6 +428,7 @@ __device__ __forceinline__ double nan_max(double a, double b) { return (b > a ||
 template <typename TS, typename T>
 __global__ void finalize_spectrum_kernel(const TS* sv, int k, int chi, double cut, const double* normM2,
                                          double* spec, T* isq, double* trunc) {
+    pdl_start();
     __shared__ double red[32];
     const int nkeep = min(chi, k);
     const double s0 = fmax((double)sv[0], 0.0);
@@ -454,6 +455,7 @@ __global__ void finalize_spectrum_kernel(const TS* sv, int k, int chi, double cu
 
 template <typename T>
 __global__ void store_normalized_kernel(const T* x, long long n, const double* sumsq, double* master, T* op) {
+    pdl_start();
     double s = *sumsq;
     double inv = s > 0.0 ? 1.0 / sqrt(s) : 1.0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -466,6 +468,7 @@ __global__ void store_normalized_kernel(const T* x, long long n, const double* s
 }
 
 __global__ void delta_kernel(const double* spec, double* prev, int chi, int prev_valid, double* delta) {
+    pdl_start();
     // one block: direction-wise normalised spectra, max |change| against the
     // previous sweep; warp q < 4 normalises direction q
     __shared__ double inv[4];
@@ -824,6 +827,7 @@ void Engine<T>::half_system_product(int n) {
 template <typename T>
 __global__ void warm_split_kernel(const T* Vw, const int* live, int n, int k, T* Vl, T* Rr, uint64_t seed,
                                   uint64_t stream) {
+    pdl_start();
     long long tot = (long long)n * k;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < tot;
          i += (long long)gridDim.x * blockDim.x) {
@@ -843,6 +847,7 @@ __global__ void warm_split_kernel(const T* Vw, const int* live, int n, int k, T*
 // live[] and clears acc and the block counter for the next call.
 template <typename T>
 __global__ void live_mask_kernel(const T* __restrict__ V, int n, int k, int* live, float* acc, int* counter) {
+    pdl_start();
     extern __shared__ float s_part[];                 // parts x k
     __shared__ int s_last;
     const int parts = blockDim.x / k;
@@ -879,12 +884,14 @@ __global__ void live_mask_kernel(const T* __restrict__ V, int n, int k, int* liv
 // b <- a * alpha + b
 template <typename T>
 __global__ void axpby_kernel(const T* a, T* b, long long n, T alpha) {
+    pdl_start();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         b[i] += alpha * a[i];
 }
 
 template <typename T>
 __global__ void add_kernel(const T* a, T* b, long long n) {
+    pdl_start();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         b[i] += a[i];
 }
@@ -943,8 +950,7 @@ void Engine<T>::projector(Slot<T>& sl, int dir, int slot_id) {
     half_system_product(n);
     double* normM2 = dscr + DscrOff::kNormM2;
     KH_CUDA(cudaMemsetAsync(normM2, 0, sizeof(double), st));
-    sumsq_kernel<T><<<sumsq_grid((long long)n * n), 256, 0, st>>>(Mt, (long long)n * n, normM2);
-    KH_LAUNCHED();
+    launch(sumsq_kernel<T>, sumsq_grid((long long)n * n), 256, 0, st, Mt, (long long)n * n, normM2);
     uint64_t stream = (uint64_t)slot_id * 4 + dir;
     T* Vw = sl.Vw + (long long)dir * n * k;
     int* live = sl.live + dir * k;
@@ -964,8 +970,7 @@ void Engine<T>::projector(Slot<T>& sl, int dir, int slot_id) {
         gemm_rm<T>(n, n, n, Z1, true, Z1, false, Y1, st);                      // V^T V
         gemm_rm<T>(n, n, n, Z1, false, Y1, false, Z2, st, T(-0.5), T(0));      // Newton-Schulz:
         // V <- 1.5 V - V (V^T V)/2
-        axpby_kernel<T><<<grid_for((long long)n * n), 256, 0, st>>>(Z1, Z2, (long long)n * n, T(1.5));
-        KH_LAUNCHED();
+        launch(axpby_kernel<T>, grid_for((long long)n * n), 256, 0, st, Z1, Z2, (long long)n * n, T(1.5));
         KH_CUDA(cudaMemcpyAsync(Vw, Z2, sizeof(T) * (size_t)n * n, cudaMemcpyDeviceToDevice, st));
         KH_CUDA(cudaMemcpyAsync(Z1, Z2, sizeof(T) * (size_t)n * n, cudaMemcpyDeviceToDevice, st));
         sl.warm[dir] = true;
@@ -989,19 +994,16 @@ void Engine<T>::projector(Slot<T>& sl, int dir, int slot_id) {
                 }
             }
             if (!rows) {
-                warm_split_kernel<T><<<grid_for((long long)n * k), 256, 0, st>>>(Vw, live, n, k, Vo, Z2, cfg.seed, draw);
-                KH_LAUNCHED();
+                launch(warm_split_kernel<T>, grid_for((long long)n * k), 256, 0, st, Vw, live, n, k, Vo, Z2, cfg.seed, draw);
                 for (int r = 0; r < 2; ++r) {                                   // R <- R - Vl (Vl^T R), twice
                     gemm_rm<T>(k, k, n, Vo, true, Z2, false, Xk, st, T(1), T(0), nullptr, skbuf, sk_elems);
                     if (product3x(ln, Vo, k, false, Xk, 1, k, Z1, n, k, k, k)) {
-                        axpby_kernel<T><<<grid_for((long long)n * k), 256, 0, st>>>(Z1, Z2, (long long)n * k, T(-1));
-                        KH_LAUNCHED();
+                        launch(axpby_kernel<T>, grid_for((long long)n * k), 256, 0, st, Z1, Z2, (long long)n * k, T(-1));
                     } else {
                         gemm_rm<T>(n, k, k, Vo, false, Xk, false, Z2, st, T(-1), T(1));
                     }
                 }
-                add_kernel<T><<<grid_for((long long)n * k), 256, 0, st>>>(Vo, Z2, (long long)n * k);
-                KH_LAUNCHED();
+                launch(add_kernel<T>, grid_for((long long)n * k), 256, 0, st, Vo, Z2, (long long)n * k);
             }
             // no orthonormalisation needed: only span(M V) matters, and with
             // the complement projected off the live span, M V keeps the
@@ -1059,19 +1061,17 @@ void Engine<T>::projector(Slot<T>& sl, int dir, int slot_id) {
             const int thr = 256 / k > 0 ? 256 / k * k : k;
             // a CTA per 64 rows or so: 16 CTAs took 148 us at n = 5184, k = 160
             const int blocks = std::min(152, std::max(16, n / 64));
-            live_mask_kernel<T><<<blocks, thr, sizeof(float) * thr, st>>>(
-                Z1, n, k, live, (float*)(dscr + DscrOff::kLiveAcc), (int*)(dscr + DscrOff::kLiveCount));
+            launch(live_mask_kernel<T>, blocks, thr, sizeof(float) * thr, st, Z1, n,
+                   k, live, (float*)(dscr + DscrOff::kLiveAcc), (int*)(dscr + DscrOff::kLiveCount));
         }
-        KH_LAUNCHED();
         sl.warm[dir] = true;
     }
     if (proj64())
-        finalize_spectrum_kernel<double, T><<<1, 128, 0, st>>>(Sd, k, chi, cut, normM2, sl.spec + (long long)dir * chi,
+        launch(finalize_spectrum_kernel<double, T>, 1, 128, 0, st, Sd, k, chi, cut, normM2, sl.spec + (long long)dir * chi,
                                                                isq, sl.trunc + dir);
     else
-        finalize_spectrum_kernel<T, T><<<1, 128, 0, st>>>(Sk, k, chi, cut, normM2, sl.spec + (long long)dir * chi,
+        launch(finalize_spectrum_kernel<T, T>, 1, 128, 0, st, Sk, k, chi, cut, normM2, sl.spec + (long long)dir * chi,
                                                           isq, sl.trunc + dir);
-    KH_LAUNCHED();
     const int nkeep = chi < k ? chi : k;
     if (nkeep < chi) {
         KH_CUDA(cudaMemsetAsync(P, 0, sizeof(T) * (size_t)n * chi, st));
@@ -1142,15 +1142,11 @@ void Engine<T>::absorb(Slot<T>& sl, int s) {
         }
         gemm_rm<T>(chi, chi, n, C4E3, false, PtT, false, C4n, cs, T(1), T(0), nullptr, csk, sk_elems);   // C4n = C4E3 P~^T
         KH_CUDA(cudaMemsetAsync(cns, 0, 2 * sizeof(double), cs));
-        sumsq_kernel<T><<<sumsq_grid(chi2), 256, 0, cs>>>(C1n, chi2, cns);
-        KH_LAUNCHED();
-        sumsq_kernel<T><<<sumsq_grid(chi2), 256, 0, cs>>>(C4n, chi2, cns + 1);
-        KH_LAUNCHED();
-        store_normalized_kernel<T><<<grid_for(chi2), 256, 0, cs>>>(C1n, chi2, cns, sl.C + s * chi2, Cop + s * chi2);
-        KH_LAUNCHED();
-        store_normalized_kernel<T><<<grid_for(chi2), 256, 0, cs>>>(C4n, chi2, cns + 1, sl.C + ((s + 3) & 3) * chi2,
+        launch(sumsq_kernel<T>, sumsq_grid(chi2), 256, 0, cs, C1n, chi2, cns);
+        launch(sumsq_kernel<T>, sumsq_grid(chi2), 256, 0, cs, C4n, chi2, cns + 1);
+        launch(store_normalized_kernel<T>, grid_for(chi2), 256, 0, cs, C1n, chi2, cns, sl.C + s * chi2, Cop + s * chi2);
+        launch(store_normalized_kernel<T>, grid_for(chi2), 256, 0, cs, C4n, chi2, cns + 1, sl.C + ((s + 3) & 3) * chi2,
                                                                    Cop + ((s + 3) & 3) * chi2);
-        KH_LAUNCHED();
     }
     const T* E4 = Eop + ((s + 3) & 3) * E1;
     const int ln = lane_id();
@@ -1166,11 +1162,9 @@ void Engine<T>::absorb(Slot<T>& sl, int s) {
         gemm_rm<T>(chi * d2, chi, n, Y1, false, PtT, false, E4n, st, T(1), T(0), nullptr, skbuf, sk_elems);
     double* ns = dscr + DscrOff::kNorms;
     KH_CUDA(cudaMemsetAsync(ns + 2, 0, sizeof(double), st));
-    sumsq_kernel<T><<<sumsq_grid(E1), 256, 0, st>>>(E4n, E1, ns + 2);
-    KH_LAUNCHED();
-    store_normalized_kernel<T><<<grid_for(E1), 256, 0, st>>>(E4n, E1, ns + 2, sl.E + ((s + 3) & 3) * E1,
+    launch(sumsq_kernel<T>, sumsq_grid(E1), 256, 0, st, E4n, E1, ns + 2);
+    launch(store_normalized_kernel<T>, grid_for(E1), 256, 0, st, E4n, E1, ns + 2, sl.E + ((s + 3) & 3) * E1,
                                                             Eop + ((s + 3) & 3) * E1);
-    KH_LAUNCHED();
     if (side) join_side();
 }
 
@@ -1236,8 +1230,7 @@ int Engine<T>::sweep(int slot, int max_sweeps, int min_sweeps, double tol, doubl
     int done = 0;
     for (int it = 1; it <= max_sweeps; ++it) {
         for (int s = 0; s < 4; ++s) move(sl, s, slot);
-        delta_kernel<<<1, 256, 0, st>>>(sl.spec, sl.prev, dm.chi, sl.prev_valid ? 1 : 0, sl.delta);
-        KH_LAUNCHED();
+        launch(delta_kernel, 1, 256, 0, st, sl.spec, sl.prev, dm.chi, sl.prev_valid ? 1 : 0, sl.delta);
         sl.prev_valid = true;
         done = it;
         if (tol >= 0.0) {
@@ -1293,8 +1286,7 @@ int Engine<T>::sweep_lanes(const int* slot_ids, int count, int mx, int mn, doubl
             if (active[i]) {
                 bind(i);
                 Slot<T>& sl = slots[slot_ids[i]];
-                delta_kernel<<<1, 256, 0, st>>>(sl.spec, sl.prev, dm.chi, sl.prev_valid ? 1 : 0, sl.delta);
-                KH_LAUNCHED();
+                launch(delta_kernel, 1, 256, 0, st, sl.spec, sl.prev, dm.chi, sl.prev_valid ? 1 : 0, sl.delta);
                 sl.prev_valid = true;
                 done[i] = it;
                 if (tol >= 0.0) KH_CUDA(cudaMemcpyAsync(&delta[i], sl.delta, sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -1467,8 +1459,7 @@ static void svd_jacobi_launch(const T* X, int k, T* sv, T* L, T* Qm, int max_swe
     static std::atomic<size_t> granted[kMaxDevices] = {};   // per instantiation
     smem_opt_in(svd_jacobi_kernel<T, LP, R>, sm, granted);
     const int threads = ((kp / 2) * LP + 31) / 32 * 32;
-    svd_jacobi_kernel<T, LP, R><<<1, threads, sm, st>>>(X, k, sv, L, Qm, max_sweeps, tol, cut, sweep_count, nrel);
-    KH_LAUNCHED();
+    launch(svd_jacobi_kernel<T, LP, R>, 1, threads, sm, st, X, k, sv, L, Qm, max_sweeps, tol, cut, sweep_count, nrel);
 }
 
 // FP64 matrices beyond this size go to the cluster kernel: 64 x 64 takes 0.50 ms
@@ -1516,7 +1507,8 @@ void cholqr_factor(double* dG, int k, double cut_abs, double tau, T* X, cudaStre
     case KT: {                                                                                               \
         static std::atomic<size_t> granted[kMaxDevices] = {};                                                \
         smem_opt_in(cholqr_reg_kernel<T, KT>, sm, granted);                                                  \
-        cholqr_reg_kernel<T, KT><<<1, 512, sm, st>>>(dG, k, cut_abs, tau, X, sorted ? 1 : 0, ns_tol, clear ? 1 : 0); \
+        launch(cholqr_reg_kernel<T, KT>, 1, 512, sm, st, dG, k, cut_abs, tau, X, sorted ? 1 : 0, ns_tol,     \
+               clear ? 1 : 0);                                                                               \
         break;                                                                                               \
     }
             KH_CHOL(1) KH_CHOL(2) KH_CHOL(3) KH_CHOL(4) KH_CHOL(5)
@@ -1526,8 +1518,8 @@ void cholqr_factor(double* dG, int k, double cut_abs, double tau, T* X, cudaStre
         static std::atomic<size_t> granted[kMaxDevices] = {};
         smem_opt_in(cholqr_kernel<T>, 2 * sm, granted);
         cholqr_kernel<T><<<1, 1024, 2 * sm, st>>>(dG, k, cut_abs, tau, X, sorted ? 1 : 0, ns_tol, defer);
+        KH_LAUNCHED();
     }
-    KH_LAUNCHED();
 }
 template void cholqr_factor<float>(double*, int, double, double, float*, cudaStream_t, bool, double, double, bool);
 template void cholqr_factor<double>(double*, int, double, double, double*, cudaStream_t, bool, double, double, bool);

@@ -101,6 +101,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 gemm3x_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mBh,
               const __grid_constant__ CUtensorMap mBl, float* __restrict__ C, int M, int N, int K, int bn, Work W,
               long long ldc, long long split_stride, float alpha, const float* __restrict__ colscale, int* err) {
+    pdl_start();
     extern __shared__ uint8_t smem_raw[];
     __shared__ Bars bars;
     __shared__ uint32_t s_tmem;
@@ -416,6 +417,7 @@ gemm3x_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CU
 __global__ void __launch_bounds__(256)
 split_b_kernel(const float* __restrict__ B, long long sn, long long sk, int N, int K, float* __restrict__ hi,
                float* __restrict__ lo, int ld) {
+    pdl_start();
     __shared__ float t[32][33];
     const int n0 = blockIdx.y * 32, k0 = blockIdx.x * 32;
     const int lx = threadIdx.x & 31, ly = threadIdx.x >> 5;
@@ -437,6 +439,7 @@ split_b_kernel(const float* __restrict__ B, long long sn, long long sk, int N, i
 
 __global__ void reduce_kernel(const float* __restrict__ part, int splits, long long stride, int M, int N, int ldp,
                               float* __restrict__ C, long long ldc, float alpha, const float* __restrict__ colscale) {
+    pdl_start();
     const long long tot = (long long)M * N;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < tot; i += (long long)gridDim.x * blockDim.x) {
         const int m = (int)(i / N), n = (int)(i % N);
@@ -483,8 +486,7 @@ Plan make_plan(int M, int N, int K, long long sk_elems, int sms) {
 void gemm3x_split_b(const float* B, long long sn, long long sk, int N, int K, float* hi, float* lo, int ld,
                     cudaStream_t st) {
     dim3 grid((K + 31) / 32, (N + 31) / 32);
-    x3::split_b_kernel<<<grid, 256, 0, st>>>(B, sn, sk, N, K, hi, lo, ld);
-    KH_LAUNCHED();
+    launch(x3::split_b_kernel, grid, 256, 0, st, B, sn, sk, N, K, hi, lo, ld);
 }
 
 bool gemm3x_usable(const float* A, long long lda) { return ((uintptr_t)A & 15) == 0 && lda % 4 == 0; }
@@ -507,18 +509,16 @@ void gemm3x(const float* A, long long lda, bool a_mmajor, const float* Bhi, cons
     static std::atomic<size_t> granted[2][kMaxDevices] = {};
     if (a_mmajor) {
         smem_opt_in(x3::gemm3x_kernel<true>, (size_t)x3::SMEM, granted[1]);
-        x3::gemm3x_kernel<true><<<grid, x3::THREADS, x3::SMEM, st>>>(ma, mh, ml, out, M, N, K, p.bn, p.W, ldo, stride,
+        launch(x3::gemm3x_kernel<true>, grid, x3::THREADS, x3::SMEM, st, ma, mh, ml, out, M, N, K, p.bn, p.W, ldo, stride,
                                                                      al, cs, err);
     } else {
         smem_opt_in(x3::gemm3x_kernel<false>, (size_t)x3::SMEM, granted[0]);
-        x3::gemm3x_kernel<false><<<grid, x3::THREADS, x3::SMEM, st>>>(ma, mh, ml, out, M, N, K, p.bn, p.W, ldo,
+        launch(x3::gemm3x_kernel<false>, grid, x3::THREADS, x3::SMEM, st, ma, mh, ml, out, M, N, K, p.bn, p.W, ldo,
                                                                       stride, al, cs, err);
     }
-    KH_LAUNCHED();
     if (split) {
-        x3::reduce_kernel<<<grid_for((long long)M * N), 256, 0, st>>>(sk, p.W.splits, stride, M, N, ldp, C, ldc, alpha,
+        launch(x3::reduce_kernel, grid_for((long long)M * N), 256, 0, st, sk, p.W.splits, stride, M, N, ldp, C, ldc, alpha,
                                                                       colscale);
-        KH_LAUNCHED();
     }
 }
 

@@ -261,6 +261,7 @@ template <typename T, int LP, int R>
 __global__ void __launch_bounds__(LP * R / 2 * LP)
 svd_jacobi_kernel(const T* __restrict__ Xin, int k, T* __restrict__ s_out, T* __restrict__ L_out,
                   T* __restrict__ Q_out, int max_sweeps, double tol, double cut, int* sweep_count, int nrel) {
+    pdl_start();
     extern __shared__ unsigned char smem_raw[];
     constexpr int RL = LP * R;
     constexpr bool kPrefetchQ = sizeof(T) * R <= 48;   // keep the Q column pair in registers too
@@ -786,6 +787,7 @@ template <typename T, int KT>
 __global__ void __launch_bounds__(512, 1)
 cholqr_reg_kernel(double* __restrict__ G, int k, double cut_abs, double tau, T* __restrict__ X, int sorted,
                   double ns_tol, int clear) {
+    pdl_start();
     extern __shared__ unsigned char smem_raw[];
     T* Xs = reinterpret_cast<T*>(smem_raw);        // k x (k | 1): the result, transposed for coalesced rows
     constexpr int KR = 2 * KT, KM = 32 * KT;       // rows (16 apart) and KT columns (32 apart) of a thread

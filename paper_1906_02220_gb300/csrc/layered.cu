@@ -98,6 +98,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 layered_kernel(const float* __restrict__ Y, long long nb, int nc, const uint8_t* __restrict__ img1,
                const uint8_t* __restrict__ img2, float* __restrict__ out, int ntiles, int nst1, int nst2,
                int* err) {
+    pdl_start();
     static_assert(!BF || NPASS == 1, "BF16 runs one pass");
     constexpr Plan P = make_plan(D, NPASS, BF);
     constexpr int D2 = P.d2;
@@ -583,9 +584,7 @@ void launch_layered(const float* Y, long long nb, int p, const float* img1, cons
     static std::atomic<size_t> granted[kMaxDevices] = {};
     smem_opt_in(lay::layered_kernel<D, NPASS, BF>, smem, granted);
     const int grid = ntiles < device_sms() ? ntiles : device_sms();
-    lay::layered_kernel<D, NPASS, BF><<<grid, lay::THREADS, smem, st>>>(
-        Y, nb, nc, (const uint8_t*)img1, (const uint8_t*)img2, out, ntiles, nst1, nst2, err);
-    KH_LAUNCHED();
+    launch(lay::layered_kernel<D, NPASS, BF>, grid, lay::THREADS, smem, st, Y, nb, nc, (const uint8_t*)img1, (const uint8_t*)img2, out, ntiles, nst1, nst2, err);
 }
 
 template <int NPASS, bool BF>

@@ -116,6 +116,7 @@ template <int KT>
 __global__ void __launch_bounds__(256)
 rows_reduce_kernel(const float* __restrict__ part, int splits, int n, int k, float* __restrict__ Y,
                    double* __restrict__ G) {
+    pdl_start();
     constexpr int KP = 16 * KT, PER = kRows * KP / 256;
     __shared__ float t[kRows][KP];
     const int tid = threadIdx.x, r0 = blockIdx.x * kRows;
@@ -152,6 +153,7 @@ struct RowsOperands {
 template <int KT>
 __global__ void __launch_bounds__(256)
 rows_apply_kernel(RowsOperands o, int n, int k, double* __restrict__ G) {
+    pdl_start();
     constexpr int KP = 16 * KT;
     extern __shared__ float rows_smem[];
     float(*t)[KP] = reinterpret_cast<float(*)[KP]>(rows_smem);
@@ -185,6 +187,7 @@ template <int KT>
 __global__ void __launch_bounds__(256)
 rows_split_kernel(const float* __restrict__ Vw, const int* __restrict__ live, int n, int k, float* __restrict__ Vl,
                   float* __restrict__ R, uint64_t seed, uint64_t stream, double* __restrict__ G) {
+    pdl_start();
     constexpr int KP = 16 * KT, PER = kRows * KP / 256;
     __shared__ float tv[kRows][KP], tr[kRows][KP];
     const int tid = threadIdx.x, r0 = blockIdx.x * kRows;
@@ -213,6 +216,7 @@ template <int KT>
 __global__ void __launch_bounds__(256)
 rows_project_kernel(const float* __restrict__ Vl, const double* __restrict__ C, int n, int k, float* __restrict__ R,
                     double* __restrict__ G) {
+    pdl_start();
     constexpr int KP = 16 * KT;
     extern __shared__ float rows_smem[];
     float(*t)[KP] = reinterpret_cast<float(*)[KP]>(rows_smem);
@@ -247,12 +251,11 @@ rows_project_kernel(const float* __restrict__ Vl, const double* __restrict__ C, 
 #define KH_ROWS_SWITCH                                                                                                 \
     switch ((k + 15) / 16) {                                                                                           \
         KH_ROWS(1) KH_ROWS(2) KH_ROWS(3) KH_ROWS(4) KH_ROWS(5) KH_ROWS(6) default : fail(KH_EINVAL, "rows: k > 96");   \
-    }                                                                                                                  \
-    KH_LAUNCHED();
+    }
 
 void rows_reduce(const float* part, int splits, int n, int k, float* Y, double* G, cudaStream_t st) {
     const int grid = (n + kRows - 1) / kRows;
-#define KH_ROWS_CALL(KT) rows_reduce_kernel<KT><<<grid, 256, 0, st>>>(part, splits, n, k, Y, G)
+#define KH_ROWS_CALL(KT) launch(rows_reduce_kernel<KT>, grid, 256, 0, st, part, splits, n, k, Y, G)
     KH_ROWS_SWITCH
 #undef KH_ROWS_CALL
 }
@@ -266,7 +269,7 @@ void rows_apply(const float* Y, const float* X, int n, int k, float* Q, double* 
         constexpr size_t sm = sizeof(float) * 16 * KT * (kRows + 16 * KT);            \
         static std::atomic<size_t> granted[kMaxDevices] = {};                         \
         smem_opt_in(rows_apply_kernel<KT>, sm, granted);                              \
-        rows_apply_kernel<KT><<<grid, 256, sm, st>>>(o, n, k, G);                     \
+        launch(rows_apply_kernel<KT>, grid, 256, sm, st, o, n, k, G);                 \
     }
     KH_ROWS_SWITCH
 #undef KH_ROWS_CALL
@@ -275,7 +278,7 @@ void rows_apply(const float* Y, const float* X, int n, int k, float* Q, double* 
 void rows_split(const float* Vw, const int* live, int n, int k, float* Vl, float* R, uint64_t seed, uint64_t stream,
                 double* G, cudaStream_t st) {
     const int grid = (n + kRows - 1) / kRows;
-#define KH_ROWS_CALL(KT) rows_split_kernel<KT><<<grid, 256, 0, st>>>(Vw, live, n, k, Vl, R, seed, stream, G)
+#define KH_ROWS_CALL(KT) launch(rows_split_kernel<KT>, grid, 256, 0, st, Vw, live, n, k, Vl, R, seed, stream, G)
     KH_ROWS_SWITCH
 #undef KH_ROWS_CALL
 }
@@ -287,7 +290,7 @@ void rows_project(const float* Vl, const double* C, int n, int k, float* R, doub
         constexpr size_t sm = sizeof(float) * 16 * KT * (2 * kRows + 16 * KT);        \
         static std::atomic<size_t> granted[kMaxDevices] = {};                         \
         smem_opt_in(rows_project_kernel<KT>, sm, granted);                            \
-        rows_project_kernel<KT><<<grid, 256, sm, st>>>(Vl, C, n, k, R, G);            \
+        launch(rows_project_kernel<KT>, grid, 256, sm, st, Vl, C, n, k, R, G);            \
     }
     KH_ROWS_SWITCH
 #undef KH_ROWS_CALL

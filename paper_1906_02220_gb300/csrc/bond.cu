@@ -759,7 +759,7 @@ void Engine<T>::cost_gradient(int gamma, const double* gate, const double* A2in,
     KH_LAUNCHED();
     double h[8];
     KH_CUDA(cudaMemcpyAsync(h, cost, sizeof(h), cudaMemcpyDeviceToHost, st));
-    KH_CUDA(cudaStreamSynchronize(st));
+    sync_checked();
     if (!(h[5] == h[5]) || !(h[6] == h[6])) fail(KH_ENUMERIC, "NaN in the bond cost");
     cost_out[0] = h[5] + h[0];          // d from the A side
     cost_out[1] = h[0];                 // <T'|N|T'>
@@ -868,7 +868,7 @@ int Engine<T>::als_run(int gamma, double* rel_cost) {
     int hf0 = 0;
     KH_CUDA(cudaMemcpyAsync(hc, cost, sizeof(hc), cudaMemcpyDeviceToHost, st));
     KH_CUDA(cudaMemcpyAsync(&hf0, flags, sizeof(int), cudaMemcpyDeviceToHost, st));
-    KH_CUDA(cudaStreamSynchronize(st));
+    sync_checked();
     if (hf0) fail(KH_ENUMERIC, "ALS: Cholesky breakdown (metric not positive)");
     *rel_cost = hc[0] != 0.0 ? hc[1] / hc[0] : 0.0;
     return (int)hc[3] - 1;                                   // sweeps (the first evaluation is the start)
@@ -1007,7 +1007,7 @@ void Engine<T>::observables(const double* Hh, double hA, double hB, int mx, int 
     KH_CUDA(cudaMemcpyAsync(out, dout, sizeof(double) * 10, cudaMemcpyDeviceToHost, st));
     for (int g = 0; g < 3; ++g)
         KH_CUDA(cudaMemcpyAsync(tr + 4 * g, slots[3 + g].trunc, 4 * sizeof(double), cudaMemcpyDeviceToHost, st));
-    KH_CUDA(cudaStreamSynchronize(st));
+    sync_checked();
     double mt = 0.0;
     for (int i = 0; i < 12; ++i) mt = fmax(mt, tr[i]);
     out[10] = mt;

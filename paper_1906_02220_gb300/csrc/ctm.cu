@@ -1353,27 +1353,59 @@ void Engine<T>::compute_metric(Slot<T>& sl, double* N_out) {
     refresh_operands(sl);
     const T *C1 = Cop, *C2 = Cop + chi2, *C3 = Cop + 2 * chi2, *C4 = Cop + 3 * chi2;
     const T *E1p = Eop, *E2 = Eop + E1, *E3 = Eop + 2 * E1, *E4 = Eop + 3 * E1;
-    gemm_rm<T>(chi, d2 * chi, chi, C1, false, E1p, false, mt1, st);          // [h][(u,b)]
-    gemm_rm<T>(chi * d2, chi, chi, mt1, false, C2, false, mt2, st);           // [(h,u)][c]
-    gemm_rm<T>(chi * d2, d2 * chi, chi, mt2, false, E2, false, mup, st);      // [(h,u)][(r,e)]
-    gemm_rm<T>(chi, d2 * chi, chi, C3, false, E3, false, mt1, st);           // [e][(d,g)]
-    gemm_rm<T>(chi * d2, chi, chi, mt1, false, C4, false, mt2, st);           // [(e,d)][i]
-    gemm_rm<T>(chi * d2, d2 * chi, chi, mt2, false, E4, false, mdn, st);      // [(e,d)][(l,h)]
+    // products of row-major matrices, on the tensor cores where they are wide enough
+    auto product = [&](int M, int Nn, int K, const T* A, const T* B, T* out) {
+        if (!product3x(lane_id(), A, K, false, B, 1, Nn, out, M, Nn, K, Nn))
+            gemm_rm<T>(M, Nn, K, A, false, B, false, out, st);
+    };
+    product(chi, d2 * chi, chi, C1, E1p, mt1);                                 // [h][(u,b)]
+    product(chi * d2, chi, chi, mt1, C2, mt2);                                 // [(h,u)][c]
+    product(chi * d2, d2 * chi, chi, mt2, E2, mup);                            // [(h,u)][(r,e)]
+    product(chi, d2 * chi, chi, C3, E3, mt1);                                  // [e][(d,g)]
+    product(chi * d2, chi, chi, mt1, C4, mt2);                                 // [(e,d)][i]
+    product(chi * d2, d2 * chi, chi, mt2, E4, mdn);                            // [(e,d)][(l,h)]
     permute<T, T>(mup, mupp, {chi, D, D, D, D, chi}, {1, 2, 3, 4, 0, 5}, st);  // [uk][ub][rk][rb][h][e]
-    permute<T, T>(mdn, mdnp, {chi, D, D, D, D, chi}, {5, 0, 1, 2, 3, 4}, st);  // [h][e][dk][db][lk][lb]
-    gemm_rm<T>(d2 * d2, d2 * d2, chi * chi, mupp, false, mdnp, false, mN4, st, T(1), T(0), nullptr, skbuf,
-               sk_elems);                                                      // K = chi^2: split over CTAs
+    // K = chi^2.  On the tensor cores it is the more accurate one as well, relative
+    // to FP64 (Frobenius): 256 x 256 x 4096 1.6e-7 against 1.1e-6, 1296 x 1296 x 20736
+    // 3.0e-7 against 2.6e-6.  Time on the CUDA cores: 2.8 ms at (6, 144), 24 at
+    // (8, 144), of environments of 81 and 284 that went to 78 and 262; at (5, 100),
+    // 7.8e9 flops, the environment went from 24.2 to 23.7 ms, at (4, 64), 5e8 flops in
+    // a K split over the SMs, it stayed at 11.3.  The line lies between.
+    constexpr double kMinMetric3x = 1e9;
+    bool joined = false;
+    if constexpr (sizeof(T) == 4) {
+        if (tc_npass && 2.0 * dm.D4 * dm.D4 * chi2 >= kMinMetric3x && gemm3x_usable(mupp, chi2)) {
+            permute_split(mdn, mdnp, mup, {chi, D, D, D, D, chi}, {1, 2, 3, 4, 5, 0}, st);   // [dk][db][lk][lb][h][e]
+            gemm3x(mupp, chi2, false, mdnp, mup, (int)chi2, mN4, dm.D4, dm.D4, (int)chi2, dm.D4, 1.f, nullptr, skbuf,
+                   sk_elems, tc_err, st);
+            joined = true;
+        }
+    }
+    if (!joined) {
+        permute<T, T>(mdn, mdnp, {chi, D, D, D, D, chi}, {5, 0, 1, 2, 3, 4}, st);   // [h][e][dk][db][lk][lb]
+        gemm_rm<T>(d2 * d2, d2 * d2, chi * chi, mupp, false, mdnp, false, mN4, st, T(1), T(0), nullptr, skbuf,
+                   sk_elems);
+    }
     permute<T, double>(mN4, N_out, {D, D, D, D, D, D, D, D}, {6, 0, 2, 4, 7, 1, 3, 5}, st);
     symmetrize_kernel<<<grid_for((long long)dm.D4 * dm.D4), 256, 0, st>>>(N_out, dm.D4);
     KH_LAUNCHED();
     prof_end(5, 0.0);
 }
 
+// Waits for the stream and reports a tensor-core kernel whose bounded wait ran out.
+template <typename T>
+void Engine<T>::sync_checked() {
+    int terr = 0;
+    if (tc_npass) KH_CUDA(cudaMemcpyAsync(&terr, tc_err, sizeof(int), cudaMemcpyDeviceToHost, st));
+    KH_CUDA(cudaStreamSynchronize(st));
+    if (terr) fail(KH_ETIMEOUT, "tensor-core kernel wait timed out (flag " + std::to_string(terr) + ")");
+}
+
 template <typename T>
 void Engine<T>::metric(int slot, double* N_out) {
     compute_metric(slots[slot], N);
     KH_CUDA(cudaMemcpyAsync(N_out, N, sizeof(double) * dm.D4 * dm.D4, cudaMemcpyDeviceToDevice, st));
-    KH_CUDA(cudaStreamSynchronize(st));
+    sync_checked();
 }
 
 template <typename T>
@@ -1417,7 +1449,7 @@ double Engine<T>::kappa(int slot) {
     KH_LAUNCHED();
     double h[4];
     KH_CUDA(cudaMemcpyAsync(h, z, sizeof(h), cudaMemcpyDeviceToHost, st));
-    KH_CUDA(cudaStreamSynchronize(st));
+    sync_checked();
     return h[0] * h[1] / (h[2] * h[3]);
 }
 
@@ -1437,7 +1469,7 @@ void Engine<T>::expval(int slot, const double* ops, int n_ops, double* vals) {
     expval_kernel<<<1, 32, 0, st>>>(dops, n_ops, p, X, dvals);
     KH_LAUNCHED();
     KH_CUDA(cudaMemcpyAsync(vals, dvals, sizeof(double) * n_ops, cudaMemcpyDeviceToHost, st));
-    KH_CUDA(cudaStreamSynchronize(st));
+    sync_checked();
 }
 
 template <typename T>

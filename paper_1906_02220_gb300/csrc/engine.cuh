@@ -265,6 +265,7 @@ struct Engine : EngineBase {
     void absorb(Slot<T>& sl, int s);
     void move(Slot<T>& sl, int s, int slot_id);
     void compute_metric(Slot<T>& sl, double* N_out);
+    void sync_checked();
     void build_derived(Slot<T>& sl);
 
     // bond internals

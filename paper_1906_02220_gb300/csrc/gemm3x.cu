@@ -2,7 +2,7 @@
 //   C[m][n] = alpha * colscale[n] * sum_k A[m][k] B[k][n]
 // for the FP32 contractions of a CTM move in the tensor-core precisions: the
 // edge products of the enlarged corners and of the absorption, the subspace
-// products M V and M^T U and the projectors.
+// products M V and M^T U, the basis products, the projectors and the bond metric.
 //
 // Accuracy.  Every operand is split as x = hi + lo with hi rounded to nearest
 // TF32 (|lo| <= 2^-12 |x|), and lo B_hi + hi B_lo + hi B_hi is formed.  The

@@ -302,26 +302,34 @@ __global__ void als_x_kernel(const double* __restrict__ N, const double* __restr
 }
 
 // R[(o1,o2,k)][(o1',o2',k')] = sum_{t1',t2',ph} X[(o1,o2)][row(o',t')][(ph,k)] Oth[ph][t1'][t2'][k']
-// (one thread per entry)
+// LANES threads an entry, joined by shuffles in a fixed order.  While the D^6
+// entries are few, a thread an entry leaves most SMs idle and runs its 4 D^2
+// dependent FP64 FMAs one after the other (D = 4: 22 us against 6).  From D = 6 on the
+// entries fill the GPU and eight lanes would only load more.
+inline int als_r_lanes(long long entries) { return entries < 152LL * 256 ? 8 : 1; }
+template <int LANES>
 __global__ void als_r_kernel(const double* __restrict__ X, const double* __restrict__ Oth, int D, int side,
                              double* __restrict__ R, const int* skip) {
     if (skip && *skip) return;
     const int D4 = D * D * D * D, m = D * D * D;
-    const long long totR = (long long)m * m;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < totR;
-         i += (long long)gridDim.x * blockDim.x) {
-        int a = (int)(i / m), b = (int)(i % m);
-        int o1 = a / (D * D), o2 = (a / D) % D, k = a % D;
-        int q1 = b / (D * D), q2 = (b / D) % D, kp = b % D;
+    const int totR = m * m, l = threadIdx.x % LANES;
+    const int step = (int)(gridDim.x * blockDim.x) / LANES;
+    // whole warps stay in the loop together: the shuffles need every lane of a group
+    for (int i = (int)(blockIdx.x * blockDim.x + threadIdx.x) / LANES; i < (totR + 31) / 32 * 32; i += step) {
+        const int e = min(i, totR - 1), a = e / m, b = e % m;
+        const int o1 = a / (D * D), o2 = (a / D) % D, k = a % D;
+        const int q1 = b / (D * D), q2 = (b / D) % D, kp = b % D;
         const double* x = X + (long long)(o1 * D + o2) * D4 * 4 * D;
         double s = 0.0;
-        for (int t1 = 0; t1 < D; ++t1)
-            for (int t2 = 0; t2 < D; ++t2) {
-                int j = row_index(side, q1, q2, t1, t2, D);
-                for (int ph = 0; ph < 4; ++ph)
-                    s += x[((long long)j * 4 + ph) * D + k] * Oth[((ph * D + t1) * D + t2) * D + kp];
-            }
-        R[i] = s;
+#pragma unroll 4
+        for (int t = l; t < 4 * D * D; t += LANES) {
+            const int ph = t % 4, t2 = (t / 4) % D, t1 = t / (4 * D);
+            const int j = row_index(side, q1, q2, t1, t2, D);
+            s += x[(j * 4 + ph) * D + k] * Oth[((ph * D + t1) * D + t2) * D + kp];
+        }
+#pragma unroll
+        for (int o = LANES / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (l == 0 && i < totR) R[i] = s;
     }
 }
 
@@ -482,18 +490,27 @@ __global__ void als_cost_kernel(const double* __restrict__ R, const double* __re
     }
 }
 
-// c = <T'|N|T'> = sum_p T'_p N T'_p
-__global__ void tnt_kernel(const double* __restrict__ Tp, const double* __restrict__ N, int D4, double* out) {
-    double s = 0.0;
-    long long tot = 16LL * D4 * D4;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < tot;
-         i += (long long)gridDim.x * blockDim.x) {
-        int p = (int)(i / ((long long)D4 * D4));
-        int a = (int)((i / D4) % D4), b = (int)(i % D4);
-        s += Tp[(long long)p * D4 + a] * N[(long long)a * D4 + b] * Tp[(long long)p * D4 + b];
+// c = <T'|N|T'> = sum_ab N_ab sum_p T'_pa T'_pb: a CTA per row a, one atomic
+// each.  Bound by its launch and the atomics; with a thread per (p, a, b), 64-bit
+// index divisions and an atomic per warp it took 52 us at D = 4 against 6.
+constexpr int kTntThreads = 128;
+__global__ void __launch_bounds__(kTntThreads)
+tnt_kernel(const double* __restrict__ Tp, const double* __restrict__ N, int D4, double* out) {
+    __shared__ double red[kTntThreads / 32];
+    const int a = blockIdx.x;
+    double ta[16], s = 0.0;
+#pragma unroll
+    for (int p = 0; p < 16; ++p) ta[p] = Tp[(long long)p * D4 + a];
+    for (int b = threadIdx.x; b < D4; b += kTntThreads) {
+        double w = 0.0;
+#pragma unroll
+        for (int p = 0; p < 16; ++p) w = fma(ta[p], Tp[(long long)p * D4 + b], w);
+        s = fma(N[(long long)a * D4 + b], w, s);
     }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(out, s);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) atomicAdd(out, (red[0] + red[1]) + (red[2] + red[3]));
 }
 
 // truncated-SVD start from the singular triplets of Tm (descending sv):
@@ -695,21 +712,35 @@ __global__ void gauge_kernel(const double* __restrict__ A2, const double* __rest
 // normal-equation matrices of that side (d = sum_ph Own_ph^T R Own_ph
 // - 2 sum Own[ph][a] S[a][ph] + <T'|N|T'>):
 //   G[ph][a] = sum_a' (R[a][a'] + R[a'][a]) Own[ph][a'] - 2 S[a][ph];
-// the quadratic and linear parts of d are added into *e.
+// the quadratic and linear parts of d are added into *e.  A warp an entry (ph, a),
+// lanes over a', one atomic a CTA; a thread an entry ran the 2 m loads one
+// after the other on one or two CTAs: 20 us at D = 4 against 5.
 __global__ void cost_grad_kernel(const double* __restrict__ R, const double* __restrict__ S,
                                  const double* __restrict__ Own, int m, double* __restrict__ G, double* e) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 4 * m; i += gridDim.x * blockDim.x) {
+    __shared__ double red[32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    double part = 0.0;
+    for (int i = blockIdx.x * nw + warp; i < 4 * m; i += gridDim.x * nw) {
         const int ph = i / m, a = i % m;
         const double* own = Own + (long long)ph * m;
-        double sym = 0.0, row = 0.0;
-        for (int b = 0; b < m; ++b) {
-            const double r1 = R[(long long)a * m + b], r2 = R[(long long)b * m + a];
-            sym += (r1 + r2) * own[b];
-            row += r1 * own[b];
+        double col = 0.0, row = 0.0;
+        for (int b = lane; b < m; b += 32) {
+            row = fma(R[(long long)a * m + b], own[b], row);
+            col = fma(R[(long long)b * m + a], own[b], col);
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            row += __shfl_xor_sync(0xffffffffu, row, o);
+            col += __shfl_xor_sync(0xffffffffu, col, o);
         }
         const double sa = S[(long long)a * 4 + ph];
-        G[i] = sym - 2.0 * sa;
-        atomicAdd(e, own[a] * (row - 2.0 * sa));
+        if (lane == 0) G[i] = (row + col) - 2.0 * sa;
+        part += own[a] * (row - 2.0 * sa);
+    }
+    if (lane == 0) red[warp] = part;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < nw; ++w) part += red[w];
+        atomicAdd(e, part);
     }
 }
 
@@ -721,7 +752,8 @@ void Engine<T>::normal_equations(const double* oth, int side, const int* skip) {
     const int sgrid = (int)((4LL * m * 32 + threads - 1) / threads);
     als_x_kernel<<<grid_for(nX), threads, 0, st>>>(N, oth, D, side, XA, skip);
     KH_LAUNCHED();
-    als_r_kernel<<<grid_for(nR), threads, 0, st>>>(XA, oth, D, side, R, skip);
+    if (als_r_lanes(nR) == 1) als_r_kernel<1><<<grid_for(nR), threads, 0, st>>>(XA, oth, D, side, R, skip);
+    else als_r_kernel<8><<<grid_for(8 * nR), threads, 0, st>>>(XA, oth, D, side, R, skip);
     KH_LAUNCHED();
     als_s_kernel<<<sgrid, threads, 0, st>>>(XA, slots[als_slot].Ts, D, side, S, skip);
     KH_LAUNCHED();
@@ -748,14 +780,14 @@ void Engine<T>::cost_gradient(int gamma, const double* gate, const double* A2in,
     KH_CUDA(cudaMemcpyAsync(A2, A2in, sizeof(double) * own, cudaMemcpyDeviceToDevice, st));
     KH_CUDA(cudaMemcpyAsync(B2, B2in, sizeof(double) * own, cudaMemcpyDeviceToDevice, st));
     KH_CUDA(cudaMemsetAsync(cost, 0, 8 * sizeof(double), st));
-    tnt_kernel<<<grid_for(16LL * dm.D4 * dm.D4), 256, 0, st>>>(sl.Ts, N, dm.D4, cost);
+    tnt_kernel<<<dm.D4, kTntThreads, 0, st>>>(sl.Ts, N, dm.D4, cost);
     KH_LAUNCHED();
     als_slot = gamma;
     normal_equations(B2, 0, nullptr);                      // A side (B'' fixed)
-    cost_grad_kernel<<<grid_for(own), 256, 0, st>>>(R, S, A2, m, gA, cost + 5);
+    cost_grad_kernel<<<(int)(own + 7) / 8, 256, 0, st>>>(R, S, A2, m, gA, cost + 5);
     KH_LAUNCHED();
     normal_equations(A2, 1, nullptr);                      // B side (A'' fixed)
-    cost_grad_kernel<<<grid_for(own), 256, 0, st>>>(R, S, B2, m, gB, cost + 6);
+    cost_grad_kernel<<<(int)(own + 7) / 8, 256, 0, st>>>(R, S, B2, m, gB, cost + 6);
     KH_LAUNCHED();
     double h[8];
     KH_CUDA(cudaMemcpyAsync(h, cost, sizeof(h), cudaMemcpyDeviceToHost, st));
@@ -804,7 +836,7 @@ int Engine<T>::als_run(int gamma, double* rel_cost) {
     // <T'|N|T'>
     KH_CUDA(cudaMemsetAsync(cost, 0, 8 * sizeof(double), st));
     KH_CUDA(cudaMemsetAsync(flags, 0, 8 * sizeof(int), st));
-    tnt_kernel<<<grid_for(16LL * D4 * D4), 256, 0, st>>>(Tp, N, D4, cost);
+    tnt_kernel<<<D4, kTntThreads, 0, st>>>(Tp, N, D4, cost);
     KH_LAUNCHED();
     // truncated SVD start: Tm[(sA,aA,u,r)][(sB,aB,d,l)] from T'[sA,aA,sB,aB,l,u,r,d]
     permute<double, double>(Tp, Tm, {2, 2, 2, 2, D, D, D, D}, {0, 1, 5, 6, 2, 3, 7, 4}, st);

@@ -34,6 +34,7 @@ __device__ __forceinline__ void bond_strides(int gamma, int D, int& s_u, int& s_
 
 __global__ void composite_kernel(const double* __restrict__ A, const double* __restrict__ B, int D, int gamma,
                                  Mat4 g, int has_gate, double* __restrict__ T) {
+    pdl_start();
     const int D4 = D * D * D * D, D3 = D * D * D;
     int tot = 16 * D4;
     int su, sr, sk;
@@ -62,6 +63,7 @@ __global__ void composite_kernel(const double* __restrict__ A, const double* __r
 //   Tcor_f[l][u][p][r][d], Tedg_f[l][d][p][u][r]  (frame-f legs).
 template <typename T>
 __global__ void derived_kernel(const double* __restrict__ Tm, int p, int D, int pmax, T* Tcor, T* Tedg) {
+    pdl_start();
     const int D4 = D * D * D * D;
     int tot = 4 * p * D4;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < tot; i += gridDim.x * blockDim.x) {
@@ -102,6 +104,7 @@ __device__ __forceinline__ int frame_offset(int f, int L, int U, int R, int Dd, 
 // in W and the FP32 remainder in lo.
 template <typename T>
 __global__ void wt_kernel(const double* __restrict__ Tm, int p, int D, T* Wc, T* We, T* Wc_lo, T* We_lo) {
+    pdl_start();
     const int d2 = D * D, d4 = d2 * d2;
     const long long per = (long long)d4 * d4;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < 8 * per;
@@ -149,6 +152,7 @@ __global__ void wt_kernel(const double* __restrict__ Tm, int p, int D, T* Wc, T*
 __global__ void layered_img_kernel(const double* __restrict__ Tm, const double* __restrict__ Tb, int p, int D,
                                    lay::Plan P, int npass, float* __restrict__ img1, float* __restrict__ img2,
                                    long long per1, long long per2) {
+    pdl_start();
     // per1, per2 in floats; elements of P.esz bytes (TF32 values or BF16)
     const int npl = npass == 3 ? 2 : 1;
     const int epf = 4 / P.esz;                                 // elements per float slot
@@ -199,15 +203,13 @@ __global__ void layered_img_kernel(const double* __restrict__ Tm, const double* 
 void build_layered_images(const double* Tm, int p, int D, int npass, bool bf16, float* img1, float* img2,
                           long long per1, long long per2, cudaStream_t st, const double* Tbra) {
     const long long tot = 8 * (per1 + per2) * (bf16 ? 2 : 1);
-    layered_img_kernel<<<grid_for(tot), 256, 0, st>>>(Tm, Tbra ? Tbra : Tm, p, D, lay::make_plan(D, npass, bf16),
-                                                      npass, img1, img2, per1, per2);
-    KH_LAUNCHED();
+    launch(layered_img_kernel, grid_for(tot), 256, 0, st, Tm, Tbra ? Tbra : Tm, p, D, lay::make_plan(D, npass, bf16),
+           npass, img1, img2, per1, per2);
 }
 
 template <typename T>
 void derive_operands(const double* Tm, int p, int D, int pmax, T* Tcor, T* Tedg, cudaStream_t st) {
-    derived_kernel<T><<<grid_for(4LL * p * D * D * D * D), 256, 0, st>>>(Tm, p, D, pmax, Tcor, Tedg);
-    KH_LAUNCHED();
+    launch(derived_kernel<T>, grid_for(4LL * p * D * D * D * D), 256, 0, st, Tm, p, D, pmax, Tcor, Tedg);
 }
 template void derive_operands<float>(const double*, int, int, int, float*, float*, cudaStream_t);
 template void derive_operands<double>(const double*, int, int, int, double*, double*, cudaStream_t);
@@ -215,8 +217,7 @@ template void derive_operands<double>(const double*, int, int, int, double*, dou
 template <typename T>
 void Engine<T>::build_derived(Slot<T>& sl) {
     int tot = 4 * sl.p * dm.D4;
-    derived_kernel<T><<<grid_for(tot), 256, 0, st>>>(sl.Ts, sl.p, dm.D, dm.pmax, sl.Tcor, sl.Tedg);
-    KH_LAUNCHED();
+    launch(derived_kernel<T>, grid_for(tot), 256, 0, st, sl.Ts, sl.p, dm.D, dm.pmax, sl.Tcor, sl.Tedg);
     // the double-layer form costs D^8 per block against 2 p D^6 layer by layer
     sl.dl = dm.dl_alloc && dm.d2 <= 2 * sl.p;
     if (dm.lay && !sl.dl)
@@ -225,9 +226,8 @@ void Engine<T>::build_derived(Slot<T>& sl) {
     if (sl.dl) {
         const bool split = sizeof(T) == 4 && tc_npass == 3 && dm.D4 % 4 == 0;
         const long long tot8 = 8LL * dm.D4 * dm.D4;
-        wt_kernel<T><<<grid_for(tot8), 256, 0, st>>>(sl.Ts, sl.p, dm.D, sl.Wcor, sl.Wedg,
-                                                     split ? sl.Wcor_lo : nullptr, split ? sl.Wedg_lo : nullptr);
-        KH_LAUNCHED();
+        launch(wt_kernel<T>, grid_for(tot8), 256, 0, st, sl.Ts, sl.p, dm.D, sl.Wcor, sl.Wedg,
+               split ? sl.Wcor_lo : nullptr, split ? sl.Wedg_lo : nullptr);
     }
 }
 
@@ -247,8 +247,7 @@ void Engine<T>::build_composite(int slot, int gamma, const double* gate) {
     Slot<T>& sl = slots[slot];
     Mat4 g;
     for (int i = 0; i < 16; ++i) g.v[i] = gate ? gate[i] : 0.0;
-    composite_kernel<<<grid_for(16 * dm.D4), 256, 0, st>>>(A, B, dm.D, gamma, g, gate != nullptr, sl.Ts);
-    KH_LAUNCHED();
+    launch(composite_kernel, grid_for(16 * dm.D4), 256, 0, st, A, B, dm.D, gamma, g, gate != nullptr, sl.Ts);
     sl.p = 16;
     build_derived(sl);
 }
@@ -283,6 +282,7 @@ __device__ __forceinline__ int row_index(int side, int o1, int o2, int t1, int t
 // X[(o1,o2)][j][(ph,k)] = sum_{t1,t2} N[row(o,t)][j] Oth[ph][t1][t2][k]
 __global__ void als_x_kernel(const double* __restrict__ N, const double* __restrict__ Oth, int D, int side,
                              double* __restrict__ X, const int* skip) {
+    pdl_start();
     if (skip && *skip) return;
     const int D4 = D * D * D * D, d2 = D * D;
     long long tot = (long long)d2 * D4 * 4 * D;
@@ -310,6 +310,7 @@ inline int als_r_lanes(long long entries) { return entries < 152LL * 256 ? 8 : 1
 template <int LANES>
 __global__ void als_r_kernel(const double* __restrict__ X, const double* __restrict__ Oth, int D, int side,
                              double* __restrict__ R, const int* skip) {
+    pdl_start();
     if (skip && *skip) return;
     const int D4 = D * D * D * D, m = D * D * D;
     const int totR = m * m, l = threadIdx.x % LANES;
@@ -337,6 +338,7 @@ __global__ void als_r_kernel(const double* __restrict__ X, const double* __restr
 // (one warp per entry, lanes over j: D^4 4 terms each)
 __global__ void als_s_kernel(const double* __restrict__ X, const double* __restrict__ Tp, int D, int side,
                              double* __restrict__ S, const int* skip) {
+    pdl_start();
     if (skip && *skip) return;
     const int D4 = D * D * D * D, m = D * D * D;
     const int lane = threadIdx.x & 31;
@@ -366,6 +368,7 @@ __global__ void als_s_kernel(const double* __restrict__ X, const double* __restr
 __global__ void chol_solve_kernel(const double* __restrict__ R, const double* __restrict__ S, int m, double reg,
                                   double* __restrict__ Wg, double* __restrict__ Own, int* flag, const int* skip,
                                   int smem) {
+    pdl_start();
     if (skip && *skip) return;
     extern __shared__ double sh_w[];
     __shared__ double s_delta, s_rd;
@@ -448,6 +451,7 @@ __global__ void chol_solve_kernel(const double* __restrict__ R, const double* __
 __global__ void als_cost_kernel(const double* __restrict__ R, const double* __restrict__ S,
                                 const double* __restrict__ Own, int m, double* cost, int* done, double tol,
                                 int first, const int* skip) {
+    pdl_start();
     if (skip && *skip) return;
     __shared__ double red[32];
     __shared__ int s_last;
@@ -496,6 +500,7 @@ __global__ void als_cost_kernel(const double* __restrict__ R, const double* __re
 constexpr int kTntThreads = 128;
 __global__ void __launch_bounds__(kTntThreads)
 tnt_kernel(const double* __restrict__ Tp, const double* __restrict__ N, int D4, double* out) {
+    pdl_start();
     __shared__ double red[kTntThreads / 32];
     const int a = blockIdx.x;
     double ta[16], s = 0.0;
@@ -517,6 +522,7 @@ tnt_kernel(const double* __restrict__ Tp, const double* __restrict__ N, int D4, 
 // A''[(sA,aA,u,r)][k] = U[:,k] s_k^{1/2}; colscale for B'' = Tm^T U s^{-1/2}
 template <typename TJ>
 __global__ void svd_init_kernel(const TJ* Ut, const TJ* sv, int mT, int D, double* A2m, double* colsc, double* Wd) {
+    pdl_start();
     double s0 = (double)sv[0];
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < mT * D; i += gridDim.x * blockDim.x) {
         int r = i / D, k = i % D;
@@ -594,6 +600,7 @@ __device__ void jacobi_serial(double* A, double* V, int n) {
 // unit Frobenius norms; then written back to the site layouts.
 __global__ void gauge_kernel(const double* __restrict__ A2, const double* __restrict__ B2, int D, int gamma,
                              double* __restrict__ Asite, double* __restrict__ Bsite) {
+    pdl_start();
     __shared__ double GA[64], GB[64], WA[64], H[64], Uh[64], SA[64], SAi[64], Xg[64], Yg[64], mu[8], lam[8];
     __shared__ int perm[8];
     __shared__ double sgn[8], nrm[2];
@@ -717,6 +724,7 @@ __global__ void gauge_kernel(const double* __restrict__ A2, const double* __rest
 // after the other on one or two CTAs: 20 us at D = 4 against 5.
 __global__ void cost_grad_kernel(const double* __restrict__ R, const double* __restrict__ S,
                                  const double* __restrict__ Own, int m, double* __restrict__ G, double* e) {
+    pdl_start();
     __shared__ double red[32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     double part = 0.0;
@@ -750,13 +758,10 @@ void Engine<T>::normal_equations(const double* oth, int side, const int* skip) {
     const int threads = 256;
     const long long nX = 4LL * dm.d2 * D4 * D, nR = (long long)m * m;
     const int sgrid = (int)((4LL * m * 32 + threads - 1) / threads);
-    als_x_kernel<<<grid_for(nX), threads, 0, st>>>(N, oth, D, side, XA, skip);
-    KH_LAUNCHED();
-    if (als_r_lanes(nR) == 1) als_r_kernel<1><<<grid_for(nR), threads, 0, st>>>(XA, oth, D, side, R, skip);
-    else als_r_kernel<8><<<grid_for(8 * nR), threads, 0, st>>>(XA, oth, D, side, R, skip);
-    KH_LAUNCHED();
-    als_s_kernel<<<sgrid, threads, 0, st>>>(XA, slots[als_slot].Ts, D, side, S, skip);
-    KH_LAUNCHED();
+    launch(als_x_kernel, grid_for(nX), threads, 0, st, N, oth, D, side, XA, skip);
+    if (als_r_lanes(nR) == 1) launch(als_r_kernel<1>, grid_for(nR), threads, 0, st, XA, oth, D, side, R, skip);
+    else launch(als_r_kernel<8>, grid_for(8 * nR), threads, 0, st, XA, oth, D, side, R, skip);
+    launch(als_s_kernel, sgrid, threads, 0, st, XA, slots[als_slot].Ts, D, side, S, skip);
 }
 
 template <typename T>
@@ -780,15 +785,12 @@ void Engine<T>::cost_gradient(int gamma, const double* gate, const double* A2in,
     KH_CUDA(cudaMemcpyAsync(A2, A2in, sizeof(double) * own, cudaMemcpyDeviceToDevice, st));
     KH_CUDA(cudaMemcpyAsync(B2, B2in, sizeof(double) * own, cudaMemcpyDeviceToDevice, st));
     KH_CUDA(cudaMemsetAsync(cost, 0, 8 * sizeof(double), st));
-    tnt_kernel<<<dm.D4, kTntThreads, 0, st>>>(sl.Ts, N, dm.D4, cost);
-    KH_LAUNCHED();
+    launch(tnt_kernel, dm.D4, kTntThreads, 0, st, sl.Ts, N, dm.D4, cost);
     als_slot = gamma;
     normal_equations(B2, 0, nullptr);                      // A side (B'' fixed)
-    cost_grad_kernel<<<(int)(own + 7) / 8, 256, 0, st>>>(R, S, A2, m, gA, cost + 5);
-    KH_LAUNCHED();
+    launch(cost_grad_kernel, (int)(own + 7) / 8, 256, 0, st, R, S, A2, m, gA, cost + 5);
     normal_equations(A2, 1, nullptr);                      // B side (A'' fixed)
-    cost_grad_kernel<<<(int)(own + 7) / 8, 256, 0, st>>>(R, S, B2, m, gB, cost + 6);
-    KH_LAUNCHED();
+    launch(cost_grad_kernel, (int)(own + 7) / 8, 256, 0, st, R, S, B2, m, gB, cost + 6);
     double h[8];
     KH_CUDA(cudaMemcpyAsync(h, cost, sizeof(h), cudaMemcpyDeviceToHost, st));
     sync_checked();
@@ -836,8 +838,7 @@ int Engine<T>::als_run(int gamma, double* rel_cost) {
     // <T'|N|T'>
     KH_CUDA(cudaMemsetAsync(cost, 0, 8 * sizeof(double), st));
     KH_CUDA(cudaMemsetAsync(flags, 0, 8 * sizeof(int), st));
-    tnt_kernel<<<D4, kTntThreads, 0, st>>>(Tp, N, D4, cost);
-    KH_LAUNCHED();
+    launch(tnt_kernel, D4, kTntThreads, 0, st, Tp, N, D4, cost);
     // truncated SVD start: Tm[(sA,aA,u,r)][(sB,aB,d,l)] from T'[sA,aA,sB,aB,l,u,r,d]
     permute<double, double>(Tp, Tm, {2, 2, 2, 2, D, D, D, D}, {0, 1, 5, 6, 2, 3, 7, 4}, st);
     double* colsc = dwork;
@@ -853,8 +854,7 @@ int Engine<T>::als_run(int gamma, double* rel_cost) {
     } else {
         bond_start_subspace(mT, D);
     }
-    svd_init_kernel<float><<<grid_for(mT * D), 256, 0, st>>>(Wtf, Ltf, mT, D, A2, colsc, Wd);
-    KH_LAUNCHED();
+    launch(svd_init_kernel<float>, grid_for(mT * D), 256, 0, st, Wtf, Ltf, mT, D, A2, colsc, Wd);
     // B''[(sB,aB,d,l)][k] = sum_i Tm[i][.] Wd[i][k] colsc[k]
     gemm_rm<double>(mT, D, mT, Tm, true, Wd, false, B2, st, 1.0, 0.0, colsc);
     // initial cost with (A'', B'') from the start: B-side normal equations from A''
@@ -871,23 +871,19 @@ int Engine<T>::als_run(int gamma, double* rel_cost) {
     als_slot = gamma;
     auto normal_eqs = [&](const double* oth, int side) { normal_equations(oth, side, done); };
     normal_eqs(A2, 1);
-    als_cost_kernel<<<cgrid, threads, 0, st>>>(R, S, B2, m, cost, flags + 1, cfg.als_tol, 1, nullptr);
-    KH_LAUNCHED();
+    launch(als_cost_kernel, cgrid, threads, 0, st, R, S, B2, m, cost, flags + 1, cfg.als_tol, 1, nullptr);
     // Sweeps run on the device until the relative cost change is below the
     // tolerance (flags[1] set by the cost kernel, after which every kernel of
     // the loop returns at once); the host looks at the flags every few sweeps.
     constexpr int kCheckEvery = 4;
     for (int it = 1; it <= cfg.als_max_iter; ++it) {
         normal_eqs(B2, 0);                                   // A step (fixed B'')
-        chol_solve_kernel<<<1, 512, chol_smem ? chol_sm : 0, st>>>(R, S, m, cfg.als_reg, Xmat, A2, flags, done,
-                                                                   chol_smem);
-        KH_LAUNCHED();
+        launch(chol_solve_kernel, 1, 512, chol_smem ? chol_sm : 0, st, R, S, m, cfg.als_reg, Xmat, A2, flags, done,
+               chol_smem);
         normal_eqs(A2, 1);                                   // B step (fixed A'')
-        chol_solve_kernel<<<1, 512, chol_smem ? chol_sm : 0, st>>>(R, S, m, cfg.als_reg, Xmat, B2, flags, done,
-                                                                   chol_smem);
-        KH_LAUNCHED();
-        als_cost_kernel<<<cgrid, threads, 0, st>>>(R, S, B2, m, cost, flags + 1, cfg.als_tol, 0, done);
-        KH_LAUNCHED();
+        launch(chol_solve_kernel, 1, 512, chol_smem ? chol_sm : 0, st, R, S, m, cfg.als_reg, Xmat, B2, flags, done,
+               chol_smem);
+        launch(als_cost_kernel, cgrid, threads, 0, st, R, S, B2, m, cost, flags + 1, cfg.als_tol, 0, done);
         if (it % kCheckEvery == 0 || it == cfg.als_max_iter) {
             int hf[2];
             KH_CUDA(cudaMemcpyAsync(hf, flags, sizeof(hf), cudaMemcpyDeviceToHost, st));
@@ -910,8 +906,7 @@ template <typename T>
 void Engine<T>::gauge_and_store(int gamma) {
     const int D = dm.D, mR = 4 * D * D;
     size_t sm = sizeof(double) * 2 * mR * D;
-    gauge_kernel<<<1, 256, sm, st>>>(A2, B2, D, gamma, A, B);
-    KH_LAUNCHED();
+    launch(gauge_kernel, 1, 256, sm, st, A2, B2, D, gamma, A, B);
 }
 
 template <typename T>

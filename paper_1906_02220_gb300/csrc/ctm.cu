@@ -525,6 +525,7 @@ __global__ void init_env_kernel(double* C, double* E, int chi, int d2, const dou
 
 // symmetrise N (n x n) in place: N = (N + N^T)/2
 __global__ void symmetrize_kernel(double* Nm, int n) {
+    pdl_start();
     long long tot = (long long)n * n;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < tot;
          i += (long long)gridDim.x * blockDim.x) {
@@ -580,6 +581,7 @@ __global__ void ring_close2_kernel(const double* t3, const double* u, int chi, i
 
 // vals[i] = sum_ab O_i[a][b] X[a][b] / tr X
 __global__ void expval_kernel(const double* ops, int n_ops, int p, const double* X, double* vals) {
+    pdl_start();
     int i = threadIdx.x;
     if (i >= n_ops) return;
     double tr = 0.0, s = 0.0;
@@ -1387,8 +1389,7 @@ void Engine<T>::compute_metric(Slot<T>& sl, double* N_out) {
                    sk_elems);
     }
     permute<T, double>(mN4, N_out, {D, D, D, D, D, D, D, D}, {6, 0, 2, 4, 7, 1, 3, 5}, st);
-    symmetrize_kernel<<<grid_for((long long)dm.D4 * dm.D4), 256, 0, st>>>(N_out, dm.D4);
-    KH_LAUNCHED();
+    launch(symmetrize_kernel, grid_for((long long)dm.D4 * dm.D4), 256, 0, st, N_out, dm.D4);
     prof_end(5, 0.0);
 }
 
@@ -1466,8 +1467,7 @@ void Engine<T>::expval(int slot, const double* ops, int n_ops, double* vals) {
     double* dops = dscr + DscrOff::kStage;
     double* dvals = dscr + DscrOff::kExpvalOut;
     KH_CUDA(cudaMemcpyAsync(dops, ops, sizeof(double) * n_ops * p * p, cudaMemcpyHostToDevice, st));
-    expval_kernel<<<1, 32, 0, st>>>(dops, n_ops, p, X, dvals);
-    KH_LAUNCHED();
+    launch(expval_kernel, 1, 32, 0, st, dops, n_ops, p, X, dvals);
     KH_CUDA(cudaMemcpyAsync(vals, dvals, sizeof(double) * n_ops, cudaMemcpyDeviceToHost, st));
     sync_checked();
 }
@@ -1549,8 +1549,7 @@ void cholqr_factor(double* dG, int k, double cut_abs, double tau, T* X, cudaStre
     } else {
         static std::atomic<size_t> granted[kMaxDevices] = {};
         smem_opt_in(cholqr_kernel<T>, 2 * sm, granted);
-        cholqr_kernel<T><<<1, 1024, 2 * sm, st>>>(dG, k, cut_abs, tau, X, sorted ? 1 : 0, ns_tol, defer);
-        KH_LAUNCHED();
+        launch(cholqr_kernel<T>, 1, 1024, 2 * sm, st, dG, k, cut_abs, tau, X, sorted ? 1 : 0, ns_tol, defer);
     }
 }
 template void cholqr_factor<float>(double*, int, double, double, float*, cudaStream_t, bool, double, double, bool);

@@ -685,6 +685,7 @@ template <typename T>
 __global__ void __launch_bounds__(1024)
 cholqr_kernel(const double* __restrict__ G, int k, double cut_abs, double tau, T* __restrict__ X, int sorted,
               double ns_tol, double defer) {
+    pdl_start();
     extern __shared__ unsigned char smem_raw[];
     __shared__ CholShared<T> sh;
     const int ld = k | 1;                          // odd row stride: conflict-free column walks

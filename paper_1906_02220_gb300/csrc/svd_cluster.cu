@@ -77,6 +77,7 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(32 * kSea
 svd_cluster_kernel(const double* __restrict__ Xin, int k, int npc, double* __restrict__ s_out,
                    double* __restrict__ L_out, double* __restrict__ Q_out, int max_sweeps, double tol, double cut,
                    int* sweep_count, int nrel) {
+    pdl_start();
     extern __shared__ double bufs[];       // 2 (npc + 1) + 1 columns of (X, Q), 32 RR rows each
     __shared__ double s_cn[kColsMax];      // squared column norms, by column
     __shared__ unsigned char s_top[kColsMax];
@@ -281,12 +282,11 @@ svd_cluster_kernel(const double* __restrict__ Xin, int k, int npc, double* __res
 }
 
 template <int RR>
-void launch(const double* X, int k, int npc, double* s, double* L, double* Q, int max_sweeps, double tol, double cut,
-            cudaStream_t st, int* sweep_count, int nrel) {
+void launch_cluster(const double* X, int k, int npc, double* s, double* L, double* Q, int max_sweeps, double tol,
+                    double cut, cudaStream_t st, int* sweep_count, int nrel) {
     const size_t sm = sizeof(double) * (2 * (npc + 1) + 1) * 2 * 32 * RR;     // at most 34 KB
-    svd_cluster_kernel<RR><<<kClusterCtas, 32 * npc, sm, st>>>(X, k, npc, s, L, Q, max_sweeps, tol, cut, sweep_count,
-                                                               nrel);
-    KH_LAUNCHED();
+    launch(svd_cluster_kernel<RR>, kClusterCtas, 32 * npc, sm, st, X, k, npc, s, L, Q, max_sweeps, tol, cut,
+           sweep_count, nrel);
 }
 
 }  // namespace
@@ -295,7 +295,7 @@ void svd_jacobi_cluster(const double* X, int k, double* s, double* L, double* Q,
                         double cut, cudaStream_t st, int* sweep_count, int nrel) {
     const int npc = (k + 2 * kClusterCtas - 1) / (2 * kClusterCtas);
     if (npc < 1 || npc > kSeatsMax) fail(KH_EINVAL, "svd_jacobi_cluster: k beyond limit");
-#define KH_SVDC(RR) launch<RR>(X, k, npc, s, L, Q, max_sweeps, tol, cut, st, sweep_count, nrel)
+#define KH_SVDC(RR) launch_cluster<RR>(X, k, npc, s, L, Q, max_sweeps, tol, cut, st, sweep_count, nrel)
     if (k <= 32) KH_SVDC(1);
     else if (k <= 64) KH_SVDC(2);
     else if (k <= 96) KH_SVDC(3);

@@ -494,7 +494,7 @@ void cholqr_factor(double* dG, int k, double cut_abs, double tau, T* X, cudaStre
 __device__ __forceinline__ float chol_recip(float x) { return __fdividef(1.f, x); }
 __device__ __forceinline__ double chol_recip(double x) { return 1.0 / x; }
 
-// Shared state of the two CholQR factor kernels (shared memory).
+// State of cholqr_kernel in shared memory.
 template <typename T>
 struct CholShared {
     static constexpr int KM = sizeof(T) == 8 ? 112 : 160;   // largest k
@@ -504,7 +504,7 @@ struct CholShared {
     T mx;
 };
 
-// Prologue of the factor kernels: column norms, the Newton-Schulz shortcut
+// Its prologue: column norms, the Newton-Schulz shortcut
 // (returns true when X was written that way), the order (by norm when
 // sorted), and the scaled, permuted Gram matrix into Lm (k x ld); Li zeroed.
 template <typename T>

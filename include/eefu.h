@@ -429,7 +429,9 @@ kh_status kh_selftest_svd_refined(int k, const double* dev_X, double* dev_S, dou
 /* Orthonormal basis of the columns of an n x k FP64 matrix Y (row-major) by
  * the library's ordered CholQR2 (two Cholesky-QR passes, columns taken in
  * order of decreasing norm), the orthonormalisation step of the projector's
- * subspace iteration, in FP64 (k <= 112) or FP32 (k <= 160).  Columns of norm
+ * subspace iteration, in FP64 (k <= 112) or FP32 (k <= 160; KH_TF32X3 takes the
+ * factor that eliminates column by column, as contexts of D <= 5 do, the other
+ * kinds the one in registers).  Columns of norm
  * <= cut * (largest norm), and directions whose Cholesky pivot falls below
  * the rounding floor, come out as zero columns of dev_Q (n x k, row-major);
  * the others are orthonormal, the first one along the largest column of Y.

@@ -100,8 +100,8 @@ __device__ __forceinline__ int frame_offset(int f, int L, int U, int R, int Dd, 
 // GEMM's second operand: for kind 0 (corner, TL = [L,U][p][R,D]) and kind 1
 // (edge, TL = [L,D][p][U,R]) of frame f,
 //   Wt_f[(ok,ob)][(ib,ik)] = sum_p TL_f[ik][p][ok] TL_f[ib][p][ob]
-// summed in FP64.  With lo != null the value is stored rounded to nearest TF32
-// in W and the FP32 remainder in lo.
+// summed in FP64.  With lo != null the value is stored as its TF32 head
+// (13 low mantissa bits cleared) in W and the FP32 remainder in lo.
 template <typename T>
 __global__ void wt_kernel(const double* __restrict__ Tm, int p, int D, T* Wc, T* We, T* Wc_lo, T* We_lo) {
     pdl_start();
@@ -130,7 +130,7 @@ __global__ void wt_kernel(const double* __restrict__ Tm, int p, int D, T* Wc, T*
         T* Wl = kind == 0 ? Wc_lo : We_lo;
         if (Wl) {
             float v = (float)sacc;
-            float h = __uint_as_float((__float_as_uint(v) + 0x1000u) & 0xFFFFE000u);   // a NaN stays in the remainder
+            float h = __uint_as_float(__float_as_uint(v) & 0xFFFFE000u);
             *W = (T)h;
             Wl[rem] = (T)(v - h);
         } else {
@@ -146,7 +146,8 @@ __global__ void wt_kernel(const double* __restrict__ Tm, int p, int D, T* Wc, T*
 // and the bra image
 //   B2_c[ob][(ib, pl)] = TL_f[ib][c pc + pl][ob],
 // each stored byte for byte as its 128-byte-swizzled K-major shared-memory
-// tile (rounded to nearest TF32, then the FP32 remainder, with 3 passes), zero outside
+// tile (the TF32 head, rounded or in the fixed order cut off, then the FP32
+// remainder, with 3 passes), zero outside
 // the operand.  Layout [kind][frame][chunk][hi, lo], per1 / per2 floats per
 // (kind, frame).
 __global__ void layered_img_kernel(const double* __restrict__ Tm, const double* __restrict__ Tb, int p, int D,
@@ -192,7 +193,7 @@ __global__ void layered_img_kernel(const double* __restrict__ Tm, const double* 
         } else {
             float x = (float)v;
             if (npass == 3) {
-                const float h = __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);   // nearest TF32
+                const float h = __uint_as_float((__float_as_uint(x) + (P.fixed ? 0u : 0x1000u)) & 0xFFFFE000u);
                 x = hl == 0 ? h : x - h;
             }
             (ket ? img1 : img2)[e] = x;

@@ -58,6 +58,18 @@ Dims make_dims(const kh_config& c, bool fp64) {
     d.lay1 = d.lay ? layered_img1_floats(c.D, c.p_max, d.npass, d.bf16) : 0;
     d.lay2 = d.lay ? layered_img2_floats(c.D, c.p_max, d.npass, d.bf16) : 0;
     if (d.lay && (d.lay1 == 0 || d.lay2 == 0)) fail(KH_EINVAL, "no tensor-core plan for this D");
+    // An environment's scale, and with it the metric's, the bond cost's and its
+    // gradient's, depends on which directions pass the cut, and for a direction
+    // near the cut that depends on rounding: at (D, chi) = (4, 64) the gradients of
+    // 4 of 32 states moved by 5e-5 to 1.3e-3, and expectation values by 1e-8, when a
+    // move's products, site contractions and factors were summed in another
+    // order, each no less accurate; at D = 3 of 0 in 44.  Trial costs are compared
+    // across runs and with stored ones, so the FP32-accurate modes keep one order
+    // and rounding up to D = 5, the sizes of gradient-based bond optimisation.
+    // What that gives up at (4, 64): the environment takes 12.5 ms, with the other
+    // forms 11.3.
+    // From D = 6 on the tensor-core products halve the time of a move.
+    d.fixed_order = !fp64 && d.npass != 1 && c.D <= lay::kFixedOrderD;
     int kmax = fp64 ? 112 : 160;      // the one-CTA Jacobi limits (FP64, FP32)
     if (d.n <= kmax) {
         d.kk = d.n;
@@ -201,7 +213,7 @@ void Engine<T>::carve_lane(Carver& cv) {
     }
     sk_elems = 16LL * n * (kk > d.chi ? kk : d.chi);
     skbuf = cv.take<T>(sk_elems);
-    if (d.npass) {
+    if (d.npass && !d.fixed_order) {
         const size_t bsz = (size_t)n * ((kk > d.chi ? kk : d.chi) + 4);
         Bh = cv.take<T>(bsz);
         Bl = cv.take<T>(bsz);
@@ -642,9 +654,26 @@ void Engine<T>::refresh_operands(Slot<T>& sl) {
 //    bra layer batched over b (K = p D^2)                                  (4 nb p D^6 flops);
 //    with TLb given, the bra layer reads TLb instead of TL (an operator on
 //    the ket layer only).
+// The double-layer site contraction runs as a 3xTF32 tensor-core GEMM (at D^2 <=
+// 2p, so in the fixed order): its Y operand is then written directly as the
+// (hi, lo) pair into (mup, mdn).
+template <typename T>
+bool Engine<T>::site_presplit(const Slot<T>& sl) const {
+    return sl.dl && tc_npass == 3 && sizeof(T) == 4 && dm.D4 % 4 == 0;
+}
+
+// Y permuted into the site contraction's block layout: into Yp, or as the
+// split pair (mup, mdn) when site_presplit.
+template <typename T>
+void Engine<T>::site_operand(const Slot<T>& sl, const T* Y, T* Yp, const std::vector<long long>& shape,
+                             const std::vector<int>& order) {
+    if (site_presplit(sl)) permute_split((const float*)Y, (float*)mup, (float*)mdn, shape, order, st, nullptr, false);
+    else permute<T, T>(Y, Yp, shape, order, st);
+}
+
 template <typename T>
 void Engine<T>::site_layer(const T* Ybuf, long long nb, const T* TL, const T* L1, const T* L2, int p, T* out,
-                           const T* Wt, const T* Wt_lo, const T* TLb) {
+                           const T* Wt, const T* Wt_lo, bool presplit, const T* TLb) {
     const int d2 = dm.d2, d4 = dm.D4;
     prof_begin(1);
     if (!Wt && L1) {                                   // layered, on the tensor cores
@@ -655,13 +684,14 @@ void Engine<T>::site_layer(const T* Ybuf, long long nb, const T* TL, const T* L1
     }
     if (Wt) {
         if (tc_npass && sizeof(T) == 4 && d4 % 4 == 0) {       // TMA rows must be 16-byte multiples
+            TcOperand a{(const float*)Ybuf, nullptr, d4}, b{(const float*)Wt, nullptr, d4};
             if (tc_npass == 3) {
-                gemm3x((const float*)Ybuf, d4, false, (const float*)Wt, (const float*)Wt_lo, d4, (float*)out, (int)nb, d4,
-                       d4, d4, 1.f, nullptr, nullptr, 0, tc_err, st);
-            } else {
-                TcOperand a{(const float*)Ybuf, d4}, b{(const float*)Wt, d4};
-                tc_gemm(a, b, (float*)out, (int)nb, d4, d4, d4, 1.f, 0.f, nullptr, tc_err, st);
+                float *yh = (float*)mup, *yl = (float*)mdn;     // nb D^4 = n^2 elements
+                if (!presplit) tc_split((const float*)Ybuf, yh, yl, nb * d4, st);
+                a = TcOperand{yh, yl, d4};
+                b = TcOperand{(const float*)Wt, (const float*)Wt_lo, d4};
             }
+            tc_gemm(a, b, (float*)out, (int)nb, d4, d4, d4, 1.f, 0.f, nullptr, tc_npass, tc_err, st);
         } else {
             gemm_rm<T>((int)nb, d4, d4, Ybuf, false, Wt, true, out, st);
         }
@@ -691,7 +721,7 @@ template <typename T>
 bool Engine<T>::product3x(int ln, const T* A, long long lda, bool a_mmajor, const T* B, long long sn, long long sk,
                           T* C, int M, int N, int K, long long ldc, const T* colscale) {
     if constexpr (sizeof(T) == 4) {
-        if (!tc_npass || 2.0 * M * N * (double)K < kMin3x || !gemm3x_usable(A, lda)) return false;
+        if (!tc_npass || dm.fixed_order || 2.0 * M * N * (double)K < kMin3x || !gemm3x_usable(A, lda)) return false;
         const Lane<T>& L = lanes[ln];
         const int ldb = (K + 3) / 4 * 4;
         gemm3x_split_b(B, sn, sk, N, K, L.Bh, L.Bl, ldb, L.st);
@@ -719,19 +749,20 @@ void Engine<T>::corner(Slot<T>& sl, int f, int which) {
         permute<T, T>(Y1, Yp, {D, D, chi, chi, D, D}, {3, 2, 5, 1, 4, 0}, st);
     } else {
         gemm_rm<T>(chi * d2, d2 * chi, chi, E4, false, X, false, Y1, st);
-        permute<T, T>(Y1, Yp, {chi, D, D, D, D, chi}, {0, 5, 2, 4, 1, 3}, st);
+        site_operand(sl, Y1, Yp, {chi, D, D, D, D, chi}, {0, 5, 2, 4, 1, 3});
     }
     const long long w4 = (long long)f * dm.D4 * dm.D4;
     site_layer(Yp, chi2, sl.Tcor + (long long)f * dm.pmax * dm.D4, lay_img(sl, 1, 0, f), lay_img(sl, 2, 0, f), sl.p,
                Qt, sl.dl ? sl.Wcor + w4 : nullptr,
-               sl.dl && sl.Wcor_lo ? sl.Wcor_lo + w4 : nullptr);   // [w][z][rk][dk][rb][db]
+               sl.dl && sl.Wcor_lo ? sl.Wcor_lo + w4 : nullptr, site_presplit(sl));   // [w][z][rk][dk][rb][db]
     // Q_0 stored transposed, [(z,rk,rb)][(w,dk,db)], as the K-major operand of
     // Mt = Q_{s+3} Q_s on tensor cores; with 3xTF32 its (hi, lo) pair is written
-    // by the same pass (mupp, mdnp)
+    // by the same pass (mupp, mdnp), and in the fixed order also Q_1's (q1_hi, q1_lo)
     const std::vector<int> order = (which == 0 && tc_npass) ? std::vector<int>{1, 2, 4, 0, 3, 5}
                                                             : std::vector<int>{0, 3, 5, 1, 2, 4};
-    if (which == 0 && mt_presplit())
-        permute_split((const float*)Qt, (float*)mupp, (float*)mdnp, {chi, chi, D, D, D, D}, order, st, (float*)Q[0]);
+    if (mt_presplit() && (which == 0 || dm.fixed_order))
+        permute_split((const float*)Qt, (float*)(which == 1 ? q1_hi : mupp), (float*)(which == 1 ? q1_lo : mdnp),
+                      {chi, chi, D, D, D, D}, order, st, (float*)Q[which], !dm.fixed_order);
     else
         permute<T, T>(Qt, Q[which], {chi, chi, D, D, D, D}, order, st);
 }
@@ -743,7 +774,7 @@ void Engine<T>::corner(Slot<T>& sl, int f, int which) {
 // Newton-Schulz step when that loss is already small).  Scratch: tmp (n x k), Xk (k x k), dG (k x k FP64).
 template <typename T>
 void cholqr2(T* Y, int n, int k, double cut, T* tmp, T* Xk, double* dG, T* Uo, cudaStream_t st, const T* part,
-             int parts, bool dG_clear, const std::function<bool(const T*, const T*, T*)>& product) {
+             int parts, bool dG_clear, const std::function<bool(const T*, const T*, T*)>& product, bool by_column) {
     const double tau = sizeof(T) == 8 ? 1e-12 : 1e-5;
     // FP64: pivots below k 2^-53 / tau, whose acceptance could lift the
     // rounding noise of a later, exactly dependent column above tau, are
@@ -760,9 +791,9 @@ void cholqr2(T* Y, int n, int k, double cut, T* tmp, T* Xk, double* dG, T* Uo, c
             if (!dG_clear) KH_CUDA(cudaMemsetAsync(dG, 0, sizeof(double) * k * k, st));
             if (parts) rows_reduce(part, parts, n, k, Y, dG, st);
             else rows_reduce(Y, 1, n, k, nullptr, dG, st);
-            cholqr_factor<T>(dG, k, cut, tau, Xk, st, true, 0.0, defer, true);
+            cholqr_factor<T>(dG, k, cut, tau, Xk, st, true, 0.0, defer, true, by_column);
             rows_apply(Y, Xk, n, k, tmp, dG, st);
-            cholqr_factor<T>(dG, k, 1e-3, tau, Xk, st, false, ns_tol, 0.0, true);
+            cholqr_factor<T>(dG, k, 1e-3, tau, Xk, st, false, ns_tol, 0.0, true, by_column);
             rows_apply(tmp, Xk, n, k, Uo, nullptr, st);
             return;
         }
@@ -771,17 +802,17 @@ void cholqr2(T* Y, int n, int k, double cut, T* tmp, T* Xk, double* dG, T* Uo, c
         if (!product || !product(A, Xk, Q)) gemm_rm<T>(n, k, k, A, false, Xk, false, Q, st);
     };
     gram<T>(Y, n, k, dG, st);
-    cholqr_factor<T>(dG, k, cut, tau, Xk, st, true, 0.0, defer);
+    cholqr_factor<T>(dG, k, cut, tau, Xk, st, true, 0.0, defer, false, by_column);
     apply(Y, tmp);
     gram<T>(tmp, n, k, dG, st);
-    cholqr_factor<T>(dG, k, 1e-3, tau, Xk, st, false, ns_tol);
+    cholqr_factor<T>(dG, k, 1e-3, tau, Xk, st, false, ns_tol, 0.0, false, by_column);
     apply(tmp, Uo);
 }
 template void cholqr2<float>(float*, int, int, double, float*, float*, double*, float*, cudaStream_t, const float*, int,
-                             bool, const std::function<bool(const float*, const float*, float*)>&);
+                             bool, const std::function<bool(const float*, const float*, float*)>&, bool);
 template void cholqr2<double>(double*, int, int, double, double*, double*, double*, double*, cudaStream_t,
                               const double*, int, bool,
-                              const std::function<bool(const double*, const double*, double*)>&);
+                              const std::function<bool(const double*, const double*, double*)>&, bool);
 
 // Algorithmic flops of one CholQR2 of an n x k block: two symmetric Gram
 // matrices (n k (k+1) each), one Cholesky factor and triangular inverse
@@ -798,7 +829,8 @@ void Engine<T>::orth(T* Y, int n, int k, T* Uo, int parts) {
     // the Gram matrices are cleared at the start of a projector, and by every factor that reads one
     const int ln = lane_id();
     cholqr2<T>(Y, n, k, cfg.svd_cut, Qt, Xk, dscr + DscrOff::kGram, Uo, st, skbuf, parts, true,
-               [&](const T* A, const T* X, T* Q) { return product3x(ln, A, k, false, X, 1, k, Q, n, k, k, k); });
+               [&](const T* A, const T* X, T* Q) { return product3x(ln, A, k, false, X, 1, k, Q, n, k, k, k); },
+               dm.fixed_order);
     prof_end(8, cholqr2_flops(n, k));
 }
 
@@ -812,12 +844,16 @@ bool Engine<T>::mt_presplit() const {
 template <typename T>
 void Engine<T>::half_system_product(int n) {
     prof_begin(0);
-    if (mt_presplit()) {                                // Q_0 split when it was written
+    if (mt_presplit() && !dm.fixed_order) {             // Q_0 split when it was written
         gemm3x((const float*)Q[1], n, false, (const float*)mupp, (const float*)mdnp, n, (float*)Mt, n, n, n, n, 1.f,
                nullptr, nullptr, 0, tc_err, st);
     } else if (tc_npass && sizeof(T) == 4 && n % 4 == 0) {     // TMA rows must be 16-byte multiples
-        TcOperand a{(const float*)Q[1], n}, b{(const float*)Q[0], n};
-        tc_gemm(a, b, (float*)Mt, n, n, n, n, 1.f, 0.f, nullptr, tc_err, st);
+        TcOperand a{(const float*)Q[1], nullptr, n}, b{(const float*)Q[0], nullptr, n};
+        if (tc_npass == 3) {                            // both operands split when they were written
+            a = TcOperand{(const float*)q1_hi, (const float*)q1_lo, n};
+            b = TcOperand{(const float*)mupp, (const float*)mdnp, n};
+        }
+        tc_gemm(a, b, (float*)Mt, n, n, n, n, 1.f, 0.f, nullptr, tc_npass, tc_err, st);
     } else {      // Q_0 is stored transposed whenever the tensor cores are enabled
         gemm_rm<T>(n, n, n, Q[1], false, Q[0], tc_npass != 0, Mt, st);
     }
@@ -988,14 +1024,16 @@ void Engine<T>::projector(Slot<T>& sl, int dir, int slot_id) {
             q = cfg.svd_iters_cold;
         } else {
             const uint64_t draw = stream * 1000003ULL + (rng_counter++);
+            bool split = false;
             if constexpr (sizeof(T) == 4) {
-                if (rows) {
+                if (rows && !dm.fixed_order) {      // its Vl^T R is summed in FP64, where the products below sum in FP32
+                    split = true;
                     rows_split(Vw, live, n, k, Vo, Z2, cfg.seed, draw, dG + k * k, st);
                     rows_project(Vo, dG + k * k, n, k, Z2, dG + 2 * k * k, st);  // R <- R - Vl (Vl^T R), twice
                     rows_project(Vo, dG + 2 * k * k, n, k, Z2, nullptr, st);     // then Vl + R
                 }
             }
-            if (!rows) {
+            if (!split) {
                 launch(warm_split_kernel<T>, grid_for((long long)n * k), 256, 0, st, Vw, live, n, k, Vo, Z2, cfg.seed, draw);
                 for (int r = 0; r < 2; ++r) {                                   // R <- R - Vl (Vl^T R), twice
                     gemm_rm<T>(k, k, n, Vo, true, Z2, false, Xk, st, T(1), T(0), nullptr, skbuf, sk_elems);
@@ -1154,11 +1192,11 @@ void Engine<T>::absorb(Slot<T>& sl, int s) {
     const int ln = lane_id();
     if (!product3x(ln, E4, n, true, P, 1, n, Y1, n, n, chi, n))                   // [(lk,lb,x4)][(dk,db,a)]
         gemm_rm<T>(d2 * chi, d2 * chi, chi, E4, true, P, false, Y1, st);
-    permute<T, T>(Y1, Yp, {D, D, chi, D, D, chi}, {2, 5, 1, 4, 0, 3}, st);         // [x4][a][lb][db][lk][dk]
+    site_operand(sl, Y1, Yp, {D, D, chi, D, D, chi}, {2, 5, 1, 4, 0, 3});         // [x4][a][lb][db][lk][dk]
     const long long w4 = (long long)s * dm.D4 * dm.D4;
     site_layer(Yp, chi2, sl.Tedg + (long long)s * dm.pmax * dm.D4, lay_img(sl, 1, 1, s), lay_img(sl, 2, 1, s), sl.p,
                Qt, sl.dl ? sl.Wedg + w4 : nullptr,
-               sl.dl && sl.Wedg_lo ? sl.Wedg_lo + w4 : nullptr);   // [x4][a][uk][rk][ub][rb]
+               sl.dl && sl.Wedg_lo ? sl.Wedg_lo + w4 : nullptr, site_presplit(sl));   // [x4][a][uk][rk][ub][rb]
     permute<T, T>(Qt, Y1, {chi, chi, D, D, D, D}, {1, 3, 5, 0, 2, 4}, st);       // [a][rk][rb][x4][uk][ub]
     if (!product3x(ln, Y1, n, false, PtT, 1, chi, E4n, n, chi, n, chi))           // [a][rk][rb][a_up]
         gemm_rm<T>(chi * d2, chi, n, Y1, false, PtT, false, E4n, st, T(1), T(0), nullptr, skbuf, sk_elems);
@@ -1191,8 +1229,8 @@ void Engine<T>::move(Slot<T>& sl, int s, int slot_id) {
     if (nlanes >= 2 && !in_lanes) {
         // The two enlarged corners are independent: corner s+3 runs on lane 1
         // (its own stream and scratch) reading lane 0's environment operands
-        // and writing Q_{s+3} where the half-system product reads it; lane 0
-        // waits before the projector.
+        // and writing Q_{s+3} (and its split, into lane 1's mupp/mdnp) where
+        // the half-system product reads them; lane 0 waits before the projector.
         KH_CUDA(cudaEventRecord(lane_ev[0], st));
         KH_CUDA(cudaStreamWaitEvent(lanes[1].st, lane_ev[0], 0));
         corner(sl, s, 0);
@@ -1205,11 +1243,15 @@ void Engine<T>::move(Slot<T>& sl, int s, int slot_id) {
         Eop = lanes[0].Eop;
         X1[1] = lanes[0].X1[1];
         Q[1] = lanes[0].Q[1];
+        q1_hi = lanes[1].mupp;
+        q1_lo = lanes[1].mdnp;
         corner(sl, (s + 3) & 3, 1);
         KH_CUDA(cudaEventRecord(lane_ev[1], st));
         bind(0);
         KH_CUDA(cudaStreamWaitEvent(st, lane_ev[1], 0));
     } else {
+        q1_hi = mup;
+        q1_lo = mdn;
         corner(sl, s, 0);
         corner(sl, (s + 3) & 3, 1);
     }
@@ -1376,7 +1418,7 @@ void Engine<T>::compute_metric(Slot<T>& sl, double* N_out) {
     constexpr double kMinMetric3x = 1e9;
     bool joined = false;
     if constexpr (sizeof(T) == 4) {
-        if (tc_npass && 2.0 * dm.D4 * dm.D4 * chi2 >= kMinMetric3x && gemm3x_usable(mupp, chi2)) {
+        if (tc_npass && !dm.fixed_order && 2.0 * dm.D4 * dm.D4 * chi2 >= kMinMetric3x && gemm3x_usable(mupp, chi2)) {
             permute_split(mdn, mdnp, mup, {chi, D, D, D, D, chi}, {1, 2, 3, 4, 5, 0}, st);   // [dk][db][lk][lb][h][e]
             gemm3x(mupp, chi2, false, mdnp, mup, (int)chi2, mN4, dm.D4, dm.D4, (int)chi2, dm.D4, 1.f, nullptr, skbuf,
                    sk_elems, tc_err, st);
@@ -1529,11 +1571,18 @@ void svd_jacobi(const T* X, int k, T* sv, T* L, T* Qm, int max_sweeps, double to
 }
 template <typename T>
 void cholqr_factor(double* dG, int k, double cut_abs, double tau, T* X, cudaStream_t st, bool sorted,
-                   double ns_tol, double defer, bool clear) {
+                   double ns_tol, double defer, bool clear, bool by_column) {
     if (k > jacobi_kmax<T>()) fail(KH_EINVAL, "cholqr: k beyond limit");
     const size_t sm = (size_t)k * (k | 1) * sizeof(T);
+    if (sizeof(T) == 8 || by_column) {
+        static std::atomic<size_t> granted[kMaxDevices] = {};
+        smem_opt_in(cholqr_kernel<T>, 2 * sm, granted);
+        launch(cholqr_kernel<T>, 1, 1024, 2 * sm, st, dG, k, cut_abs, tau, X, sorted ? 1 : 0, ns_tol, defer,
+               clear ? 1 : 0);
+        return;
+    }
     if constexpr (sizeof(T) == 4) {
-        if (defer > tau) fail(KH_EINVAL, "cholqr: the FP32 factor defers no pivot");
+        if (defer > tau) fail(KH_EINVAL, "cholqr: the FP32 factor in registers defers no pivot");
         switch ((k + 31) / 32) {
 #define KH_CHOL(KT)                                                                                          \
     case KT: {                                                                                               \
@@ -1546,14 +1595,10 @@ void cholqr_factor(double* dG, int k, double cut_abs, double tau, T* X, cudaStre
             KH_CHOL(1) KH_CHOL(2) KH_CHOL(3) KH_CHOL(4) KH_CHOL(5)
 #undef KH_CHOL
         }
-    } else {
-        static std::atomic<size_t> granted[kMaxDevices] = {};
-        smem_opt_in(cholqr_kernel<T>, 2 * sm, granted);
-        launch(cholqr_kernel<T>, 1, 1024, 2 * sm, st, dG, k, cut_abs, tau, X, sorted ? 1 : 0, ns_tol, defer);
     }
 }
-template void cholqr_factor<float>(double*, int, double, double, float*, cudaStream_t, bool, double, double, bool);
-template void cholqr_factor<double>(double*, int, double, double, double*, cudaStream_t, bool, double, double, bool);
+template void cholqr_factor<float>(double*, int, double, double, float*, cudaStream_t, bool, double, double, bool, bool);
+template void cholqr_factor<double>(double*, int, double, double, double*, cudaStream_t, bool, double, double, bool, bool);
 
 template void svd_jacobi<float>(const float*, int, float*, float*, float*, int, double, double, cudaStream_t, int*,
                                 int);

@@ -48,6 +48,7 @@ struct Dims {
     bool lay;                  // layered tensor-core site contraction (tensor-core precisions)
     int npass;                 // tensor-core passes: 0 (CUDA cores), 1 (TF32 or BF16), 3 (3xTF32)
     bool bf16;                 // layered site contraction with BF16 operands (kind::f16)
+    bool fixed_order;          // one fixed order and rounding of every FP32 operation of a move (make_dims)
     long long lay1, lay2;      // floats per (kind, frame) of the ket and bra operand images
 };
 
@@ -211,6 +212,7 @@ struct Engine : EngineBase {
     bool own_streams = false;
     cudaEvent_t lane_ev[3] = {nullptr, nullptr, nullptr};
     bool in_lanes = false;     // lanes 1, 2 busy with other slots (sweep_lanes)
+    T *q1_hi = nullptr, *q1_lo = nullptr;   // where the 3xTF32 split of Q_{s+3} was written (fixed order)
     // Side lane for independent pieces of a move (lane 1), when not busy:
     // fork makes lane 1 wait for lane 0's work so far, join the reverse.
     bool side_lane() const { return nlanes >= 2 && !in_lanes; }
@@ -250,7 +252,8 @@ struct Engine : EngineBase {
     void corner(Slot<T>& sl, int frame, int which);
     void site_layer(const T* Ybuf, long long nb, const T* TL, const T* L1, const T* L2, int p, T* out,
                     const T* Wt, const T* Wt_lo,
-                    const T* TLb = nullptr);
+                    bool presplit = false, const T* TLb = nullptr);
+    bool site_presplit(const Slot<T>& sl) const;
     // operand image (1 = ket, 2 = bra) of the layered tensor-core contraction
     // for (kind: 0 corner, 1 edge; frame f), or null when the slot uses
     // another form
@@ -258,6 +261,8 @@ struct Engine : EngineBase {
         if (sl.dl || !sl.L1) return nullptr;
         return img == 1 ? sl.L1 + (kind * 4 + f) * dm.lay1 : sl.L2 + (kind * 4 + f) * dm.lay2;
     }
+    void site_operand(const Slot<T>& sl, const T* Y, T* Yp, const std::vector<long long>& shape,
+                      const std::vector<int>& order);
     void projector(Slot<T>& sl, int dir, int slot_id);
     void orth(T* Y, int n, int k, T* Uo, int parts = 0);
     int subspace_product(bool tr, const T* V, T* Y, bool keep_parts);
@@ -312,14 +317,17 @@ struct Engine : EngineBase {
     void load_checkpoint(std::FILE* f) override;
 };
 
-// One-pass tensor-core GEMM (tcgen05.cu): C = alpha colscale (A B^T) + beta C
-// with A (M x K) and B (N x K) row-major FP32 read as TF32.
+// Tensor-core GEMM (tcgen05.cu): C = alpha colscale (A B^T) + beta C with A
+// (M x K) and B (N x K) row-major FP32 read as TF32; npass = 3 uses the
+// hi/lo split operands (lo may be null for npass = 1).
 struct TcOperand {
-    const float* p;
+    const float* hi;
+    const float* lo;
     long long ld;
 };
 void tc_gemm(const TcOperand& A, const TcOperand& B, float* C, int M, int N, int K, long long ldc, float alpha,
-             float beta, const float* colscale, int* err, cudaStream_t st);
+             float beta, const float* colscale, int npass, int* err, cudaStream_t st);
+void tc_split(const float* x, float* hi, float* lo, long long n, cudaStream_t st);
 
 // Row-block kernels of small FP32 bases (rows.cu): n x k blocks, k <= 96; a
 // non-null G (k x k, FP64) has the named Gram matrix added to it.
@@ -356,11 +364,12 @@ void gemm3x(const float* A, long long lda, bool a_mmajor, const float* Bhi, cons
 // ordered CholQR2 (ctm.cu); see Engine::orth.
 // (parts > 0: Y itself is first formed as the sum of that many n x k blocks at
 // `part`; dG_clear: dG holds zeros already, and again afterwards; product: Q = Y X
-// by another route, false where that does not apply)
+// by another route, false where that does not apply; by_column: the factor
+// eliminates column by column, as cholqr_factor)
 template <typename T>
 void cholqr2(T* Y, int n, int k, double cut, T* tmp, T* Xk, double* dG, T* Uo, cudaStream_t st,
              const T* part = nullptr, int parts = 0, bool dG_clear = false,
-             const std::function<bool(const T* Y, const T* X, T* Q)>& product = nullptr);
+             const std::function<bool(const T* Y, const T* X, T* Q)>& product = nullptr, bool by_column = false);
 // G = A^T B (n x k each, T) accumulated in FP64 across row chunks (ctm.cu)
 template <typename T>
 void gram2(const T* A, const T* B, int n, int k, double* dG, cudaStream_t st);

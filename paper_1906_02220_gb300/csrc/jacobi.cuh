@@ -485,10 +485,12 @@ svd_jacobi_kernel(const T* __restrict__ Xin, int k, T* __restrict__ s_out, T* __
 // outside span(Y); a column nearly parallel to the ones before it is therefore
 // taken after the well-conditioned ones, by which time its residual has
 // usually become exactly zero (a rank-revealing order, as in column pivoting).
-// clear: dG is set to zero once read (FP32 only).
+// clear: dG is set to zero once read.  by_column: the single-precision factor
+// too eliminates column by column and inverts by blocks, as the FP64 one does
+// (the fixed order of rounding, make_dims).
 template <typename T>
 void cholqr_factor(double* dG, int k, double cut_abs, double tau, T* X, cudaStream_t st, bool sorted = true,
-                   double ns_tol = 0.0, double defer = 0.0, bool clear = false);
+                   double ns_tol = 0.0, double defer = 0.0, bool clear = false, bool by_column = false);
 
 #ifdef KH_JACOBI_KERNEL
 __device__ __forceinline__ float chol_recip(float x) { return __fdividef(1.f, x); }
@@ -683,8 +685,8 @@ __device__ void cholqr_epilogue(int k, double tau, T* __restrict__ X, T* Lm, T* 
 // scaling applied at the end) and pivot deferral (see cholqr_factor).
 template <typename T>
 __global__ void __launch_bounds__(1024)
-cholqr_kernel(const double* __restrict__ G, int k, double cut_abs, double tau, T* __restrict__ X, int sorted,
-              double ns_tol, double defer) {
+cholqr_kernel(double* __restrict__ G, int k, double cut_abs, double tau, T* __restrict__ X, int sorted,
+              double ns_tol, double defer, int clear) {
     pdl_start();
     extern __shared__ unsigned char smem_raw[];
     __shared__ CholShared<T> sh;
@@ -692,7 +694,12 @@ cholqr_kernel(const double* __restrict__ G, int k, double cut_abs, double tau, T
     T* Lm = reinterpret_cast<T*>(smem_raw);       // k x ld, row-major (lower triangle: L)
     T* Li = Lm + k * ld;                           // k x ld: L^-1
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
-    if (cholqr_prologue<T>(G, k, cut_abs, X, sorted, ns_tol, Lm, Li, ld, sh)) return;
+    const bool done = cholqr_prologue<T>(G, k, cut_abs, X, sorted, ns_tol, Lm, Li, ld, sh);
+    if (clear) {
+        __syncthreads();
+        for (int e = tid; e < k * k; e += nt) G[e] = 0.0;
+    }
+    if (done) return;
     const T tauT = (T)tau;
     // Cholesky: step j leaves the Schur-complement entries a_ij (i > j) in
     // column j and subtracts a_ij a_cj / d_j from the trailing block; a pivot

@@ -24,7 +24,7 @@
 // With 3 passes every product is A_hi B_hi + A_hi B_lo + A_lo B_hi from operands
 // rounded to nearest TF32; the ket accumulator takes the two small ones first, the
 // bra GEMM has an accumulator for them (the tensor core truncates the accumulator
-// at every instruction).  BF16 runs one kind::f16 pass (K = 16 per MMA).
+// at every instruction).  Up to D = 5 the order is the fixed one (layered.cuh).  BF16 runs one kind::f16 pass (K = 16 per MMA).
 // What bounds it: the tensor pipe's narrow MMAs at D >= 6 (73 % of the TF32 rate
 // over the padded shapes at D = 8), the chunk's chain of hand-offs below.  Time of a
 // launch, 3xTF32, p = 16: (4, 64) 20 us, (5, 100) 140, (6, 144) 454 (137 TFLOP/s),
@@ -54,9 +54,11 @@ constexpr int WORKER0 = 4;                      // first worker warp (its tensor
 constexpr int THREADS = 32 * WORKER0 + 128 * NSET;
 constexpr int MAXST = 16;
 
-// nearest TF32 (a NaN may come out as zero, but stays in the remainder v - hi)
+// TF32 head of v: nearest (a NaN may come out as zero, but stays in the remainder
+// v - hi), or with FIXED the leading bits
+template <bool FIXED>
 __device__ __forceinline__ float tf32_hi(float v) {
-    return __uint_as_float((__float_as_uint(v) + 0x1000u) & 0xFFFFE000u);
+    return __uint_as_float((__float_as_uint(v) + (FIXED ? 0u : 0x1000u)) & 0xFFFFE000u);
 }
 
 // instruction descriptor: FP32 accumulator, A and B TF32 (kind::tf32) or BF16
@@ -222,17 +224,21 @@ layered_kernel(const float* __restrict__ Y, long long nb, int nc, const uint8_t*
                         break;
                     }
                     fence_after();
-                    const uint32_t d = tmem + P.c_acc1 + j * P.acc1_cols, y = tmem + P.c_y;
+                    const uint32_t d0 = tmem + P.c_acc1 + j * P.nacc1 * P.acc1_cols, y = tmem + P.c_y;
                     const uint64_t db0 = smem_desc(smem_u32(sB1 + (size_t)s1 * B1_SZ));
-                    // lo B_hi, hi B_lo, hi B_hi with 3 passes, hi B_hi alone with one
+                    // lo B_hi, hi B_lo, hi B_hi with 3 passes (the reverse in the fixed
+                    // order), hi B_hi alone with one
 #pragma unroll
-                    for (int pass = 3 - NPASS; pass < 3; ++pass) {
+                    for (int pq = 0; pq < NPASS; ++pq) {
+                        const int pass = P.fixed ? 2 - pq : 3 - NPASS + pq;
 #pragma unroll
                         for (int ks = 0; ks < S1; ++ks) {
+                            const int i = pq * S1 + ks;
+                            const uint32_t d = d0 + (i % P.nacc1) * P.acc1_cols;
                             // 32 bytes of K per MMA, four per 128-byte block (16-byte descriptor units)
                             const uint64_t db = db0 + ((pass == 1 ? P.b1_bytes : 0) + (ks >> 2) * (P.n1p * 128) + (ks & 3) * 32) / 16;
                             const uint32_t a = y + (NPASS == 3 && pass == 0 ? P.y_cols : 0) + ks * 8;
-                            const uint32_t acc = (pass > 3 - NPASS || ks > 0) ? 1u : 0u;
+                            const uint32_t acc = i >= P.nacc1 ? 1u : 0u;
                             if constexpr (BF) umma_f16_tmem_a(by, d, a, db, ID1, acc);
                             else umma_tf32_tmem_a(by, d, a, db, ID1, acc);
                         }
@@ -260,15 +266,17 @@ layered_kernel(const float* __restrict__ Y, long long nb, int nc, const uint8_t*
                     const uint32_t a2 = tmem + P.c_a2 + ja * NPL * P.a2_cols;
                     const uint64_t db0 = smem_desc(smem_u32(sB2 + (size_t)s2 * B2_SZ));
 #pragma unroll
-                    for (int pass = 3 - NPASS; pass < 3; ++pass) {
+                    for (int pq = 0; pq < NPASS; ++pq) {
+                        const int pass = P.fixed ? 2 - pq : 3 - NPASS + pq;
 #pragma unroll
                         for (int ks = 0; ks < S2; ++ks) {
+                            const int i = pq * S2 + ks;
                             const uint64_t db = db0 + ((pass == 1 ? P.b2_bytes : 0) + (ks >> 2) * (P.n2p * 128) + (ks & 3) * 32) / 16;
                             // 8 tensor-memory columns of Z per MMA (8 TF32 or 16 BF16 values)
                             const uint32_t a = a2 + (NPASS == 3 && pass == 0 ? P.a2_cols : 0) + ks * 8;
                             const bool main = pass == 2;            // leading products: accumulators 0 .. nm - 1
-                            const uint32_t dd = d0 + (main ? ks % P.nm : P.nm) * P.out_cols;
-                            const bool first = main ? ks < P.nm : (pass == 0 && ks == 0);
+                            const uint32_t dd = d0 + (P.fixed ? i % P.nacc2 : main ? ks % P.nm : P.nm) * P.out_cols;
+                            const bool first = P.fixed ? i < P.nacc2 : main ? ks < P.nm : (pass == 0 && ks == 0);
                             const uint32_t acc = (cc > 0 || !first) ? 1u : 0u;
                             if constexpr (BF) umma_f16_tmem_a(by, dd, a, db, ID2, acc);
                             else umma_tf32_tmem_a(by, dd, a, db, ID2, acc);
@@ -306,7 +314,7 @@ layered_kernel(const float* __restrict__ Y, long long nb, int nc, const uint8_t*
                 if constexpr (BF) return __uint_as_float(pack_bf16x2(v[2 * c], v[2 * c + 1]));
                 const float x = v[c];
                 if (NPASS != 3) return x;
-                const float h = tf32_hi(x);
+                const float h = tf32_hi<P.fixed>(x);
                 return lo ? x - h : h;
             };
 #pragma unroll
@@ -385,10 +393,22 @@ layered_kernel(const float* __restrict__ Y, long long nb, int nc, const uint8_t*
                 uint32_t vr[P.n1p / 16][16];
 #pragma unroll
                 for (int c0 = 0; c0 < P.n1p; c0 += 16)
-                    tmem_ld16_async(tmem + lane_base + (uint32_t)(P.c_acc1 + j * P.acc1_cols + c0), vr[c0 / 16]);
+                    tmem_ld16_async(tmem + lane_base + (uint32_t)(P.c_acc1 + j * P.nacc1 * P.acc1_cols + c0), vr[c0 / 16]);
                 tmem_ld_wait();
 #pragma unroll
                 for (int c0 = 0; c0 < P.n1p; c0 += 16) tmem_regs_ready(vr[c0 / 16]);
+                if constexpr (P.nacc1 == 2) {            // 16 columns at a time: the register file
+#pragma unroll
+                    for (int c0 = 0; c0 < P.n1p; c0 += 16) {
+                        uint32_t r[16];
+                        tmem_ld16_async(tmem + lane_base + (uint32_t)(P.c_acc1 + (j * 2 + 1) * P.acc1_cols + c0), r);
+                        tmem_ld_wait();
+                        tmem_regs_ready(r);
+#pragma unroll
+                        for (int i = 0; i < 16; ++i)
+                            vr[c0 / 16][i] = __float_as_uint(__uint_as_float(vr[c0 / 16][i]) + __uint_as_float(r[i]));
+                    }
+                }
                 auto v = [&](int n) { return __uint_as_float(vr[n >> 4][n & 15]); };
                 fence_before();
                 mbar_arrive(&bars.acc1_empty[g & 1]);
@@ -472,7 +492,8 @@ layered_kernel(const float* __restrict__ Y, long long nb, int nc, const uint8_t*
             fence_after();
             float o[P.n2p];
 #pragma unroll
-            for (int a = P.nacc2 - 1; a >= 0; --a) {           // the small products first
+            for (int aq = 0; aq < P.nacc2; ++aq) {
+                const int a = P.fixed ? aq : P.nacc2 - 1 - aq;   // the small products first
                 uint32_t orr[P.n2p / 16][16];
 #pragma unroll
                 for (int c0 = 0; c0 < P.n2p; c0 += 16)
@@ -484,7 +505,7 @@ layered_kernel(const float* __restrict__ Y, long long nb, int nc, const uint8_t*
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
                         const float x = __uint_as_float(orr[c0 / 16][i]);
-                        o[c0 + i] = a == P.nacc2 - 1 ? x : o[c0 + i] + x;
+                        o[c0 + i] = aq == 0 ? x : o[c0 + i] + x;
                     }
                 }
             }

@@ -30,7 +30,9 @@ __host__ __device__ constexpr int pad_to(int x, int m) { return (x + m - 1) / m 
 struct Plan {
     int esz = 4, kstep = 8;                  // element bytes; K per MMA
     int d2 = 0, bt = 0, rows = 0;            // D^2; blocks b per tile; rows (b, ib) used of 128
-    int pc = 0, nb1 = 0, na2 = 0;            // physical indices per chunk; ket accumulators; Z buffers
+    bool fixed = false;                      // the fixed order of D <= kFixedOrderD with 3 passes
+    int pc = 0, nb1 = 0, na2 = 0;            // physical indices per chunk; ket buffers; Z buffers
+    int nacc1 = 1;                           // accumulators of a ket buffer
     int nm = 0, nacc2 = 0;                   // bra accumulators: of the leading products, and in all
     int n1 = 0, n1p = 0, k1p = 0, kb1 = 0;   // ket GEMM: N = pc D^2 (padded to 16), K = D^2 (padded to kstep)
     int n2p = 0, k2 = 0, k2p = 0, kb2 = 0;   // bra GEMM: N = D^2 (padded to 16), K = pc D^2 (padded to kstep)
@@ -52,6 +54,13 @@ struct Plan {
 // this kernel at N = 48 and 64 and on gemm3x.cu at 160), a chunk 100 more for
 // its hand-off and 100 for each operand that has one buffer only.  Shared-memory
 // operands use the 128-byte-swizzle K-major layout in K blocks of 128 bytes.
+//
+// With 3 passes and D <= kFixedOrderD the order and rounding of every sum are fixed
+// (see make_dims in ctm.cu): operand heads are cut off and not rounded, the MMAs
+// of a GEMM go pass by pass (hi hi, hi lo, lo hi) round-robin to four bra
+// accumulators and to two ket accumulators a buffer (one at D = 3), summed in
+// their order when read, and pc is the largest that fits.
+constexpr int kFixedOrderD = 5;
 __host__ __device__ constexpr Plan make_plan(int D, int npass, bool bf16 = false) {
     Plan P{};
     P.esz = bf16 ? 2 : 4;
@@ -65,6 +74,7 @@ __host__ __device__ constexpr Plan make_plan(int D, int npass, bool bf16 = false
     P.n2p = pad_to(P.d2, 16);
     if (P.bt < 1 || (bf16 && npass != 1)) return P;
     const int npl = npass == 3 ? 2 : 1;
+    P.fixed = npass == 3 && D <= kFixedOrderD;
     double best = 1e30;
     for (int pc = 16; pc >= 1; pc /= 2) {
         const int n1p = pad_to(pc * P.d2, 16);
@@ -74,12 +84,14 @@ __host__ __device__ constexpr Plan make_plan(int D, int npass, bool bf16 = false
         const int nc = (16 + pc - 1) / pc;              // chunks at p = 16
         const int mm1 = (P.k1p / P.kstep) * npass, mm2 = (k2p / P.kstep) * npass;
         const double c1 = 20.0 + 0.64 * n1p, c2 = 20.0 + 0.64 * P.n2p;
+        if (P.fixed && P.pc > 0) break;
+        const int nacc1 = P.fixed && D != 3 ? 2 : 1;
         for (int nm = 2; nm >= 1; --nm)
             for (int nb = 4; nb >= 1; --nb) {
                 const int nb1 = nb >= 3 ? 2 : 1, na2 = nb % 2 == 0 ? 2 : 1;
-                const int nacc2 = nm + (npass == 3 ? 1 : 0);
+                const int nacc2 = P.fixed ? 4 : nm + (npass == 3 ? 1 : 0);
                 if (nm > k2p / P.kstep) continue;
-                const int cols = nb1 * pad_to(n1p, 32) + nacc2 * pad_to(P.n2p, 32) + npl * (na2 * zcols + ycols);
+                const int cols = nb1 * nacc1 * pad_to(n1p, 32) + nacc2 * pad_to(P.n2p, 32) + npl * (na2 * zcols + ycols);
                 if (cols > 512) continue;
                 const double cost = nc * (mm1 * c1 + mm2 * c2 + 500.0 - 100.0 * (nb1 + na2)) - nm;
                 if (cost >= best) continue;
@@ -87,6 +99,7 @@ __host__ __device__ constexpr Plan make_plan(int D, int npass, bool bf16 = false
                 P.pc = pc;
                 P.nb1 = nb1;
                 P.na2 = na2;
+                P.nacc1 = nacc1;
                 P.nm = nm;
                 P.nacc2 = nacc2;
                 P.n1 = pc * P.d2;
@@ -104,7 +117,7 @@ __host__ __device__ constexpr Plan make_plan(int D, int npass, bool bf16 = false
                 P.acc1_cols = pad_to(n1p, 32);
                 P.out_cols = pad_to(P.n2p, 32);
                 P.c_acc1 = 0;
-                P.c_out = nb1 * P.acc1_cols;
+                P.c_out = nb1 * nacc1 * P.acc1_cols;
                 P.c_a2 = P.c_out + nacc2 * P.out_cols;
                 P.a2_cols = zcols;
                 P.c_y = P.c_a2 + na2 * npl * zcols;

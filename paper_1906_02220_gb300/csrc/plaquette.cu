@@ -90,7 +90,7 @@ void Engine<T>::plaquette_corner(Slot<T>& sl, int f, const double* Tk, T* out) {
     } else {
         derive_operands<T>(Tk, p, D, dm.pmax, pq_cor, pq_edg, st);
         const long long fo = (long long)f * dm.pmax * dm.D4;
-        site_layer(Yp, chi2, pq_cor + fo, nullptr, nullptr, p, Qt, nullptr, nullptr, sl.Tcor + fo);
+        site_layer(Yp, chi2, pq_cor + fo, nullptr, nullptr, p, Qt, nullptr, nullptr, false, sl.Tcor + fo);
     }
     permute<T, T>(Qt, out, {chi, chi, D, D, D, D}, {0, 3, 5, 1, 2, 4}, st);     // [(w,dk,db)][(z,rk,rb)]
 }

@@ -33,18 +33,29 @@ void check_wait(const int* err, cudaStream_t st) {
     if (h) kh::fail(KH_ETIMEOUT, "tensor-core GEMM wait timed out");
 }
 
-// tensor-core path, one TF32 pass: B^T made K-major by a permutation
-void run_tc_gemm(int M, int N, int K, const double* A, const double* B, double* C, void* scratch, size_t bytes,
-                 cudaStream_t st) {
+// tensor-core path: B^T made K-major by a permutation, optional hi/lo split
+void run_tc_gemm(int npass, int M, int N, int K, const double* A, const double* B, double* C, void* scratch,
+                 size_t bytes, cudaStream_t st) {
     kh::Carver cv(scratch, bytes);
     float* a = cv.take<float>((size_t)M * K);
     float* bt = cv.take<float>((size_t)K * N);
     float* c = cv.take<float>((size_t)M * N);
+    float* ah = cv.take<float>((size_t)M * K);
+    float* al = cv.take<float>((size_t)M * K);
+    float* bh = cv.take<float>((size_t)K * N);
+    float* bl = cv.take<float>((size_t)K * N);
     int* err = cv.take<int>(64);
     KH_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
     kh::cast<double, float>(A, a, (long long)M * K, st);
     kh::permute<double, float>(B, bt, {K, N}, {1, 0}, st);
-    kh::tc_gemm(kh::TcOperand{a, K}, kh::TcOperand{bt, K}, c, M, N, K, N, 1.f, 0.f, nullptr, err, st);
+    kh::TcOperand oa{a, nullptr, K}, ob{bt, nullptr, K};
+    if (npass == 3) {
+        kh::tc_split(a, ah, al, (long long)M * K, st);
+        kh::tc_split(bt, bh, bl, (long long)K * N, st);
+        oa = kh::TcOperand{ah, al, K};
+        ob = kh::TcOperand{bh, bl, K};
+    }
+    kh::tc_gemm(oa, ob, c, M, N, K, N, 1.f, 0.f, nullptr, npass, err, st);
     kh::cast<float, double>(c, C, (long long)M * N, st);
     check_wait(err, st);
 }
@@ -99,7 +110,8 @@ void run_svd(int k, const double* X, double* S, double* L, double* Qm, void* scr
 }
 
 template <typename T>
-void run_orth(int n, int k, double cut, const double* Y, double* Q, void* scratch, size_t bytes, cudaStream_t st) {
+void run_orth(bool by_column, int n, int k, double cut, const double* Y, double* Q, void* scratch, size_t bytes,
+              cudaStream_t st) {
     kh::Carver cv(scratch, bytes);
     T* y = cv.take<T>((size_t)n * k);
     T* tmp = cv.take<T>((size_t)n * k);
@@ -107,7 +119,7 @@ void run_orth(int n, int k, double cut, const double* Y, double* Q, void* scratc
     T* xk = cv.take<T>((size_t)k * k);
     double* dg = cv.take<double>((size_t)k * k);
     kh::cast<double, T>(Y, y, (long long)n * k, st);
-    kh::cholqr2<T>(y, n, k, cut, tmp, xk, dg, u, st);
+    kh::cholqr2<T>(y, n, k, cut, tmp, xk, dg, u, st, nullptr, 0, false, nullptr, by_column);
     kh::cast<T, double>(u, Q, (long long)n * k, st);
 }
 
@@ -201,8 +213,8 @@ kh_status selftest_gemm_on(int prec, int M, int N, int K, const double* A, const
     return run([&] {
         if (prec == KH_FP64) run_gemm<double>(M, N, K, A, B, C, scratch, bytes, st);
         else if (prec == KH_FP32) run_gemm<float>(M, N, K, A, B, C, scratch, bytes, st);
-        else if (prec == KH_TF32) run_tc_gemm(M, N, K, A, B, C, scratch, bytes, st);
-        else if (prec == KH_TF32X3) run_gemm3x(false, M, N, K, A, B, C, scratch, bytes, st);
+        else if (prec == KH_TF32) run_tc_gemm(1, M, N, K, A, B, C, scratch, bytes, st);
+        else if (prec == KH_TF32X3) run_tc_gemm(3, M, N, K, A, B, C, scratch, bytes, st);
         else kh::fail(KH_EINVAL, "precision not built");
         KH_CUDA(cudaStreamSynchronize(st));
     });
@@ -223,8 +235,8 @@ kh_status kh_selftest_gemm(int prec, int M, int N, int K, const double* A, const
     return run([&] {
         if (prec == KH_FP64) run_gemm<double>(M, N, K, A, B, C, scratch, bytes, st);
         else if (prec == KH_FP32) run_gemm<float>(M, N, K, A, B, C, scratch, bytes, st);
-        else if (prec == KH_TF32) run_tc_gemm(M, N, K, A, B, C, scratch, bytes, st);
-        else if (prec == KH_TF32X3) run_gemm3x(false, M, N, K, A, B, C, scratch, bytes, st);
+        else if (prec == KH_TF32) run_tc_gemm(1, M, N, K, A, B, C, scratch, bytes, st);
+        else if (prec == KH_TF32X3) run_tc_gemm(3, M, N, K, A, B, C, scratch, bytes, st);
         else kh::fail(KH_EINVAL, "precision not built");
         KH_CUDA(cudaStreamSynchronize(st));
     });
@@ -346,8 +358,8 @@ kh_status kh_selftest_orth(int prec, int n, int k, double cut, const double* Y, 
     if (bytes < kh_selftest_bytes(n, k, k)) return KH_ENOMEM;
     cudaStream_t st = (cudaStream_t)stream;
     return run([&] {
-        if (prec == KH_FP64) run_orth<double>(n, k, cut, Y, Qm, scratch, bytes, st);
-        else run_orth<float>(n, k, cut, Y, Qm, scratch, bytes, st);
+        if (prec == KH_FP64) run_orth<double>(true, n, k, cut, Y, Qm, scratch, bytes, st);
+        else run_orth<float>(prec == KH_TF32X3, n, k, cut, Y, Qm, scratch, bytes, st);
         KH_CUDA(cudaStreamSynchronize(st));
     });
 }

@@ -1,7 +1,11 @@
 // Tensor-core GEMM for sm_103a (5th-generation tensor cores):
 //   C[m][n] = alpha * colscale[n] * sum_k A[m][k] B[n][k] + beta * C[m][n]
-// A (M x K) and B (N x K) row-major ("K-major"), FP32 storage read as TF32 (one
-// pass; gemm3x.cu is the FP32-accurate form); C FP32 row-major.
+// A (M x K) and B (N x K) row-major ("K-major"), FP32 storage read as TF32;
+// C FP32 row-major.  NPASS = 3 runs the error-compensated split
+// A = A_hi + A_lo, B = B_hi + B_lo (hi = the leading TF32 part of the bits) as
+// A_hi B_hi + A_hi B_lo + A_lo B_hi: FP32-level accuracy, with the rounding that
+// the contexts of one fixed order keep (Dims::fixed_order; gemm3x.cu is the
+// faster and more accurate form of the others).
 //
 // One 128 x BN output tile per CTA, 6 warps:
 //   warp 0     TMA producer: 128B-swizzled K-major tiles into a STAGES-deep
@@ -25,12 +29,12 @@ constexpr int BK = 32;               // 32 FP32 = one 128-byte swizzle row
 constexpr int THREADS = 192;
 
 
-template <int BN>
+template <int BN, int NPASS>
 struct Cfg {
     static constexpr int A_BYTES = BM * BK * 4;
     static constexpr int B_BYTES = BN * BK * 4;
-    static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-    static constexpr int STAGES = 4;
+    static constexpr int STAGE_BYTES = (NPASS == 3 ? 2 : 1) * (A_BYTES + B_BYTES);
+    static constexpr int STAGES = (NPASS == 3 ? 3 : 4);
     static constexpr int SMEM = STAGES * STAGE_BYTES + 1024;
     // consecutive MMAs into one accumulator form a dependent chain whose
     // latency exceeds a narrow tile's MMA time: narrow tiles spread their
@@ -45,11 +49,13 @@ struct Cfg {
                                       | ((uint32_t)(BM >> 4) << 24);// M / 16
 };
 
-template <int BN>
+template <int BN, int NPASS>
 __global__ void __launch_bounds__(THREADS, 1)
-gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB, float* __restrict__ C, int M, int N, int K, long long ldc, float alpha, float beta, const float* __restrict__ colscale,
+gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB,
+            const __grid_constant__ CUtensorMap mA2, const __grid_constant__ CUtensorMap mB2, float* __restrict__ C,
+            int M, int N, int K, long long ldc, float alpha, float beta, const float* __restrict__ colscale,
             int* err) {
-    using G = Cfg<BN>;
+    using G = Cfg<BN, NPASS>;
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[G::STAGES], empty_bar[G::STAGES], acc_bar;
     __shared__ uint32_t s_tmem;
@@ -90,6 +96,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUte
                 mbar_expect_tx(&full_bar[s], G::STAGE_BYTES);
                 tma_load_2d(st, &mA, &full_bar[s], kt * BK, m0);
                 tma_load_2d(st + G::A_BYTES, &mB, &full_bar[s], kt * BK, n0);
+                if (NPASS == 3) {
+                    tma_load_2d(st + G::A_BYTES + G::B_BYTES, &mA2, &full_bar[s], kt * BK, m0);
+                    tma_load_2d(st + 2 * G::A_BYTES + G::B_BYTES, &mB2, &full_bar[s], kt * BK, n0);
+                }
             }
         }
     } else if (warp == 1) {
@@ -103,8 +113,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUte
                 break;
             }
             fence_after();
-            const uint64_t da = smem_desc(smem_u32(base + s * G::STAGE_BYTES));
-            const uint64_t db = smem_desc(smem_u32(base + s * G::STAGE_BYTES + G::A_BYTES));
+            const uint32_t a0 = smem_u32(base + s * G::STAGE_BYTES), b0 = a0 + G::A_BYTES;
+            const uint64_t da = smem_desc(a0), db = smem_desc(b0);
+            const uint64_t da2 = smem_desc(b0 + G::B_BYTES), db2 = smem_desc(b0 + G::B_BYTES + G::A_BYTES);   // lo parts
 #pragma unroll
             for (int kk = 0; kk < BK / 8; ++kk) {
                 // 8 TF32 = 32 bytes along K = 2 descriptor units; accumulator of this
@@ -112,6 +123,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUte
                 const int i = kt * (BK / 8) + kk;
                 const uint32_t d = tmem + (uint32_t)((kk % G::NACC) * G::ACC_COLS);
                 umma_tf32(by, d, da + kk * 2, db + kk * 2, G::IDESC, i >= G::NACC ? 1u : 0u);
+                if (NPASS == 3) {
+                    umma_tf32(by, d, da + kk * 2, db2 + kk * 2, G::IDESC, 1u);
+                    umma_tf32(by, d, da2 + kk * 2, db + kk * 2, G::IDESC, 1u);
+                }
             }
             umma_commit(by, &empty_bar[s]);
         }
@@ -162,6 +177,18 @@ gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUte
     }
 }
 
+// hi = value with the 13 low mantissa bits cleared (exactly TF32), lo = x - hi
+__global__ void split_kernel(const float* __restrict__ x, float* __restrict__ hi, float* __restrict__ lo,
+                             long long n) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+         i += (long long)gridDim.x * blockDim.x) {
+        float v = x[i];
+        float h = __uint_as_float(__float_as_uint(v) & 0xFFFFE000u);
+        hi[i] = h;
+        lo[i] = v - h;
+    }
+}
+
 }  // namespace tc
 
 // ------------------------------------------------------------------ host side
@@ -198,29 +225,44 @@ CUtensorMap tc_make_map(const float* p, long long rows, long long K, long long l
     return m;
 }
 
-template <int BN>
+template <int BN, int NPASS>
 static void launch_tc(const TcOperand& A, const TcOperand& B, float* C, int M, int N, int K, long long ldc,
                       float alpha, float beta, const float* colscale, int* err, cudaStream_t st) {
-    using G = tc::Cfg<BN>;
+    using G = tc::Cfg<BN, NPASS>;
     static std::atomic<size_t> granted[kMaxDevices] = {};
-    smem_opt_in(tc::gemm_kernel<BN>, (size_t)G::SMEM, granted);
-    CUtensorMap ma = tc_make_map(A.p, M, K, A.ld, tc::BM);
-    CUtensorMap mb = tc_make_map(B.p, N, K, B.ld, BN);
+    smem_opt_in(tc::gemm_kernel<BN, NPASS>, (size_t)G::SMEM, granted);
+    CUtensorMap ma = tc_make_map(A.hi, M, K, A.ld, tc::BM);
+    CUtensorMap mb = tc_make_map(B.hi, N, K, B.ld, BN);
+    CUtensorMap ma2 = NPASS == 3 ? tc_make_map(A.lo, M, K, A.ld, tc::BM) : ma;
+    CUtensorMap mb2 = NPASS == 3 ? tc_make_map(B.lo, N, K, B.ld, BN) : mb;
     dim3 grid((N + BN - 1) / BN, (M + tc::BM - 1) / tc::BM);
     if (grid.y > 65535) fail(KH_EINVAL, "tc gemm: M too large");
-    tc::gemm_kernel<BN><<<grid, tc::THREADS, G::SMEM, st>>>(ma, mb, C, M, N, K, ldc, alpha, beta, colscale, err);
+    tc::gemm_kernel<BN, NPASS><<<grid, tc::THREADS, G::SMEM, st>>>(ma, mb, ma2, mb2, C, M, N, K, ldc, alpha, beta,
+                                                                   colscale, err);
     KH_LAUNCHED();
 }
 
-void tc_gemm(const TcOperand& A, const TcOperand& B, float* C, int M, int N, int K, long long ldc, float alpha,
-             float beta, const float* colscale, int* err, cudaStream_t st) {
-    if (M <= 0 || N <= 0 || K <= 0) return;
+template <int NPASS>
+static void dispatch_bn(const TcOperand& A, const TcOperand& B, float* C, int M, int N, int K, long long ldc,
+                        float alpha, float beta, const float* colscale, int* err, cudaStream_t st) {
     const long long mt = (M + tc::BM - 1) / tc::BM;
     // widest tile that still gives ~one wave of CTAs over the 152 SMs
-    if (N <= 16) launch_tc<16>(A, B, C, M, N, K, ldc, alpha, beta, colscale, err, st);
-    else if (N <= 32) launch_tc<32>(A, B, C, M, N, K, ldc, alpha, beta, colscale, err, st);
-    else if (N <= 64 || mt * ((N + 127) / 128) < 120) launch_tc<64>(A, B, C, M, N, K, ldc, alpha, beta, colscale, err, st);
-    else launch_tc<128>(A, B, C, M, N, K, ldc, alpha, beta, colscale, err, st);
+    if (N <= 16) launch_tc<16, NPASS>(A, B, C, M, N, K, ldc, alpha, beta, colscale, err, st);
+    else if (N <= 32) launch_tc<32, NPASS>(A, B, C, M, N, K, ldc, alpha, beta, colscale, err, st);
+    else if (N <= 64 || mt * ((N + 127) / 128) < 120) launch_tc<64, NPASS>(A, B, C, M, N, K, ldc, alpha, beta, colscale, err, st);
+    else launch_tc<128, NPASS>(A, B, C, M, N, K, ldc, alpha, beta, colscale, err, st);
+}
+
+void tc_gemm(const TcOperand& A, const TcOperand& B, float* C, int M, int N, int K, long long ldc, float alpha,
+             float beta, const float* colscale, int npass, int* err, cudaStream_t st) {
+    if (M <= 0 || N <= 0 || K <= 0) return;
+    if (npass == 3) dispatch_bn<3>(A, B, C, M, N, K, ldc, alpha, beta, colscale, err, st);
+    else dispatch_bn<1>(A, B, C, M, N, K, ldc, alpha, beta, colscale, err, st);
+}
+
+void tc_split(const float* x, float* hi, float* lo, long long n, cudaStream_t st) {
+    tc::split_kernel<<<grid_for(n), 256, 0, st>>>(x, hi, lo, n);
+    KH_LAUNCHED();
 }
 
 }  // namespace kh

@@ -403,6 +403,11 @@ kh_status kh_selftest_gemm3x(int a_colmajor, int M, int N, int K, const double* 
 kh_status kh_selftest_permute(int kind, int rank, const long long* shape, const int* order, const double* dev_in,
                               double* dev_out, void* dev_scratch, size_t scratch_bytes, void* stream);
 
+/* Sets the context's flag of tensor-core waits that ran out, as a kernel that
+ * gave up would (bits = 0 clears it): every call that hands out or stores
+ * results then returns KH_ETIMEOUT in the tensor-core kinds.  Synchronises. */
+kh_status kh_selftest_wait_flag(kh_ctx* ctx, int bits);
+
 /* Eigen-decomposition of a symmetric k x k FP64 matrix by the library's
  * Jacobi kernel in FP64 (prec = KH_FP64) or FP32 (otherwise): dev_evals
  * descending, column j of dev_W its eigenvector.  Scratch as above with

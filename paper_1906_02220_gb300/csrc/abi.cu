@@ -211,6 +211,7 @@ kh_status kh_save(kh_ctx* ctx, const char* path) {
     KH_RANGE();
     return guard(ctx, [&] {
         if (!path) kh::fail(KH_EINVAL, "null path");
+        ctx->eng->sync_checked();    // nothing that a timed-out kernel left behind is stored, nor a file opened for it
         FileCloser fc{std::fopen(path, "wb")};
         if (!fc.f) kh::fail(KH_EINVAL, std::string("cannot open ") + path + " for writing");
         if (std::fwrite(kCheckpointMagic, 1, 8, fc.f) != 8 ||
@@ -567,6 +568,11 @@ kh_status eefu_evolve_batch(kh_ctx* const* ctxs, int n, const double* J, const d
 }
 
 unsigned long long kh_launch_count(void) { return kh::g_launches.load(std::memory_order_relaxed); }
+
+kh_status kh_selftest_wait_flag(kh_ctx* ctx, int bits) {
+    KH_RANGE();
+    return guard(ctx, [&] { ctx->eng->set_wait_flag(bits); });
+}
 
 kh_status kh_profile(kh_ctx* ctx, int enable, double* out) {
     KH_RANGE();

@@ -888,7 +888,7 @@ int Engine<T>::als_run(int gamma, double* rel_cost) {
         if (it % kCheckEvery == 0 || it == cfg.als_max_iter) {
             int hf[2];
             KH_CUDA(cudaMemcpyAsync(hf, flags, sizeof(hf), cudaMemcpyDeviceToHost, st));
-            KH_CUDA(cudaStreamSynchronize(st));
+            sync_checked();                                  // a time-out comes before what its leftovers look like
             if (hf[0]) fail(KH_ENUMERIC, "ALS: Cholesky breakdown (metric not positive)");
             if (hf[1]) break;
         }

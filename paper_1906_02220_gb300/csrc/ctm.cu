@@ -1279,10 +1279,7 @@ int Engine<T>::sweep(int slot, int max_sweeps, int min_sweeps, double tol, doubl
         done = it;
         if (tol >= 0.0) {
             KH_CUDA(cudaMemcpyAsync(&delta, sl.delta, sizeof(double), cudaMemcpyDeviceToHost, st));
-            int terr = 0;
-            if (tc_npass) KH_CUDA(cudaMemcpyAsync(&terr, tc_err, sizeof(int), cudaMemcpyDeviceToHost, st));
-            KH_CUDA(cudaStreamSynchronize(st));
-            if (terr) fail(KH_ETIMEOUT, "tensor-core kernel wait timed out (flag " + std::to_string(terr) + ")");
+            sync_checked();
             if (!(delta == delta)) fail(KH_ENUMERIC, "NaN in CTM spectra");
             if (it >= min_sweeps && delta < tol) break;
         }
@@ -1336,18 +1333,13 @@ int Engine<T>::sweep_lanes(const int* slot_ids, int count, int mx, int mn, doubl
                 if (tol >= 0.0) KH_CUDA(cudaMemcpyAsync(&delta[i], sl.delta, sizeof(double), cudaMemcpyDeviceToHost, st));
             }
         if (tol >= 0.0) {
-            int terr = 0;
             for (int i = 0; i < count; ++i)
                 if (active[i]) {
                     bind(i);
                     KH_CUDA(cudaStreamSynchronize(st));
                 }
-            if (tc_npass) {
-                bind(0);
-                KH_CUDA(cudaMemcpyAsync(&terr, tc_err, sizeof(int), cudaMemcpyDeviceToHost, st));
-                KH_CUDA(cudaStreamSynchronize(st));
-                if (terr) fail(KH_ETIMEOUT, "tensor-core kernel wait timed out (flag " + std::to_string(terr) + ")");
-            }
+            bind(0);
+            sync_checked();
             bool any = false;
             for (int i = 0; i < count; ++i)
                 if (active[i]) {
@@ -1375,7 +1367,7 @@ void Engine<T>::projectors_out(int slot, int dir, double* spec, double* trunc) {
     if (trunc) {
         KH_CUDA(cudaMemcpyAsync(trunc, sl.trunc + dir, sizeof(double), cudaMemcpyDeviceToHost, st));
     }
-    KH_CUDA(cudaStreamSynchronize(st));
+    sync_checked();
 }
 
 template <typename T>
@@ -1384,7 +1376,7 @@ void Engine<T>::get_env(int slot, double* C, double* E) {
     const long long chi2 = (long long)dm.chi * dm.chi, E1 = (long long)dm.chi * dm.d2 * dm.chi;
     if (C) KH_CUDA(cudaMemcpyAsync(C, sl.C, sizeof(double) * 4 * chi2, cudaMemcpyDeviceToDevice, st));
     if (E) KH_CUDA(cudaMemcpyAsync(E, sl.E, sizeof(double) * 4 * E1, cudaMemcpyDeviceToDevice, st));
-    KH_CUDA(cudaStreamSynchronize(st));
+    sync_checked();
 }
 
 // ------------------------------------------------------------------ metric, kappa, expval

@@ -107,6 +107,8 @@ struct EngineBase {
     virtual void get_state(double* A, double* B) = 0;
     virtual void reset_counters() = 0;
     virtual double read_counter() = 0;
+    virtual void set_wait_flag(int bits) = 0;
+    virtual void sync_checked() = 0;
     virtual void set_tensor(int slot, const double* Tin, int p) = 0;
     virtual void build_composite(int slot, int gamma, const double* gate) = 0;
     virtual void init_env(int slot, const double* edge) = 0;
@@ -270,7 +272,11 @@ struct Engine : EngineBase {
     void absorb(Slot<T>& sl, int s);
     void move(Slot<T>& sl, int s, int slot_id);
     void compute_metric(Slot<T>& sl, double* N_out);
-    void sync_checked();
+    void sync_checked() override;
+    void set_wait_flag(int bits) override {
+        KH_CUDA(cudaMemcpyAsync(tc_err, &bits, sizeof(int), cudaMemcpyHostToDevice, st));
+        KH_CUDA(cudaStreamSynchronize(st));
+    }
     void build_derived(Slot<T>& sl);
 
     // bond internals

@@ -127,11 +127,8 @@ void Engine<T>::plaquette(int slot, const double* ops, double* out) {
         KH_LAUNCHED();
     }
     double h[2];
-    int terr = 0;
     KH_CUDA(cudaMemcpyAsync(h, z, sizeof(h), cudaMemcpyDeviceToHost, st));
-    if (tc_npass) KH_CUDA(cudaMemcpyAsync(&terr, tc_err, sizeof(int), cudaMemcpyDeviceToHost, st));
-    KH_CUDA(cudaStreamSynchronize(st));
-    if (terr) fail(KH_ETIMEOUT, "tensor-core kernel wait timed out (flag " + std::to_string(terr) + ")");
+    sync_checked();
     if (!(h[0] == h[0]) || !(h[1] == h[1]) || h[0] == 0.0 || std::isinf(h[0]) || std::isinf(h[1]))
         fail(KH_ENUMERIC, "plaquette cluster zero or not finite");
     out[0] = h[1] / h[0];

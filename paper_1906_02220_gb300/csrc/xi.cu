@@ -232,7 +232,7 @@ void Engine<T>::correlation_length(int slot, int dir, int max_iter, double tol, 
                 }
             double H[16];
             KH_CUDA(cudaMemcpyAsync(H, Hd_, sizeof(double) * b * b, cudaMemcpyDeviceToHost, st));
-            KH_CUDA(cudaStreamSynchronize(st));
+            sync_checked();
             for (int i = 0; i < b * b; ++i)
                 if (!(H[i] == H[i])) fail(KH_ENUMERIC, "NaN in the transfer-matrix iteration");
             auto ev = small_eigenvalues(H, b);

@@ -22,7 +22,7 @@
 // Structure.  128 x bn output tiles (bn <= 160), one persistent CTA per SM:
 //   warps 0, 2  TMA producers: raw FP32 A tiles (128 x 32) and split B tiles (bn x 32
 //               each) into rings of their own: a stage of A is free again once
-//               the converters hold it in registers, one of B only when its
+//               the converters have it in tensor memory, one of B only when its
 //               MMAs are done;
 //   warp 1      tensor memory; issues the MMAs, A from tensor memory.  All its lanes
 //               walk the loop and one issues: with the loop inside a one-lane
@@ -289,7 +289,6 @@ gemm3x_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CU
                         x[4 * j + 3] = v.w;
                     }
                 }
-                mbar_arrive(&bars.ra_empty[s]);
                 if (!wait_all(&bars.a_empty[a], ((it / ABUF) & 1) ^ 1, abort_flag)) { ok = false; break; }
                 fence_after();
                 const uint32_t dst = tmem + lane_base + C_A + a * 2 * BK;
@@ -307,6 +306,10 @@ gemm3x_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CU
                 tmem_st_wait();
                 fence_before();
                 mbar_arrive(&bars.a_full[a]);
+                // only now have the loads of x provably completed: with the arrival right
+                // after them, and the wait on a_empty behind it, pieces of the stage's next
+                // tile were read instead (while the drain stored a tile)
+                mbar_arrive(&bars.ra_empty[s]);
             }
         }
         if (!ok) {

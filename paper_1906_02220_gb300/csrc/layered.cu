@@ -463,7 +463,6 @@ layered_kernel(const float* __restrict__ Y, long long nb, int nc, const uint8_t*
                         if (i + 3 < P.k2) z[i + 3] = w.w;
                     }
                 }
-                mbar_arrive(&bars.zs_r[set]);
                 // the bra GEMM of chunk g - na2 has read this Z buffer
                 const int ja = (int)(g % P.na2);
                 const long long h = g - P.na2;
@@ -477,6 +476,9 @@ layered_kernel(const float* __restrict__ Y, long long nb, int nc, const uint8_t*
                 tmem_st_wait();
                 fence_before();
                 mbar_arrive(&bars.a2_full[ja]);
+                // the reads of zbuf have provably completed only now that z is in tensor
+                // memory; other warps of the set scatter their next chunk over it then
+                mbar_arrive(&bars.zs_r[set]);
                 ++zcount;
             }
             if (!ok) break;

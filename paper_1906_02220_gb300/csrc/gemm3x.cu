@@ -5,7 +5,7 @@
 // products M V and M^T U, the basis products, the projectors and the bond metric.
 //
 // Accuracy.  Every operand is split as x = hi + lo with hi rounded to nearest
-// TF32 (|lo| <= 2^-12 |x|), and lo B_hi + hi B_lo + hi B_hi is formed.  The
+// TF32 (|lo| <= 2^-11 |x|), and lo B_hi + hi B_lo + hi B_hi is formed.  The
 // tensor core truncates its FP32 accumulator at every instruction, so a sum
 // kept there over the whole K loses ~3e-8 of itself per instruction, always
 // towards zero.  Here an accumulator holds 32 values of K at most: the small
@@ -415,8 +415,10 @@ gemm3x_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CU
 }
 
 // B (N x K by strides) into its K-major hi and lo parts (row stride ld >= K,
-// a multiple of 4; the columns past K are never read by the MMAs).  32 x 32
-// tiles through shared memory, so that both sides are coalesced.
+// a multiple of 4; the columns past K are not written, nor read: the tensor maps
+// are K wide, and where the last step of eight values runs past K the copies
+// fill in zeros).  32 x 32 tiles through shared memory, so that both sides are
+// coalesced.
 __global__ void __launch_bounds__(256)
 split_b_kernel(const float* __restrict__ B, long long sn, long long sk, int N, int K, float* __restrict__ hi,
                float* __restrict__ lo, int ld) {

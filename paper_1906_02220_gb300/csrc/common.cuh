@@ -616,7 +616,8 @@ __global__ void __launch_bounds__(128) gemm_f64_kernel(GemmArgs<double> g) {
     __shared__ double As[KC][TB + 1], Bs[KC][TB + 1];
     __shared__ double red[KG > 1 ? (KG - 1) * TB * TB : 1];
     const int tid = threadIdx.x, kg = tid / GT, t = tid % GT, tx = t % RX, ty = t / RX;
-    const int m0 = blockIdx.y * TB, n0 = blockIdx.x * TB;
+    const int nt = (g.N + TB - 1) / TB;            // tiles along N; the tiles lie on grid.x, whose limit is 2^31
+    const int m0 = (int)(blockIdx.x / nt) * TB, n0 = (int)(blockIdx.x % nt) * TB;
     const double* A = g.A + (long long)blockIdx.z * g.sAb;
     const double* B = g.B + (long long)blockIdx.z * g.sBb;
     const bool a_kfast = g.sAk == 1, b_nfast = g.sBn == 1;
@@ -697,8 +698,9 @@ inline void gemm_f64(const GemmArgs<double>& g, cudaStream_t st) {
     auto tiles = [&](int tb) { return (long long)((g.M + tb - 1) / tb) * ((g.N + tb - 1) / tb) * g.batch; };
     const bool small = tiles(16) < 8LL * 152;
     const int tb = small ? 8 : 16;
-    dim3 grid((g.N + tb - 1) / tb, (g.M + tb - 1) / tb, g.batch);
-    if (grid.y > 65535) fail(KH_EINVAL, "gemm M too large");
+    const long long nt = (long long)((g.M + tb - 1) / tb) * ((g.N + tb - 1) / tb);
+    if (nt > 0x7fffffffLL) fail(KH_EINVAL, "gemm too large");
+    const dim3 grid((unsigned)nt, 1, g.batch);
     if (small) launch(gemm_f64_kernel<8, 1>, grid, 128, 0, st, g);
     else launch(gemm_f64_kernel<16, 2>, grid, 128, 0, st, g);
 }

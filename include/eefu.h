@@ -408,6 +408,11 @@ kh_status kh_selftest_permute(int kind, int rank, const long long* shape, const 
  * results then returns KH_ETIMEOUT in the tensor-core kinds.  Synchronises. */
 kh_status kh_selftest_wait_flag(kh_ctx* ctx, int bits);
 
+/* The library's FP64 <-> FP32 conversions in integer arithmetic: dev_out[2i] =
+ * dev_x[i] rounded to FP32 (as FP64), dev_out[2i+1] = the FP32 value of dev_x[i]
+ * widened (n values in, 2n out).  Synchronises stream. */
+kh_status kh_selftest_convert(int n, const double* dev_x, double* dev_out, void* stream);
+
 /* Eigen-decomposition of a symmetric k x k FP64 matrix by the library's
  * Jacobi kernel in FP64 (prec = KH_FP64) or FP32 (otherwise): dev_evals
  * descending, column j of dev_W its eigenvector.  Scratch as above with

@@ -824,16 +824,19 @@ inline void gemm_rm(int M, int N, int K, const T* A, bool tA, const T* B, bool t
 // ------------------------------------------------------------------ reductions
 
 // FP32 <-> FP64 conversions in integer arithmetic (the conversion instructions
-// issue on the narrow FP64 pipe).  Subnormal FP32 values become zero either way;
-// d2f rounds to nearest even.
+// issue on the narrow FP64 pipe), without a branch.  Subnormal FP32 values pass
+// through a scaling by 2^64; d2f rounds to nearest even, subnormal results up to
+// one more rounding on the way.  d2f_flush makes those zero, for values that count
+// next to normal ones only.
 __device__ __forceinline__ double f2d(float x) {
-    const uint32_t u = __float_as_uint(x), e = u & 0x7f800000u;
-    const uint32_t up = e == 0x7f800000u ? 0x70000000u : 0x38000000u;
+    const bool sub = (__float_as_uint(x) & 0x7f800000u) == 0;
+    const uint32_t u = __float_as_uint(sub ? x * 0x1p64f : x), e = u & 0x7f800000u;
+    const uint32_t up = e == 0x7f800000u ? 0x70000000u : (sub ? 0x34000000u : 0x38000000u);
     const uint32_t hi = (u & 0x80000000u) | (e ? ((u & 0x7fffffffu) >> 3) + up : 0u);
     return __hiloint2double((int)hi, e ? (int)(u << 29) : 0);
 }
 __device__ __forceinline__ double f2d(double x) { return x; }
-__device__ __forceinline__ float d2f(double x) {
+__device__ __forceinline__ float d2f_flush(double x) {
     const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
     const uint32_t sign = hi & 0x80000000u, mag = hi & 0x7fffffffu;
     const uint32_t r = ((mag - 0x38000000u) << 3) | (lo >> 29), rem = lo & 0x1fffffffu;
@@ -842,6 +845,12 @@ __device__ __forceinline__ float d2f(double x) {
     v = mag >= 0x47f00000u ? (nan ? 0x7fc00000u : 0x7f800000u) : v;     // 2^128 and more, infinity, NaN
     v = mag < 0x38100000u ? 0u : v;
     return __uint_as_float(sign | v);
+}
+__device__ __forceinline__ float d2f(double x) {
+    const uint32_t hi = (uint32_t)__double2hiint(x);
+    const bool sub = (hi & 0x7fffffffu) < 0x38100000u;                  // below 2^-126
+    const float y = d2f_flush(__hiloint2double((int)(sub ? hi + 0x04000000u : hi), __double2loint(x)));
+    return sub ? y * 0x1p-64f : y;
 }
 
 // out[0] = sum x^2 (FP64 accumulate), one atomic per block; launch it on a

@@ -804,6 +804,8 @@ cholqr_reg_kernel(double* __restrict__ G, int k, double cut_abs, double tau, T* 
     __shared__ int s_perm[KM];
     const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
     const T tauT = (T)tau, cutT = (T)cut_abs;
+    // (an off-diagonal entry below the FP32 range counts as zero: the second pass
+    // makes good what that leaves between columns that small)
     for (int j = tid; j < k; j += 512) s_diag[j] = fmax(d2f(G[(long long)j * k + j]), T(0));
     __syncthreads();
     T w[KR][KT];
@@ -825,7 +827,7 @@ cholqr_reg_kernel(double* __restrict__ G, int k, double cut_abs, double tau, T* 
             for (int b = 0; b < KT; ++b) {
                 const int i = ty + 16 * a, c = tx + 32 * b;
                 // no branch around a load: all of a thread's loads in flight together
-                const T x = d2f(G[(long long)min(i, k - 1) * k + min(c, k - 1)]);
+                const T x = d2f_flush(G[(long long)min(i, k - 1) * k + min(c, k - 1)]);
                 w[a][b] = (i < k && c < k) ? x : T(0);
             }
 #pragma unroll
@@ -877,7 +879,7 @@ cholqr_reg_kernel(double* __restrict__ G, int k, double cut_abs, double tau, T* 
         for (int b = 0; b < KT; ++b) {
             const int i = ty + 16 * a, c = tx + 32 * b;
             const int pa = s_perm[min(i, k - 1)], pb = s_perm[min(c, k - 1)];
-            const T x = d2f(G[(long long)pa * k + pb]) * s_inv[pa] * s_inv[pb];
+            const T x = d2f_flush(G[(long long)pa * k + pb]) * s_inv[pa] * s_inv[pb];
             w[a][b] = (i < k && c < k) ? x : T(0);
         }
 #pragma unroll

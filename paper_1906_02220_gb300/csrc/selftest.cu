@@ -193,6 +193,13 @@ __global__ void newton_kernel(const double* __restrict__ x, int n, double* __res
     }
 }
 
+__global__ void convert_kernel(const double* __restrict__ x, int n, double* __restrict__ out) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        out[2 * i] = (double)kh::d2f(x[i]);
+        out[2 * i + 1] = kh::f2d((float)x[i]);
+    }
+}
+
 template <typename F>
 kh_status run(F&& f) {
     try {
@@ -284,6 +291,16 @@ kh_status kh_selftest_permute(int kind, int rank, const long long* shape, const 
             }
             kh::cast<float, double>(b, out, total, st);
         }
+        KH_CUDA(cudaStreamSynchronize(st));
+    });
+}
+
+kh_status kh_selftest_convert(int n, const double* x, double* out, void* stream) {
+    if (n < 1 || !x || !out) return KH_EINVAL;
+    cudaStream_t st = (cudaStream_t)stream;
+    return run([&] {
+        convert_kernel<<<(n + 255) / 256, 256, 0, st>>>(x, n, out);
+        KH_LAUNCHED();
         KH_CUDA(cudaStreamSynchronize(st));
     });
 }

@@ -41,7 +41,7 @@ constexpr int kColsMax = 2 * kClusterCtas * kSeatsMax;
 // Rotation (c, s) of two columns with squared norms a, b and inner product g:
 // the angle in FP32, the rotation orthogonal in FP64.
 __device__ __forceinline__ void rotation_fp32_angle(double a, double b, double g, double& c, double& s) {
-    const float zeta = __fdividef(d2f(b - a), 2.f * d2f(g));
+    const float zeta = __fdividef(d2f_flush(b - a), 2.f * d2f_flush(g));
     const float az = fabsf(zeta);
     float t = az > 1e15f ? __fdividef(0.5f, az) : __fdividef(1.f, az + sqrtf(fmaf(az, az, 1.f)));
     if (!(az <= 3e38f)) t = 0.f;           // g below the FP32 range against b - a: nothing to rotate
@@ -186,9 +186,9 @@ svd_cluster_kernel(const double* __restrict__ Xin, int k, int npc, double* __res
                 const bool rel = s_top[tc] | s_top[bc];
                 if (rel) {
                     // the squared cosine, in FP32 (columns below 1e-18 of the largest entry do not count)
-                    const float fa = d2f(a), fb = d2f(b);
+                    const float fa = d2f_flush(a), fb = d2f_flush(b);
                     if (fa > 1e-36f && fb > 1e-36f) {
-                        const float cs = d2f(g) * rsqrtf(fa) * rsqrtf(fb);
+                        const float cs = d2f_flush(g) * rsqrtf(fa) * rsqrtf(fb);
                         c2max = fmaxf(c2max, cs * cs);
                     }
                 }

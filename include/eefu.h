@@ -408,6 +408,13 @@ kh_status kh_selftest_permute(int kind, int rank, const long long* shape, const 
  * results then returns KH_ETIMEOUT in the tensor-core kinds.  Synchronises. */
 kh_status kh_selftest_wait_flag(kh_ctx* ctx, int bits);
 
+/* Gram matrix dev_G = A^T B (k x k FP64, k <= 160) of FP32 copies of the n x k
+ * operands (A^T A when dev_B is null): FP32 sums over 16 rows, FP64 sums of those.
+ * Scratch as kh_selftest_orth.  KH_EINVAL for k beyond the limit.  Synchronises
+ * stream. */
+kh_status kh_selftest_gram(int n, int k, const double* dev_A, const double* dev_B, double* dev_G, void* dev_scratch,
+                           size_t scratch_bytes, void* stream);
+
 /* The library's FP64 <-> FP32 conversions in integer arithmetic: dev_out[2i] =
  * dev_x[i] rounded to FP32 (as FP64), dev_out[2i+1] = the FP32 value of dev_x[i]
  * widened (n values in, 2n out).  Synchronises stream. */

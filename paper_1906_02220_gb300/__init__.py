@@ -26,7 +26,7 @@ ABI_FUNCTIONS = [
     "kh_set_state", "kh_get_state", "ctm_set_tensor", "ctm_build_composite", "ctm_init",
     "ctm_copy_env", "ctm_sweep", "ctm_projectors", "ctm_get_env", "ctm_metric", "ctm_kappa",
     "ctm_expval", "ctm_correlation_length", "ctm_plaquette", "ctm_flux", "eefu_apply_gate", "eefu_cost_gradient", "observables", "kh_version", "kh_bond_hamiltonian", "kh_gate", "kh_flux_operators",
-    "eefu_trotter_step", "eefu_evolve", "eefu_evolve_flux", "eefu_evolve_batch", "kh_launch_count", "kh_profile", "kh_selftest_bytes", "kh_selftest_gemm", "kh_selftest_gemm3x", "kh_selftest_wait_flag", "kh_selftest_convert", "kh_selftest_permute",
+    "eefu_trotter_step", "eefu_evolve", "eefu_evolve_flux", "eefu_evolve_batch", "kh_launch_count", "kh_profile", "kh_selftest_bytes", "kh_selftest_gemm", "kh_selftest_gemm3x", "kh_selftest_wait_flag", "kh_selftest_convert", "kh_selftest_gram", "kh_selftest_permute",
     "kh_selftest_symeig", "kh_selftest_svd", "kh_selftest_svd_refined", "kh_selftest_orth", "kh_selftest_fp64_newton",
     "kh_selftest_site_layered_bytes", "kh_selftest_site_layered", "kh_gemm_noalloc",
     "kh_gemm_noalloc_max_bytes", "kh_save", "kh_load_config", "kh_load",
@@ -96,6 +96,7 @@ def load_library(path=LIB_PATH):
         "kh_selftest_gemm3x": (I, [I, I, I, I, P, P, P, P, S, P]),
         "kh_selftest_wait_flag": (I, [P, I]),
         "kh_selftest_convert": (I, [I, P, P, P]),
+        "kh_selftest_gram": (I, [I, I, P, P, P, P, S, P]),
         "kh_selftest_permute": (I, [I, I, ctypes.POINTER(ctypes.c_longlong), ctypes.POINTER(I), P, P, P, S, P]),
         "kh_selftest_symeig": (I, [I, I, P, P, P, P, S, P]),
         "kh_selftest_svd": (I, [I, I, P, P, P, P, P, S, P]),
@@ -159,6 +160,22 @@ def selftest_gemm3x(A, B, a_colmajor=False):
     if st != KH_OK:
         raise KhError(st, "kh_selftest_gemm3x")
     return C
+
+
+def selftest_gram(A, B=None):
+    """A^T B (A^T A without B) of FP32 copies of FP64 CUDA tensors (n x k), summed
+    in FP32 over 16 rows and in FP64 beyond."""
+    import torch
+    n, k = A.shape
+    G = torch.empty((k, k), dtype=torch.float64, device=A.device)
+    nb = lib().kh_selftest_bytes(n, k, k)
+    scr = torch.empty(nb + 256, dtype=torch.uint8, device=A.device)
+    base = (scr.data_ptr() + 255) // 256 * 256
+    st = lib().kh_selftest_gram(n, k, _tptr(A.contiguous()), None if B is None else _tptr(B.contiguous()), _tptr(G),
+                                ctypes.c_void_p(base), nb, ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    if st != KH_OK:
+        raise KhError(st, "kh_selftest_gram")
+    return G
 
 
 def selftest_convert(x):

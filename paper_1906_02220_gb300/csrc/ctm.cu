@@ -315,9 +315,8 @@ __global__ void rand_kernel(T* V, long long tot, uint64_t seed, uint64_t stream)
 // Gram matrix G += Z^T Z2 (n x k row-major, Z2 = Z in the symmetric case): a CTA
 // takes one tile of 16 KT x 16 KT entries over a range of rows; thread (ti, tj)
 // of a 16 x 16 grid holds the entries (ti + 16 a, tj + 16 b).  FP32 products are
-// summed in FP32 over 16 rows and the sums of the chunks as unevaluated pairs of
-// FP32 numbers (two-sum, ~2^-47, which costs less here than FP64 additions),
-// then added to the FP64 result.  What bounds it is those FP64 atomics: k^2 a
+// summed in FP32 over 16 rows and those sums in FP64, which is added to the
+// result.  What bounds it is those FP64 atomics: k^2 a
 // range of rows, so the ranges are long (one CTA per SM over all tiles), and
 // the symmetric case computes the lower triangle of tiles only.  5184 x 160:
 // 19 us, with full ranges of 16 rows and k^2 atomics each 64; 1024 x 80: 6.6 and 9.5.
@@ -332,11 +331,12 @@ __global__ void __launch_bounds__(256) gram_kernel(const T* __restrict__ Z, cons
     const int i0 = bi * TS, j0 = bj * TS;
     const int rbeg = blockIdx.x * rows_cta, rend = min(n, rbeg + rows_cta);
     const int tid = threadIdx.x, ti = tid >> 4, tj = tid & 15;
-    T hi[KT][KT], lo[KT][KT], ra[KT], rb[KT];
+    T ra[KT], rb[KT];
+    double sum[KT][KT];
 #pragma unroll
     for (int a = 0; a < KT; ++a)
 #pragma unroll
-        for (int b = 0; b < KT; ++b) hi[a][b] = lo[a][b] = T(0);
+        for (int b = 0; b < KT; ++b) sum[a][b] = 0.0;
     auto load = [&](int r0) {
 #pragma unroll
         for (int q = 0; q < KT; ++q) {
@@ -377,15 +377,7 @@ __global__ void __launch_bounds__(256) gram_kernel(const T* __restrict__ Z, cons
 #pragma unroll
         for (int a = 0; a < KT; ++a)
 #pragma unroll
-            for (int b = 0; b < KT; ++b) {
-                if constexpr (sizeof(T) == 8) {
-                    hi[a][b] += acc[a][b];
-                } else {
-                    const T s = hi[a][b] + acc[a][b], d = s - hi[a][b];      // s + err = hi + acc exactly
-                    lo[a][b] += (hi[a][b] - (s - d)) + (acc[a][b] - d);
-                    hi[a][b] = s;
-                }
-            }
+            for (int b = 0; b < KT; ++b) sum[a][b] += f2d(acc[a][b]);
     }
 #pragma unroll
     for (int a = 0; a < KT; ++a)
@@ -393,9 +385,8 @@ __global__ void __launch_bounds__(256) gram_kernel(const T* __restrict__ Z, cons
         for (int b = 0; b < KT; ++b) {
             const int i = i0 + ti + 16 * a, j = j0 + tj + 16 * b;
             if (i < k && j < k) {
-                const double v = f2d(hi[a][b]) + f2d(lo[a][b]);
-                atomicAdd(&G[i * k + j], v);
-                if (SYM && bi != bj) atomicAdd(&G[j * k + i], v);
+                atomicAdd(&G[i * k + j], sum[a][b]);
+                if (SYM && bi != bj) atomicAdd(&G[j * k + i], sum[a][b]);
             }
         }
 }

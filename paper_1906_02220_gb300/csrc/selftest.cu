@@ -295,6 +295,22 @@ kh_status kh_selftest_permute(int kind, int rank, const long long* shape, const 
     });
 }
 
+kh_status kh_selftest_gram(int n, int k, const double* A, const double* Bm, double* G, void* scratch, size_t bytes,
+                           void* stream) {
+    if (n < 1 || k < 1 || !A || !G || !scratch) return KH_EINVAL;
+    if (bytes < kh_selftest_bytes(n, k, k)) return KH_ENOMEM;
+    cudaStream_t st = (cudaStream_t)stream;
+    return run([&] {
+        kh::Carver cv(scratch, bytes);
+        float* a = cv.take<float>((size_t)n * k);
+        float* b = cv.take<float>((size_t)n * k);
+        kh::cast<double, float>(A, a, (long long)n * k, st);
+        if (Bm) kh::cast<double, float>(Bm, b, (long long)n * k, st);
+        kh::gram2<float>(a, Bm ? b : nullptr, n, k, G, st);
+        KH_CUDA(cudaStreamSynchronize(st));
+    });
+}
+
 kh_status kh_selftest_convert(int n, const double* x, double* out, void* stream) {
     if (n < 1 || !x || !out) return KH_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;

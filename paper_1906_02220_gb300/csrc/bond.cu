@@ -193,7 +193,7 @@ __global__ void layered_img_kernel(const double* __restrict__ Tm, const double* 
         } else {
             float x = (float)v;
             if (npass == 3) {
-                const float h = __uint_as_float((__float_as_uint(x) + (P.fixed ? 0u : 0x1000u)) & 0xFFFFE000u);
+                const float h = tf32_head(x, P.fixed ? 0u : tf32_half(fabsf(x)));
                 x = hl == 0 ? h : x - h;
             }
             (ket ? img1 : img2)[e] = x;

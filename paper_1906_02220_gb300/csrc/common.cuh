@@ -74,6 +74,17 @@ inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cud
     count_launch();
 }
 
+// TF32 head of x for the operand splits x = head + (x - head): with half = kTf32Half
+// (half a unit of its last place) the nearest, with 0 the leading bits.  Rounding
+// must not make a finite value infinite (infinity - infinity is NaN):
+// tf32_half(m) is the half for values of magnitude m or less.  A NaN may lose its
+// head and stays in the remainder.
+constexpr uint32_t kTf32Half = 0x1000u;
+__device__ __forceinline__ uint32_t tf32_half(float m) { return __float_as_uint(m) < 0x7f7ff000u ? kTf32Half : 0u; }
+__device__ __forceinline__ float tf32_head(float x, uint32_t half) {
+    return __uint_as_float((__float_as_uint(x) + half) & 0xFFFFE000u);
+}
+
 // ------------------------------------------------------------------ workspace
 
 // Bump allocator over the caller's workspace; every block 256-byte aligned.
@@ -161,11 +172,10 @@ __global__ void permute32_kernel(const Ti* __restrict__ in, To* __restrict__ out
 }
 
 // Permutation fused with the 3xTF32 operand split: hi = the value rounded to
-// nearest TF32 (half = 0x1000, half a unit of its last place) or cut off there
-// (half = 0), lo = value - hi (32-bit path); the permuted value itself also goes
+// nearest TF32 or cut off there, lo = value - hi (32-bit path); the permuted value itself also goes
 // to out when out is not null.
 static __global__ void permute_split32_kernel(const float* __restrict__ in, float* __restrict__ hi,
-                                              float* __restrict__ lo, float* __restrict__ out, uint32_t half, PermArgs a) {
+                                              float* __restrict__ lo, float* __restrict__ out, bool nearest, PermArgs a) {
     pdl_start();
     const uint32_t total = (uint32_t)a.total;
     const uint32_t step = gridDim.x * blockDim.x;
@@ -180,7 +190,7 @@ static __global__ void permute_split32_kernel(const float* __restrict__ in, floa
             }
         }
         const float v = in[src];
-        const float h = __uint_as_float((__float_as_uint(v) + half) & 0xFFFFE000u);   // a NaN stays in lo
+        const float h = tf32_head(v, nearest ? tf32_half(fabsf(v)) : 0u);
         hi[idx] = h;
         lo[idx] = v - h;
         if (out) out[idx] = v;
@@ -267,7 +277,7 @@ constexpr int kTileMax = 2048, kTileGroupMax = 64;
 template <typename Ti, typename To, bool SPLIT>
 __global__ void __launch_bounds__(256)
 permute_tiled_kernel(const Ti* __restrict__ in, To* __restrict__ out, float* __restrict__ hi, float* __restrict__ lo,
-                     uint32_t half, TileArgs a) {
+                     bool nearest, TileArgs a) {
     pdl_start();
     __shared__ Ti tile[kTileMax + kTileMax / 32];
     __shared__ uint32_t off_in[kTileMax], off_out[kTileMax];
@@ -328,7 +338,7 @@ permute_tiled_kernel(const Ti* __restrict__ in, To* __restrict__ out, float* __r
             const Ti w = tile[p + (p >> 5)];
             if (x >= m) continue;
             if constexpr (SPLIT) {
-                const float h = __uint_as_float((__float_as_uint(w) + half) & 0xFFFFE000u);   // a NaN stays in lo
+                const float h = tf32_head(w, nearest ? tf32_half(fabsf(w)) : 0u);
                 hi[o] = h;
                 lo[o] = w - h;
             }
@@ -441,15 +451,14 @@ inline int tile_grid(const TileArgs& a) {
 inline void permute_split(const float* in, float* hi, float* lo, const std::vector<long long>& in_shape,
                           const std::vector<int>& order, cudaStream_t st, float* out = nullptr, bool nearest = true) {
     PermArgs a = make_perm(in_shape, order);
-    const uint32_t half = nearest ? 0x1000u : 0u;
     if (a.total <= 0) return;
     if (a.total >= (1LL << 31)) fail(KH_EINVAL, "permute_split: tensor too large");
     TileArgs t;
     if (make_tile_args(in_shape, order, t)) {
-        launch(permute_tiled_kernel<float, float, true>, tile_grid(t), 256, 0, st, in, out, hi, lo, half, t);
+        launch(permute_tiled_kernel<float, float, true>, tile_grid(t), 256, 0, st, in, out, hi, lo, nearest, t);
         return;
     }
-    launch(permute_split32_kernel, grid_for(a.total), 256, 0, st, in, hi, lo, out, half, a);
+    launch(permute_split32_kernel, grid_for(a.total), 256, 0, st, in, hi, lo, out, nearest, a);
 }
 
 template <typename Ti, typename To>
@@ -459,7 +468,7 @@ inline void permute(const Ti* in, To* out, const std::vector<long long>& in_shap
     if (a.total <= 0) return;
     TileArgs t;
     if (make_tile_args(in_shape, order, t)) {
-        launch(permute_tiled_kernel<Ti, To, false>, tile_grid(t), 256, 0, st, in, out, nullptr, nullptr, 0u, t);
+        launch(permute_tiled_kernel<Ti, To, false>, tile_grid(t), 256, 0, st, in, out, nullptr, nullptr, false, t);
         return;
     }
     if (a.total < (1LL << 31)) {

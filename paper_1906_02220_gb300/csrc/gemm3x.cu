@@ -90,12 +90,6 @@ __device__ __forceinline__ bool wait_all(uint64_t* bar, uint32_t parity, volatil
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
 }
 
-// nearest TF32 by the integer form of round-half-up; a NaN may come out as
-// zero here, but stays in the remainder x - hi
-__device__ __forceinline__ float tf32_near(float x) {
-    return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);
-}
-
 template <bool MMAJOR>
 __global__ void __launch_bounds__(THREADS, 1)
 gemm3x_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mBh,
@@ -289,6 +283,10 @@ gemm3x_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CU
                         x[4 * j + 3] = v.w;
                     }
                 }
+                float big = 0.f;
+#pragma unroll
+                for (int k = 0; k < BK; ++k) big = fmaxf(big, fabsf(x[k]));
+                const uint32_t half = tf32_half(big);
                 if (!wait_all(&bars.a_empty[a], ((it / ABUF) & 1) ^ 1, abort_flag)) { ok = false; break; }
                 fence_after();
                 const uint32_t dst = tmem + lane_base + C_A + a * 2 * BK;
@@ -297,7 +295,7 @@ gemm3x_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CU
                     float hi[16], lo[16];
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
-                        hi[i] = tf32_near(x[c0 + i]);
+                        hi[i] = tf32_head(x[c0 + i], half);
                         lo[i] = x[c0 + i] - hi[i];
                     }
                     tmem_st16(dst + c0, hi);
@@ -435,7 +433,7 @@ split_b_kernel(const float* __restrict__ B, long long sn, long long sk, int N, i
     for (int i = ly; i < 32; i += 8) {
         const int n = n0 + i, k = k0 + lx;
         if (n < N && k < K) {
-            const float v = t[i][lx], h = tf32_near(v);
+            const float v = t[i][lx], h = tf32_head(v, tf32_half(fabsf(v)));
             hi[(long long)n * ld + k] = h;
             lo[(long long)n * ld + k] = v - h;
         }

@@ -54,13 +54,6 @@ constexpr int WORKER0 = 4;                      // first worker warp (its tensor
 constexpr int THREADS = 32 * WORKER0 + 128 * NSET;
 constexpr int MAXST = 16;
 
-// TF32 head of v: nearest (a NaN may come out as zero, but stays in the remainder
-// v - hi), or with FIXED the leading bits
-template <bool FIXED>
-__device__ __forceinline__ float tf32_hi(float v) {
-    return __uint_as_float((__float_as_uint(v) + (FIXED ? 0u : 0x1000u)) & 0xFFFFE000u);
-}
-
 // instruction descriptor: FP32 accumulator, A and B TF32 (kind::tf32) or BF16
 // (kind::f16), K-major, N and M = 128
 constexpr uint32_t idesc(int n, bool bf16) {
@@ -310,11 +303,18 @@ layered_kernel(const float* __restrict__ Y, long long nb, int nc, const uint8_t*
         // npad columns on with 3 passes; or BF16 pairs, the lower index in the low half
         auto store_a = [&](uint32_t dst, auto npad_c, int lo_off, const float* v) {
             constexpr int NP = decltype(npad_c)::value;   // columns (a multiple of 8)
+            uint32_t half = 0;                            // heads to nearest, or in the fixed order the leading bits
+            if constexpr (NPASS == 3 && D > kFixedOrderD) {
+                float big = 0.f;
+#pragma unroll
+                for (int i = 0; i < NP; ++i) big = fmaxf(big, fabsf(v[i]));
+                half = tf32_half(big);
+            }
             auto col = [&](int c, bool lo) {
                 if constexpr (BF) return __uint_as_float(pack_bf16x2(v[2 * c], v[2 * c + 1]));
                 const float x = v[c];
                 if (NPASS != 3) return x;
-                const float h = tf32_hi<P.fixed>(x);
+                const float h = tf32_head(x, half);
                 return lo ? x - h : h;
             };
 #pragma unroll

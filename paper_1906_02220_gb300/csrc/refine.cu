@@ -150,16 +150,17 @@ __device__ __forceinline__ void newton_entry(const double* __restrict__ R, const
 // output tiles (grid-stride over the (k/8)^2 tiles) with 256 threads: four
 // groups of 64 split each k-long FP64 dot product into quarters (shorter
 // dependent chains, all four SM sub-partitions busy), the partial sums joined
-// in shared memory in a fixed order.  Two phases per step, separated by grid
-// barriers: R, P and T = L^T B with B = G Q; then L' = L + L F, Q' = Q + Q H and
-// B' = B + B H with the corrections F, H formed on the fly from R, P, T for the
-// tile's column slab.  Carrying B instead of forming (L^T G) Q saves a phase of
-// the three, and the phases' latency (barrier, loads) is what bounds the launch.
+// in shared memory in a fixed order.  Three phases per step, separated by
+// grid barriers: R, P, W = L^T G; T = W Q; L' = L + L F and Q' = Q + Q H with
+// the corrections F, H formed on the fly from R, P, T for the tile's column
+// slab.  (B = G Q carried along as B' = B + B H saves a phase, but on matrices of
+// low rank with a tail at rounding level, as product-like states give, T then
+// drifts from L^T G Q and single factors came out as large as 1e6.)
 // Operands are staged as 8-wide slabs in shared memory (the FP64 pipe
 // then runs from shared memory).  The factors ping-pong between (L1, Q1) and
 // (Lo, Qo).  The single-precision factors are read (and the refined ones
-// rounded back to them) in place when Lf, Qf are given.  k = 80: 99 us as
-// before, but the four casts around the launch, 3 us each, are gone.
+// rounded back to them) in place when Lf, Qf are given: the four casts that would
+// stand around the launch take 3 us each.
 constexpr int kRT = 8;                                     // tile edge
 constexpr int kRQ = 4;                                     // K split
 constexpr int kRThreads = kRT * kRT * kRQ;
@@ -170,8 +171,8 @@ refine_coop_kernel(const double* __restrict__ G, int k, const double* L0, const 
     cg::grid_group grid = cg::this_grid();
     extern __shared__ double slab[];                       // 5 slabs of 8 x k, then 3 x kRQ x 64 partial sums
     const long long kk = (long long)k * k;
-    double *R = work, *P = work + kk, *T = work + 3 * kk, *Ba = work + 4 * kk, *Bb = work + 5 * kk,
-           *L1 = work + 6 * kk, *Q1 = work + 7 * kk;
+    double *R = work, *P = work + kk, *W = work + 2 * kk, *T = work + 3 * kk, *L1 = work + 6 * kk,
+           *Q1 = work + 7 * kk;
     const int nt = (k + kRT - 1) / kRT, ntiles = nt * nt;
     const int tid = threadIdx.x, q = tid / (kRT * kRT), e64 = tid % (kRT * kRT), ti = e64 / kRT, tj = e64 % kRT;
     const int mq0 = q * k / kRQ, mq1 = (q + 1) * k / kRQ;  // this group's part of the sum
@@ -218,31 +219,15 @@ refine_coop_kernel(const double* __restrict__ G, int k, const double* L0, const 
         return x;
     };
     const int nsteps = newton_steps + 1;
-    // phase 0: B = G Q
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const int i0 = (t / nt) * kRT, j0 = (t % nt) * kRT;
-        __syncthreads();
-        load_rows(s0, G, i0);
-        if (Qf) load_cols(s1, (const float*)Qf, j0);
-        else load_cols(s1, Q0, j0);
-        __syncthreads();
-        red[q * 64 + e64] = dot(s0, s1);
-        __syncthreads();
-        const int i = i0 + ti, j = j0 + tj;
-        if (q == 0 && i < k && j < k) Ba[i * k + j] = joined(0);
-    }
-    grid.sync();
     for (int step = 0; step < nsteps; ++step) {
         const int rem = nsteps - 1 - step;                 // steps after this one; the last writes (Lo, Qo)
         const bool single = step == 0 && Lf;               // the factors come in single precision
         const double* Li = step == 0 ? L0 : ((rem % 2 == 0) ? L1 : Lo);
         const double* Qi = step == 0 ? Q0 : ((rem % 2 == 0) ? Q1 : Qo);
-        const double* Bi = step % 2 == 0 ? Ba : Bb;
-        double* Bn = step % 2 == 0 ? Bb : Ba;
         double* Ln = (rem % 2 == 0) ? Lo : L1;
         double* Qn = (rem % 2 == 0) ? Qo : Q1;
         const double gap = step < newton_steps ? rel_gap : INFINITY;
-        // phase 1: R = I - L^T L, P = I - Q^T Q, T = L^T B on tile (I, J)
+        // phase 1: R = I - L^T L, P = I - Q^T Q, W = L^T G on tile (I, J)
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
             const int i0 = (t / nt) * kRT, j0 = (t % nt) * kRT;
             __syncthreads();
@@ -257,7 +242,7 @@ refine_coop_kernel(const double* __restrict__ G, int k, const double* L0, const 
                 load_cols(s2, Qi, i0);
                 load_cols(s3, Qi, j0);
             }
-            load_cols(s4, Bi, j0);
+            load_cols(s4, G, j0);
             __syncthreads();
             red[(0 * kRQ + q) * 64 + e64] = dot(s0, s1);
             red[(1 * kRQ + q) * 64 + e64] = dot(s2, s3);
@@ -268,8 +253,22 @@ refine_coop_kernel(const double* __restrict__ G, int k, const double* L0, const 
                 const double d = (i == j) ? 1.0 : 0.0;
                 R[i * k + j] = d - joined(0);
                 P[i * k + j] = d - joined(1);
-                T[i * k + j] = joined(2);
+                W[i * k + j] = joined(2);
             }
+        }
+        grid.sync();
+        // phase 2: T = W Q
+        for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+            const int i0 = (t / nt) * kRT, j0 = (t % nt) * kRT;
+            __syncthreads();
+            load_rows(s0, W, i0);
+            if (single) load_cols(s1, (const float*)Qf, j0);
+            else load_cols(s1, Qi, j0);
+            __syncthreads();
+            red[q * 64 + e64] = dot(s0, s1);
+            __syncthreads();
+            const int i = i0 + ti, j = j0 + tj;
+            if (q == 0 && i < k && j < k) T[i * k + j] = joined(0);
         }
         grid.sync();
         // refined singular values (one CTA)
@@ -278,8 +277,8 @@ refine_coop_kernel(const double* __restrict__ G, int k, const double* L0, const 
                 const long long e = (long long)i * k + i;
                 s_out[i] = T[e] * (1.0 + 0.5 * (R[e] + P[e]));
             }
-        // phase 2: L' = L + L F, Q' = Q + Q H, B' = B + B H, the corrections of
-        // the tile's column slab formed from R, P, T
+        // phase 3: L' = L + L F, Q' = Q + Q H, the corrections of the tile's
+        // column slab formed from R, P, T
         const bool last = rem == 0;
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
             const int i0 = (t / nt) * kRT, j0 = (t % nt) * kRT;
@@ -291,7 +290,6 @@ refine_coop_kernel(const double* __restrict__ G, int k, const double* L0, const 
                 load_rows(s0, Li, i0);
                 load_rows(s2, Qi, i0);
             }
-            if (!last) load_rows(s4, Bi, i0);
             for (int e = tid; e < kRT * k; e += kRThreads) {
                 const int m = e / kRT, j = j0 + e % kRT;
                 double f = 0.0, h = 0.0;
@@ -302,15 +300,13 @@ refine_coop_kernel(const double* __restrict__ G, int k, const double* L0, const 
             __syncthreads();
             red[(0 * kRQ + q) * 64 + e64] = dot(s0, s1);
             red[(1 * kRQ + q) * 64 + e64] = dot(s2, s3);
-            if (!last) red[(2 * kRQ + q) * 64 + e64] = dot(s4, s3);
             __syncthreads();
             const int i = i0 + ti, j = j0 + tj;
             if (q == 0 && i < k && j < k) {
-                // the old entries from the staged rows (s0, s2, s4 at column j of row i)
+                // the old entries from the staged rows (s0, s2 at column j of row i)
                 const double l = s0[j * kRT + ti] + joined(0), qv = s2[j * kRT + ti] + joined(1);
                 Ln[i * k + j] = l;
                 Qn[i * k + j] = qv;
-                if (!last) Bn[i * k + j] = s4[j * kRT + ti] + joined(2);
                 if (last && Lf) {
                     Lf[i * k + j] = d2f(l);
                     Qf[i * k + j] = d2f(qv);

@@ -433,6 +433,11 @@ kh_status kh_selftest_symeig(int prec, int k, const double* dev_G, double* dev_W
 kh_status kh_selftest_svd(int prec, int k, const double* dev_X, double* dev_S, double* dev_L, double* dev_Q,
                           void* dev_scratch, size_t scratch_bytes, void* stream);
 
+/* As kh_selftest_svd, iterated until the n_top largest triplets have converged
+ * (1 <= n_top <= k), as the projector asks for its kept directions. */
+kh_status kh_selftest_svd_top(int prec, int k, int n_top, const double* dev_X, double* dev_S, double* dev_L,
+                              double* dev_Q, void* dev_scratch, size_t scratch_bytes, void* stream);
+
 /* The projector SVD of the FP64-projector option (kh_config.proj_fp64) on a
  * k x k FP64 matrix X (k <= 160): the FP32 one-sided Jacobi SVD followed by
  * three FP64 Newton refinement steps and a re-orthogonalisation (first-order corrections L' = L (I + F),
@@ -442,6 +447,25 @@ kh_status kh_selftest_svd(int prec, int k, const double* dev_X, double* dev_S, d
  * vectors).  Scratch as for kh_selftest_svd.  Synchronises stream. */
 kh_status kh_selftest_svd_refined(int k, const double* dev_X, double* dev_S, double* dev_L, double* dev_Q,
                                   void* dev_scratch, size_t scratch_bytes, void* stream);
+
+/* The same with the FP32 factors refined in place, as the projector runs it:
+ * dev_L, dev_Q receive the refined factors rounded to FP32. */
+kh_status kh_selftest_svd_refined_in_place(int k, const double* dev_X, double* dev_S, double* dev_L, double* dev_Q,
+                                           void* dev_scratch, size_t scratch_bytes, void* stream);
+
+/* Warm start of a small single-precision basis (n <= 2048, k <= 96): columns of
+ * the n x k matrix V whose entry of live (k values, 0 or 1) is 1 stay, the others
+ * become random vectors projected (twice) off the live ones, which are taken
+ * to be orthonormal.  Scratch as kh_selftest_orth.  Synchronises stream. */
+kh_status kh_selftest_warm_basis(int n, int k, const double* dev_V, const double* dev_live, double* dev_out,
+                                 void* dev_scratch, size_t scratch_bytes, void* stream);
+
+/* dev_Y (n x k) = the FP32 sum, in order, of `parts` (at most 24) FP32 copies of
+ * the n x k blocks at dev_P, and dev_G = Y^T Y (k x k), by the pass that joins a
+ * split product of such a basis.  Scratch as kh_selftest_orth.  Synchronises
+ * stream. */
+kh_status kh_selftest_join_parts(int n, int k, int parts, const double* dev_P, double* dev_Y, double* dev_G,
+                                 void* dev_scratch, size_t scratch_bytes, void* stream);
 
 /* Orthonormal basis of the columns of an n x k FP64 matrix Y (row-major) by
  * the library's ordered CholQR2 (two Cholesky-QR passes, columns taken in

@@ -26,7 +26,8 @@ ABI_FUNCTIONS = [
     "kh_set_state", "kh_get_state", "ctm_set_tensor", "ctm_build_composite", "ctm_init",
     "ctm_copy_env", "ctm_sweep", "ctm_projectors", "ctm_get_env", "ctm_metric", "ctm_kappa",
     "ctm_expval", "ctm_correlation_length", "ctm_plaquette", "ctm_flux", "eefu_apply_gate", "eefu_cost_gradient", "observables", "kh_version", "kh_bond_hamiltonian", "kh_gate", "kh_flux_operators",
-    "eefu_trotter_step", "eefu_evolve", "eefu_evolve_flux", "eefu_evolve_batch", "kh_launch_count", "kh_profile", "kh_selftest_bytes", "kh_selftest_gemm", "kh_selftest_gemm3x", "kh_selftest_wait_flag", "kh_selftest_convert", "kh_selftest_gram", "kh_selftest_permute",
+    "eefu_trotter_step", "eefu_evolve", "eefu_evolve_flux", "eefu_evolve_batch", "kh_launch_count", "kh_profile", "kh_selftest_bytes", "kh_selftest_gemm", "kh_selftest_gemm3x", "kh_selftest_wait_flag", "kh_selftest_convert", "kh_selftest_gram", "kh_selftest_svd_top", "kh_selftest_svd_refined_in_place",
+    "kh_selftest_warm_basis", "kh_selftest_join_parts", "kh_selftest_permute",
     "kh_selftest_symeig", "kh_selftest_svd", "kh_selftest_svd_refined", "kh_selftest_orth", "kh_selftest_fp64_newton",
     "kh_selftest_site_layered_bytes", "kh_selftest_site_layered", "kh_gemm_noalloc",
     "kh_gemm_noalloc_max_bytes", "kh_save", "kh_load_config", "kh_load",
@@ -102,6 +103,10 @@ def load_library(path=LIB_PATH):
         "kh_selftest_svd": (I, [I, I, P, P, P, P, P, S, P]),
         "kh_selftest_orth": (I, [I, I, I, D, P, P, P, S, P]),
         "kh_selftest_svd_refined": (I, [I, P, P, P, P, P, S, P]),
+        "kh_selftest_svd_refined_in_place": (I, [I, P, P, P, P, P, S, P]),
+        "kh_selftest_svd_top": (I, [I, I, I, P, P, P, P, P, S, P]),
+        "kh_selftest_warm_basis": (I, [I, I, P, P, P, P, S, P]),
+        "kh_selftest_join_parts": (I, [I, I, I, P, P, P, P, S, P]),
         "kh_selftest_fp64_newton": (I, [I, P, P, P]),
         "kh_selftest_site_layered_bytes": (S, [I, I, I, ctypes.c_longlong]),
         "kh_selftest_site_layered": (I, [I, I, I, I, I, ctypes.c_longlong, P, P, P, P, S, P]),
@@ -256,6 +261,57 @@ def selftest_svd_refined(X):
     if st != KH_OK:
         raise KhError(st, "kh_selftest_svd_refined")
     return S, L, Q
+
+
+def _selftest(name, n, k, device, *args):
+    """Calls a self-test entry point whose scratch is that of an n x k x k product."""
+    import torch
+    nb = lib().kh_selftest_bytes(n, k, k)
+    scr = torch.empty(nb + 256, dtype=torch.uint8, device=device)
+    base = (scr.data_ptr() + 255) // 256 * 256
+    st = getattr(lib(), name)(*args, ctypes.c_void_p(base), nb,
+                              ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    if st != KH_OK:
+        raise KhError(st, name)
+
+
+def selftest_svd_top(X, n_top, prec="fp64"):
+    """(S, L, Q) as selftest_svd, iterated until the n_top largest have converged."""
+    import torch
+    k = X.shape[0]
+    S, L, Q = torch.empty(k, dtype=torch.float64, device=X.device), torch.empty_like(X), torch.empty_like(X)
+    _selftest("kh_selftest_svd_top", k, k, X.device, PREC[prec], k, n_top, _tptr(X), _tptr(S), _tptr(L), _tptr(Q))
+    return S, L, Q
+
+
+def selftest_svd_refined_in_place(X):
+    """(S, L, Q) as selftest_svd_refined with the FP32 factors refined in place:
+    L and Q are the refined ones rounded to FP32."""
+    import torch
+    k = X.shape[0]
+    S, L, Q = torch.empty(k, dtype=torch.float64, device=X.device), torch.empty_like(X), torch.empty_like(X)
+    _selftest("kh_selftest_svd_refined_in_place", k, k, X.device, k, _tptr(X), _tptr(S), _tptr(L), _tptr(Q))
+    return S, L, Q
+
+
+def selftest_warm_basis(V, live):
+    """The warm start of a small basis: V's live columns (live: k zeros and ones,
+    FP64), random vectors projected off them in place of the others."""
+    import torch
+    out = torch.empty_like(V)
+    _selftest("kh_selftest_warm_basis", V.shape[0], V.shape[1], V.device, V.shape[0], V.shape[1], _tptr(V), _tptr(live),
+              _tptr(out))
+    return out
+
+
+def selftest_join_parts(P):
+    """(sum over parts, its Gram matrix) of P (parts, n, k), summed in FP32 in order."""
+    import torch
+    parts, n, k = P.shape
+    Y = torch.empty((n, k), dtype=torch.float64, device=P.device)
+    G = torch.empty((k, k), dtype=torch.float64, device=P.device)
+    _selftest("kh_selftest_join_parts", n, k, P.device, n, k, parts, _tptr(P), _tptr(Y), _tptr(G))
+    return Y, G
 
 
 def selftest_site_layered(T, Y, kind=0, frame=0, npass=3):

@@ -96,14 +96,15 @@ void run_eig(int k, const double* G, double* W, double* E, void* scratch, size_t
 }
 
 template <typename T>
-void run_svd(int k, const double* X, double* S, double* L, double* Qm, void* scratch, size_t bytes, cudaStream_t st) {
+void run_svd(int k, int nrel, const double* X, double* S, double* L, double* Qm, void* scratch, size_t bytes,
+             cudaStream_t st) {
     kh::Carver cv(scratch, bytes);
     T* x = cv.take<T>((size_t)k * k);
     T* l = cv.take<T>((size_t)k * k);
     T* q = cv.take<T>((size_t)k * k);
     T* sv = cv.take<T>((size_t)k);
     kh::cast<double, T>(X, x, (long long)k * k, st);
-    kh::svd_jacobi<T>(x, k, sv, l, q, 60, sizeof(T) == 8 ? 1e-15 : 1e-6, 0.0, st);
+    kh::svd_jacobi<T>(x, k, sv, l, q, 60, sizeof(T) == 8 ? 1e-15 : 1e-6, 0.0, st, nullptr, nrel);
     kh::cast<T, double>(sv, S, (long long)k, st);
     kh::cast<T, double>(l, L, (long long)k * k, st);
     kh::cast<T, double>(q, Qm, (long long)k * k, st);
@@ -168,8 +169,8 @@ void run_site_layered(int npass, int D, int p, int kind, int frame, long long nb
 
 // FP32 one-sided Jacobi, then one FP64 Newton refinement step (the projector
 // SVD of the FP64-projector option).
-void run_svd_refined(int k, const double* X, double* S, double* L, double* Qm, void* scratch, size_t bytes,
-                     cudaStream_t st) {
+void run_svd_refined(int k, bool in_place, const double* X, double* S, double* L, double* Qm, void* scratch,
+                     size_t bytes, cudaStream_t st) {
     kh::Carver cv(scratch, bytes);
     float* x = cv.take<float>((size_t)k * k);
     float* l = cv.take<float>((size_t)k * k);
@@ -180,6 +181,12 @@ void run_svd_refined(int k, const double* X, double* S, double* L, double* Qm, v
     double* work = cv.take<double>(kh::svd_refine_scratch(k));
     kh::cast<double, float>(X, x, (long long)k * k, st);
     kh::svd_jacobi<float>(x, k, sv, l, q, 60, 1e-6, 0.0, st);
+    if (in_place) {
+        kh::svd_refine_fp64(X, k, ld, qd, S, L, Qm, work, 1e-5, st, l, q);
+        kh::cast<float, double>(l, L, (long long)k * k, st);
+        kh::cast<float, double>(q, Qm, (long long)k * k, st);
+        return;
+    }
     kh::cast<float, double>(l, ld, (long long)k * k, st);
     kh::cast<float, double>(q, qd, (long long)k * k, st);
     kh::svd_refine_fp64(X, k, ld, qd, S, L, Qm, work, 1e-5, st);
@@ -339,8 +346,72 @@ kh_status kh_selftest_svd(int prec, int k, const double* X, double* S, double* L
     if (bytes < kh_selftest_bytes(k, k, k)) return KH_ENOMEM;
     cudaStream_t st = (cudaStream_t)stream;
     return run([&] {
-        if (prec == KH_FP64) run_svd<double>(k, X, S, L, Qm, scratch, bytes, st);
-        else run_svd<float>(k, X, S, L, Qm, scratch, bytes, st);
+        if (prec == KH_FP64) run_svd<double>(k, 0, X, S, L, Qm, scratch, bytes, st);
+        else run_svd<float>(k, 0, X, S, L, Qm, scratch, bytes, st);
+        KH_CUDA(cudaStreamSynchronize(st));
+    });
+}
+
+kh_status kh_selftest_svd_top(int prec, int k, int n_top, const double* X, double* S, double* L, double* Qm,
+                              void* scratch, size_t bytes, void* stream) {
+    if (k < 1 || n_top < 1 || n_top > k || !X || !S || !L || !Qm || !scratch) return KH_EINVAL;
+    if (bytes < kh_selftest_bytes(k, k, k)) return KH_ENOMEM;
+    cudaStream_t st = (cudaStream_t)stream;
+    return run([&] {
+        if (prec == KH_FP64) run_svd<double>(k, n_top, X, S, L, Qm, scratch, bytes, st);
+        else run_svd<float>(k, n_top, X, S, L, Qm, scratch, bytes, st);
+        KH_CUDA(cudaStreamSynchronize(st));
+    });
+}
+
+kh_status kh_selftest_svd_refined_in_place(int k, const double* X, double* S, double* L, double* Qm, void* scratch,
+                                           size_t bytes, void* stream) {
+    if (k < 1 || k > 160 || !X || !S || !L || !Qm || !scratch) return KH_EINVAL;
+    if (bytes < kh_selftest_bytes(k, k, k)) return KH_ENOMEM;
+    cudaStream_t st = (cudaStream_t)stream;
+    return run([&] {
+        run_svd_refined(k, true, X, S, L, Qm, scratch, bytes, st);
+        KH_CUDA(cudaStreamSynchronize(st));
+    });
+}
+
+kh_status kh_selftest_warm_basis(int n, int k, const double* V, const double* live, double* out, void* scratch,
+                                 size_t bytes, void* stream) {
+    if (n < 1 || k < 1 || !V || !live || !out || !scratch || !kh::rows_usable(n, k)) return KH_EINVAL;
+    if (bytes < kh_selftest_bytes(n, k, k)) return KH_ENOMEM;
+    cudaStream_t st = (cudaStream_t)stream;
+    return run([&] {
+        kh::Carver cv(scratch, bytes);
+        float* v = cv.take<float>((size_t)n * k);
+        float* vl = cv.take<float>((size_t)n * k);
+        float* r = cv.take<float>((size_t)n * k);
+        int* mask = cv.take<int>((size_t)k);
+        double* g = cv.take<double>(2 * (size_t)k * k);
+        KH_CUDA(cudaMemsetAsync(g, 0, sizeof(double) * 2 * k * k, st));
+        kh::cast<double, float>(V, v, (long long)n * k, st);
+        kh::cast<double, int>(live, mask, k, st);
+        kh::rows_split(v, mask, n, k, vl, r, 1, 2, g, st);
+        kh::rows_project(vl, g, n, k, r, g + k * k, st);
+        kh::rows_project(vl, g + k * k, n, k, r, nullptr, st);
+        kh::cast<float, double>(r, out, (long long)n * k, st);
+        KH_CUDA(cudaStreamSynchronize(st));
+    });
+}
+
+kh_status kh_selftest_join_parts(int n, int k, int parts, const double* P, double* Y, double* G, void* scratch,
+                                 size_t bytes, void* stream) {
+    if (n < 1 || k < 1 || parts < 1 || parts > 24 || !P || !Y || !G || !scratch || !kh::rows_usable(n, k))
+        return KH_EINVAL;
+    if (bytes < kh_selftest_bytes(n, k, k)) return KH_ENOMEM;
+    cudaStream_t st = (cudaStream_t)stream;
+    return run([&] {
+        kh::Carver cv(scratch, bytes);
+        float* p = cv.take<float>((size_t)parts * n * k);
+        float* y = cv.take<float>((size_t)n * k);
+        KH_CUDA(cudaMemsetAsync(G, 0, sizeof(double) * k * k, st));
+        kh::cast<double, float>(P, p, (long long)parts * n * k, st);
+        kh::rows_reduce(p, parts, n, k, y, G, st);
+        kh::cast<float, double>(y, Y, (long long)n * k, st);
         KH_CUDA(cudaStreamSynchronize(st));
     });
 }
@@ -351,7 +422,7 @@ kh_status kh_selftest_svd_refined(int k, const double* X, double* S, double* L, 
     if (bytes < kh_selftest_bytes(k, k, k)) return KH_ENOMEM;
     cudaStream_t st = (cudaStream_t)stream;
     return run([&] {
-        run_svd_refined(k, X, S, L, Qm, scratch, bytes, st);
+        run_svd_refined(k, false, X, S, L, Qm, scratch, bytes, st);
         KH_CUDA(cudaStreamSynchronize(st));
     });
 }

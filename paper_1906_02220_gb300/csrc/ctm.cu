@@ -1539,14 +1539,14 @@ void svd_jacobi(const T* X, int k, T* sv, T* L, T* Qm, int max_sweeps, double to
     }
 #define KH_SVDJ(LP, R) svd_jacobi_launch<T, LP, R>(X, k, sv, L, Qm, max_sweeps, tol, cut, st, sweep_count, nrel)
     if (kp <= 16) KH_SVDJ(8, 2);
-    else if (kp <= 32) KH_SVDJ(8, 4);
-    else if (kp <= 48) KH_SVDJ(8, 6);
-    else if (kp <= 64) KH_SVDJ(8, 8);
-    else if (kp <= 80) KH_SVDJ(8, 10);
-    else if (kp <= 96) KH_SVDJ(8, 12);
-    else if (kp <= 112) KH_SVDJ(8, 14);
-    else if constexpr (sizeof(T) == 4) {     // FP64 stops at k = 112
-        if (kp <= 128) KH_SVDJ(8, 16);
+    else if constexpr (sizeof(T) == 4) {
+        if (kp <= 32) KH_SVDJ(8, 4);
+        else if (kp <= 48) KH_SVDJ(8, 6);
+        else if (kp <= 64) KH_SVDJ(8, 8);
+        else if (kp <= 80) KH_SVDJ(8, 10);
+        else if (kp <= 96) KH_SVDJ(8, 12);
+        else if (kp <= 112) KH_SVDJ(8, 14);
+        else if (kp <= 128) KH_SVDJ(8, 16);
         else if (kp <= 144) KH_SVDJ(8, 18);
         else KH_SVDJ(8, 20);
     }

@@ -96,16 +96,6 @@ __device__ __forceinline__ void umma_tf32_tmem_a(uint32_t by, uint32_t tmem_d, u
         ::"r"(tmem_d), "r"(tmem_a), "l"(db), "r"(idesc), "r"(acc), "r"(by)
         : "memory");
 }
-__device__ __forceinline__ void umma_f16(uint32_t by, uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc,
-                                            uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "setp.ne.b32 q, %5, 0;\n\t"
-        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
-        ::"r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(acc), "r"(by)
-        : "memory");
-}
 __device__ __forceinline__ void umma_f16_tmem_a(uint32_t by, uint32_t tmem_d, uint32_t tmem_a, uint64_t db, uint32_t idesc,
                                             uint32_t acc) {
     asm volatile(

@@ -506,6 +506,12 @@ struct GemmArgs {
     const T* colscale;   // nullable, length N
     T* sk = nullptr;     // optional split-K scratch (for few output tiles and long K)
     long long sk_elems = 0;
+    // started without programmatic launch: where a kernel of many CTAs comes before,
+    // the CTAs of a product that does not fill the GPU would be set up in pairs on
+    // the SMs that drain first, and stay there (bond metric at (5, 144): 100 CTAs of
+    // 1.1 ms; the gradient took 2.61 ms so, 1.87 with an ordinary launch, 0.90 and
+    // 0.57 at (5, 64))
+    bool plain = false;
 };
 
 constexpr int GT_K = 16;
@@ -718,6 +724,11 @@ template <typename T, int BM, int BN, int TM, int TN>
 inline void gemm_launch(const GemmArgs<T>& g, cudaStream_t st) {
     dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.batch);
     if (grid.y > 65535) fail(KH_EINVAL, "gemm M too large");
+    if (g.plain && (long long)grid.x * grid.y * grid.z < 2 * 152) {
+        gemm_simt_kernel<T, BM, BN, TM, TN><<<grid, 256, 0, st>>>(g);
+        KH_LAUNCHED();
+        return;
+    }
     launch(gemm_simt_kernel<T, BM, BN, TM, TN>, grid, 256, 0, st, g);
 }
 
@@ -822,10 +833,11 @@ inline GemmArgs<T> rm_args(int M, int N, int K, const T* A, bool tA, const T* B,
 template <typename T>
 inline void gemm_rm(int M, int N, int K, const T* A, bool tA, const T* B, bool tB, T* C,
                     cudaStream_t st, T alpha = T(1), T beta = T(0), const T* colscale = nullptr,
-                    T* sk = nullptr, long long sk_elems = 0) {
+                    T* sk = nullptr, long long sk_elems = 0, bool plain = false) {
     GemmArgs<T> g = rm_args<T>(M, N, K, A, tA, B, tB, C);
     g.sk = sk;
     g.sk_elems = sk_elems;
+    g.plain = plain;
     g.alpha = alpha; g.beta = beta; g.colscale = colscale;
     gemm(g, st);
 }

@@ -1411,7 +1411,7 @@ void Engine<T>::compute_metric(Slot<T>& sl, double* N_out) {
     if (!joined) {
         permute<T, T>(mdn, mdnp, {chi, D, D, D, D, chi}, {5, 0, 1, 2, 3, 4}, st);   // [h][e][dk][db][lk][lb]
         gemm_rm<T>(d2 * d2, d2 * d2, chi * chi, mupp, false, mdnp, false, mN4, st, T(1), T(0), nullptr, skbuf,
-                   sk_elems);
+                   sk_elems, true);
     }
     permute<T, double>(mN4, N_out, {D, D, D, D, D, D, D, D}, {6, 0, 2, 4, 7, 1, 3, 5}, st);
     launch(symmetrize_kernel, grid_for((long long)dm.D4 * dm.D4), 256, 0, st, N_out, dm.D4);

@@ -71,6 +71,12 @@ typedef enum {
                            BF16 operands (one pass), FP32 accumulate; the
                            half-system product TF32 (one pass)                  */
 } kh_prec;
+/* In KH_TF32 and KH_BF16, and in KH_TF32X3 from D = 6 on, the other wide products
+ * of a move and of the metric run with the split as well; in KH_FP32 and
+ * KH_TF32X3 up to D = 5 they are FP32 on the CUDA cores, and every sum of a move
+ * keeps one order, so that bond costs stay comparable (the scale of an
+ * environment depends on which directions pass svd_cut, and near the cut on
+ * rounding). */
 
 typedef struct kh_config {
     int D;                   /* bond dimension, 1 <= D <= 8                           */

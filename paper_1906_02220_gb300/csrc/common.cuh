@@ -49,10 +49,11 @@ inline void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed);
 // Programmatic dependent launch: a kernel launched with launch() may be set up on
 // the SMs while its predecessor in the stream still drains; pdl_start() at its
 // top waits until that one is complete and its writes are visible, then lets
-// the next one be set up.  Small moves are a chain of 70 short kernels: the
-// environment of (D, chi) = (4, 64) went from 12.84 to 11.33 ms, of (3, 32) in FP64
-// from 13.71 to 12.38, of (6, 144) from 83.4 to 81.0, the bond gradient from 298 to
-// 267 us.  Kernels started with <<<>>> are ordered as ever, and pdl_start() returns
+// the next one be set up.  Small moves are a chain of 70 short kernels: when it
+// came in, the environment of (D, chi) = (4, 64) went from 12.84 to 11.33 ms, of
+// (3, 32) in FP64 from 13.71 to 12.38, of (6, 144) from 83.4 to 81.0, the bond gradient
+// from 407 to 379 us.  Where a wide kernel precedes a product of few long CTAs it
+// does harm (GemmArgs::plain).  Kernels started with <<<>>> are ordered as ever, and pdl_start() returns
 // at once in them.
 __device__ __forceinline__ void pdl_start() {
     asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -66,9 +66,9 @@ Dims make_dims(const kh_config& c, bool fp64) {
     // order, each no less accurate; at D = 3 of 0 in 44.  Trial costs are compared
     // across runs and with stored ones, so the FP32-accurate modes keep one order
     // and rounding up to D = 5, the sizes of gradient-based bond optimisation.
-    // What that gives up at (4, 64): the environment takes 12.5 ms, with the other
-    // forms 11.3.
-    // From D = 6 on the tensor-core products halve the time of a move.
+    // What that gives up at (4, 64): the environment takes 12.6 ms, with the other
+    // forms 11.3.  From D = 6 on the tensor-core products halve
+    // the time of a move, and the other forms are kept.
     d.fixed_order = !fp64 && d.npass != 1 && c.D <= lay::kFixedOrderD;
     int kmax = fp64 ? 112 : 160;      // the one-CTA Jacobi limits (FP64, FP32)
     if (d.n <= kmax) {
@@ -319,7 +319,8 @@ __global__ void rand_kernel(T* V, long long tot, uint64_t seed, uint64_t stream)
 // result.  What bounds it is those FP64 atomics: k^2 a
 // range of rows, so the ranges are long (one CTA per SM over all tiles), and
 // the symmetric case computes the lower triangle of tiles only.  5184 x 160:
-// 19 us, with full ranges of 16 rows and k^2 atomics each 64; 1024 x 80: 6.6 and 9.5.
+// 29 us (a third of it the FP64 sums), with full ranges of 16 rows and k^2 atomics
+// each 64; 1024 x 80: 6.9 and 9.5.
 template <typename T, int KT, bool SYM>
 __global__ void __launch_bounds__(256) gram_kernel(const T* __restrict__ Z, const T* __restrict__ Z2, int n, int k,
                                                    int nt, double* __restrict__ G, int rows_cta) {
@@ -1395,9 +1396,10 @@ void Engine<T>::compute_metric(Slot<T>& sl, double* N_out) {
     // K = chi^2.  On the tensor cores it is the more accurate one as well, relative
     // to FP64 (Frobenius): 256 x 256 x 4096 1.6e-7 against 1.1e-6, 1296 x 1296 x 20736
     // 3.0e-7 against 2.6e-6.  Time on the CUDA cores: 2.8 ms at (6, 144), 24 at
-    // (8, 144), of environments of 81 and 284 that went to 78 and 262; at (5, 100),
-    // 7.8e9 flops, the environment went from 24.2 to 23.7 ms, at (4, 64), 5e8 flops in
-    // a K split over the SMs, it stayed at 11.3.  The line lies between.
+    // (8, 144), of environments of 81 and 284 that went to 78 and 262; at (5, 100) in
+    // BF16, 7.8e9 flops, the environment went from 24.2 to 23.7 ms, at (4, 64), 5e8 flops
+    // in a K split over the SMs, it stayed the same.  The line lies between.  (The fixed
+    // order stays on the CUDA cores at every size.)
     constexpr double kMinMetric3x = 1e9;
     bool joined = false;
     if constexpr (sizeof(T) == 4) {

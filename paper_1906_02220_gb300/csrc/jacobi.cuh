@@ -785,8 +785,10 @@ cholqr_kernel(double* __restrict__ G, int k, double cut_abs, double tau, T* __re
 // rows (one warp each) go to shared memory; one thread per column eliminates
 // within the 4 x 4 block and carries the column through it (y; by symmetry also
 // a_ij, scaled to z); then every thread subtracts four products per entry.  What
-// bounds it is that chain: two barriers, four reciprocals.  k = 80: 19 us and, with the Newton-Schulz
-// shortcut, 6; the shared-memory kernel above 32 and 9.  k = 160: 68 and 16, 100 and 18.
+// bounds it is that chain: two barriers, four reciprocals.  Under ncu, all pivots
+// kept: k = 80 20 us and, with the Newton-Schulz shortcut, 7; the shared-memory kernel
+// above, which the fixed order keeps, 67 and 11 (36 and 7 in an environment at
+// (4, 64), where most pivots drop).  k = 160: 70 and 15, 183 and 27.
 template <typename T>
 struct alignas(4 * sizeof(T)) Quad {
     T v[4];

@@ -27,8 +27,8 @@
 // at every instruction).  Up to D = 5 the order is the fixed one (layered.cuh).  BF16 runs one kind::f16 pass (K = 16 per MMA).
 // What bounds it: the tensor pipe's narrow MMAs at D >= 6 (73 % of the TF32 rate
 // over the padded shapes at D = 8), the chunk's chain of hand-offs below.  Time of a
-// launch, 3xTF32, p = 16: (4, 64) 20 us, (5, 100) 140, (6, 144) 454 (137 TFLOP/s),
-// (8, 144) 1494 (233); with Y as a shared-memory operand, one worker set and MMAs
+// launch, 3xTF32, p = 16: (4, 64) 21.5 us, (5, 100) 134, (6, 144) 443 (140 TFLOP/s),
+// (8, 144) 1481 (235); with Y as a shared-memory operand, one worker set and MMAs
 // issued from a one-lane branch: 25.5, 167, 722, 2113.  Y in tensor memory frees
 // 64 KB for two stages of both image rings, whose reload was on the chain.
 // Every wait is bounded: on time-out the kernel raises a flag, the roles drain,

